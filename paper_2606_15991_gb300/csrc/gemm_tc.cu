@@ -227,74 +227,78 @@ __global__ void __launch_bounds__(kThreads, 1)
   bool sp_have = false;
 
   if (warp == 0) {
-    // ---------------- TMA producer (one thread; the rest of the warp waits)
-    if (lane == 0) {
-      const uint64_t pol_a = policy_evict_last();
-      const uint64_t pol_b = policy_evict_last();
-      uint32_t fills[kMaxStages] = {};
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int32_t s = prog; s < TS && ok; s += step) {
-        const Unit u = unit_of(s, p);
-        int32_t tm, tn;
-        raster((uint32_t)u.tile, (uint32_t)p.gm, (uint32_t)p.gn, (uint32_t)p.group_m, &tm, &tn);
-        // a narrow tile loads only its own columns of B, through the map whose
-        // box has that many rows
-        const int ub_rows = kPair ? u.width / 2 : u.width;
-        const CUtensorMap* mb = u.cut ? &map_b_cut : &map_b;
-        const uint32_t utx = a_stage + (uint32_t)ub_rows * 128 * (uint32_t)p.kc;
-        // swap-AB: the MMA's A operand is B^T (rows = C columns, tile column
-        // tn) and its B operand is A (rows = C rows, tile row tm)
-        const int32_t arow = (kSwap ? tn : tm) * tile_m + (int32_t)rank * p.rows;
-        const int32_t brow = (kSwap ? tm : tn) * p.bn + u.col + (int32_t)rank * ub_rows;
-        for (int32_t kb = kb0; kb < kb1; kb += p.kc) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
-          if (p.inject && s == prog && kb == kb0) {
-            // test hook: this stage is never armed or filled, so its
-            // consumer's bounded wait runs out
-            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
-            continue;
-          }
-          // 2-D boxes take K at element kb * kblk; 3-D boxes take K block kb
-          // (blocks past the last one are zero-filled and never multiplied)
-          const int32_t kx = p.kc > 1 ? 0 : kb * p.kblk;
+    // ---------------- TMA producer (the whole warp walks the schedule, one
+    // elected lane issues; see elect_one)
+    const uint64_t pol_a = policy_evict_last();
+    const uint64_t pol_b = policy_evict_last();
+    uint32_t filled = 0;  // ring slots passed so far (the injected first one included)
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int32_t s = prog; s < TS && ok; s += step) {
+      const Unit u = unit_of(s, p);
+      int32_t tm, tn;
+      raster((uint32_t)u.tile, (uint32_t)p.gm, (uint32_t)p.gn, (uint32_t)p.group_m, &tm, &tn);
+      // a narrow tile loads only its own columns of B, through the map whose
+      // box has that many rows
+      const int ub_rows = kPair ? u.width / 2 : u.width;
+      const CUtensorMap* mb = u.cut ? &map_b_cut : &map_b;
+      const uint32_t utx = a_stage + (uint32_t)ub_rows * 128 * (uint32_t)p.kc;
+      // swap-AB: the MMA's A operand is B^T (rows = C columns, tile column
+      // tn) and its B operand is A (rows = C rows, tile row tm)
+      const int32_t arow = (kSwap ? tn : tm) * tile_m + (int32_t)rank * p.rows;
+      const int32_t brow = (kSwap ? tm : tn) * p.bn + u.col + (int32_t)rank * ub_rows;
+      for (int32_t kb = kb0; kb < kb1; kb += p.kc) {
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
+        // 2-D boxes take K at element kb * kblk; 3-D boxes take K block kb
+        // (blocks past the last one are zero-filled and never multiplied)
+        const int32_t kx = p.kc > 1 ? 0 : kb * p.kblk;
+        const uint32_t da = a0 + a_stage * stage, db = b0 + b_stage * stage;
+        // test hook (inject): the first stage is never armed or filled, so its
+        // consumer's bounded wait runs out
+        if (!(p.inject && filled == 0) && elect_one()) {
           if constexpr (kPair) {
             // both CTAs' copies complete on the even CTA's full barrier
             const uint32_t fb = mapa(full_bar(stage), 0);
             if (leader) mbar_arrive_expect_tx(full_bar(stage), 2 * utx);
             if (p.kc > 1) {
-              tma_load_3d_pair(a0 + a_stage * stage, &map_a, 0, arow, kb, fb, pol_a);
-              tma_load_3d_pair(b0 + b_stage * stage, mb, 0, brow, kb, fb, pol_b);
+              tma_load_3d_pair(da, &map_a, 0, arow, kb, fb, pol_a);
+              tma_load_3d_pair(db, mb, 0, brow, kb, fb, pol_b);
             } else {
-              tma_load_2d_pair(a0 + a_stage * stage, &map_a, kx, arow, fb, pol_a);
-              tma_load_2d_pair(b0 + b_stage * stage, mb, kx, brow, fb, pol_b);
+              tma_load_2d_pair(da, &map_a, kx, arow, fb, pol_a);
+              tma_load_2d_pair(db, mb, kx, brow, fb, pol_b);
             }
           } else {
             mbar_arrive_expect_tx(full_bar(stage), utx);
             if (p.kc > 1) {
-              tma_load_3d(a0 + a_stage * stage, &map_a, 0, arow, kb, full_bar(stage), pol_a);
-              tma_load_3d(b0 + b_stage * stage, mb, 0, brow, kb, full_bar(stage), pol_b);
+              tma_load_3d(da, &map_a, 0, arow, kb, full_bar(stage), pol_a);
+              tma_load_3d(db, mb, 0, brow, kb, full_bar(stage), pol_b);
             } else {
-              tma_load_2d(a0 + a_stage * stage, &map_a, kx, arow, full_bar(stage), pol_a);
-              tma_load_2d(b0 + b_stage * stage, mb, kx, brow, full_bar(stage), pol_b);
+              tma_load_2d(da, &map_a, kx, arow, full_bar(stage), pol_a);
+              tma_load_2d(db, mb, kx, brow, full_bar(stage), pol_b);
             }
           }
-          fills[stage]++;
-          if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        ++filled;
+        if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       }
-      if (!ok && (!kPair || leader)) {
-        // drain: wait (bounded) until every copy signalled on our full
-        // barriers landed (the odd CTA's copies signal the even CTA's)
-        for (int s2 = 0; s2 < p.stages; ++s2)
-          if (fills[s2]) mbar_wait(full_bar(s2), (fills[s2] - 1u) & 1u, nullptr, nullptr, 200000000ull);
+    }
+    if (!ok && (!kPair || leader)) {
+      // drain: wait (bounded) until every copy signalled on our full
+      // barriers landed (the odd CTA's copies signal the even CTA's)
+      for (uint32_t s2 = 0; s2 < (uint32_t)p.stages && s2 < filled; ++s2) {
+        uint32_t fills = (filled - s2 - 1u) / (uint32_t)p.stages + 1u;
+        if (p.inject && s2 == 0) --fills;  // never armed the first time
+        if (fills) mbar_wait(full_bar((int)s2), (fills - 1u) & 1u, nullptr, nullptr, 200000000ull);
       }
     }
     __syncwarp();
   } else if (warp == 1) {
-    // ---------------- MMA issuer (one thread of the even CTA)
-    if (lane == 0 && leader) {
+    // ---------------- MMA issuer (the even CTA's warp 1; one elected lane
+    // issues). With one diverged lane running this loop an MMA took 60 cycles
+    // to issue however small its N; @@MMA@@
+    if (leader) {
       const uint32_t idesc_full = idesc_f32acc((uint32_t)tile_m, (uint32_t)p.bn, kF8);
       const uint32_t idesc_cut = idesc_f32acc((uint32_t)tile_m, (uint32_t)p.bn_cut, kF8);
       int stage = 0;
@@ -307,37 +311,50 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t b_blk = (uint32_t)(kPair ? u.width / 2 : u.width) * 128;  // B box rows * 128
         const int acc = t & 1;
         const uint32_t use = (uint32_t)((t >> 1) & 1);
-        if (!mbar_wait(tempty_bar(acc), use ^ 1u, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
+        if (!mbar_wait_warp(tempty_bar(acc), use ^ 1u, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d = tmem_base + (uint32_t)(acc * p.bn);
         for (int32_t kb = kb0; kb < kb1; kb += p.kc) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
+          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
           tc_fence_after();
+          const uint64_t ad0 = desc_kmajor_sw128(a0 + a_stage * stage);
+          const uint64_t bd0 = desc_kmajor_sw128(b0 + b_stage * stage);
           // the stage's K blocks in K order, the same MMAs as one block per
           // stage (blocks past the tile's last are not multiplied)
           for (int32_t j = 0; j < p.kc && kb + j < kb1; ++j) {
-            const uint64_t ad = desc_kmajor_sw128(a0 + a_stage * stage + a_blk * (uint32_t)j);
-            const uint64_t bd = desc_kmajor_sw128(b0 + b_stage * stage + b_blk * (uint32_t)j);
-            // 128-byte K slice = 4 MMAs of K = 16 (bf16) or K = 32 (fp8), 32
-            // bytes apart inside the swizzle atom (start address advances by 32 >> 4).
+            const uint64_t ad = ad0 + (uint64_t)((a_blk >> 4) * (uint32_t)j);
+            const uint64_t bd = bd0 + (uint64_t)((b_blk >> 4) * (uint32_t)j);
+            const uint32_t accum0 = kb + j > kb0 ? 1u : 0u;
+            if (elect_one()) {
+              // 128-byte K slice = 4 MMAs of K = 16 (bf16) or K = 32 (fp8), 32
+              // bytes apart inside the swizzle atom (start address advances by 32 >> 4).
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const uint32_t accum = (kb + j > kb0 || k > 0) ? 1u : 0u;
-              if constexpr (kPair) mma_pair<kF8>(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, accum);
-              else mma<kF8>(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, accum);
+              for (int k = 0; k < 4; ++k) {
+                const uint32_t accum = k > 0 ? 1u : accum0;
+                if constexpr (kPair) mma_pair<kF8>(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, accum);
+                else mma<kF8>(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, accum);
+              }
+            }
+            __syncwarp();
+          }
+          if (elect_one()) {
+            if constexpr (kPair) mma_commit_pair(empty_bar(stage), 0x3);
+            else mma_commit(empty_bar(stage));
+            if (kb + p.kc >= kb1) {
+              if constexpr (kPair) mma_commit_pair(tfull_bar(acc), 0x3);
+              else mma_commit(tfull_bar(acc));
             }
           }
-          if constexpr (kPair) mma_commit_pair(empty_bar(stage), 0x3);
-          else mma_commit(empty_bar(stage));
+          __syncwarp();
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        if constexpr (kPair) mma_commit_pair(tfull_bar(acc), 0x3);
-        else mma_commit(tfull_bar(acc));
       }
       if (!ok) {
-        if constexpr (kPair) mma_commit_pair(drain_bar, 0x1);
-        else mma_commit(drain_bar);
+        if (elect_one()) {
+          if constexpr (kPair) mma_commit_pair(drain_bar, 0x1);
+          else mma_commit(drain_bar);
+        }
+        __syncwarp();
         mbar_wait(drain_bar, 0, nullptr, nullptr, 200000000ull);
       }
     }

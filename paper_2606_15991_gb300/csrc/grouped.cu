@@ -197,25 +197,30 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
   auto ring_wait = [&](uint32_t bar, uint32_t parity) {
     return kPair ? mbar_wait_cluster(bar, parity, abort_flag, p.err) : mbar_wait(bar, parity, abort_flag, p.err);
   };
+  auto ring_wait_warp = [&](uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, ring_wait(bar, parity)) != 0;
+  };
   auto ring_release = [&](int r) {
     if constexpr (kPair) mbar_arrive_cluster(mapa(rempty_bar(r), 0));
     else mbar_arrive(rempty_bar(r));
   };
 
   if (warp == 0) {
-    if (lane == 0) {
-      const uint64_t pol_stream = policy_evict_first();
-      const uint64_t pol_keep = policy_evict_last();
-      uint32_t fills[8] = {};
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int64_t j = 0; ok; ++j) {
-        const int r = (int)(j % kRing);
-        const uint32_t par = (uint32_t)((j / kRing) & 1);
-        int64_t g;
-        if (leader) {
-          if (!ring_wait(rempty_bar(r), par ^ 1u)) { ok = false; break; }
+    // ---------------- dequeues slots and streams their tiles (the whole warp
+    // walks the loop, one elected lane issues: elect_one)
+    const uint64_t pol_stream = policy_evict_first();
+    const uint64_t pol_keep = policy_evict_last();
+    uint32_t filled = 0;  // ring stages filled so far
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int64_t j = 0; ok; ++j) {
+      const int r = (int)(j % kRing);
+      const uint32_t par = (uint32_t)((j / kRing) & 1);
+      int64_t g = 0;
+      if (leader) {
+        if (!ring_wait_warp(rempty_bar(r), par ^ 1u)) { ok = false; break; }
+        if (lane == 0) {
           const int64_t d = (int64_t)atomicAdd(p.queue, 1u);
           g = d < p.total ? d : -1;
           ring[r] = g;
@@ -226,101 +231,121 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
           } else {
             mbar_arrive(rfull_bar(r));
           }
-        } else {
-          if (!ring_wait(rfull_bar(r), par)) { ok = false; break; }
-          g = ring[r];
-          ring_release(r);
         }
-        if (g < 0) break;
-        const GroupedProblem* pr;
-        int64_t tr, tc;
-        decode(g, &pr, &tr, &tc);
-        const int32_t xrow = (int32_t)(tr * pr->tile_rows + rank * 128);
-        const int32_t yrow = (int32_t)(tc * pr->bn + rank * pr->box_y);
-        const int32_t pkc = pr->kc;
-        const uint32_t tx = (kStageX + (uint32_t)pr->box_y * 128u) * (uint32_t)pkc;
-        const int64_t nk = (pr->K + 63) / 64;
-        for (int64_t kb = 0; kb < nk; kb += pkc) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.err)) { ok = false; break; }
-          // 2-D maps take K at element kb * 64; 3-D maps take K block kb (a
-          // block past the last is zero-filled and never multiplied)
-          const int32_t kx = pkc > 1 ? 0 : (int32_t)(kb * 64);
-          // streamed swap: x = B_i slab (read once), y = A_i (reused by every tile)
-          const uint64_t px = pr->stream_x ? pol_stream : pol_keep;
+        g = __shfl_sync(0xffffffffu, g, 0);
+      } else {
+        if (!ring_wait_warp(rfull_bar(r), par)) { ok = false; break; }
+        g = __shfl_sync(0xffffffffu, ring[r], 0);
+        if (lane == 0) ring_release(r);
+      }
+      if (g < 0) break;
+      const GroupedProblem* pr;
+      int64_t tr, tc;
+      decode(g, &pr, &tr, &tc);
+      const int32_t xrow = (int32_t)(tr * pr->tile_rows + rank * 128);
+      const int32_t yrow = (int32_t)(tc * pr->bn + rank * pr->box_y);
+      const int32_t pkc = pr->kc;
+      const uint32_t tx = (kStageX + (uint32_t)pr->box_y * 128u) * (uint32_t)pkc;
+      const int32_t nk = (int32_t)((pr->K + 63) / 64);
+      // streamed swap: x = B_i slab (read once), y = A_i (reused by every tile)
+      const uint64_t px = pr->stream_x ? pol_stream : pol_keep;
+      const CUtensorMap* mx = &pr->map_x;
+      const CUtensorMap* my = &pr->map_y;
+      for (int32_t kb = 0; kb < nk; kb += pkc) {
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.err)) { ok = false; break; }
+        // 2-D maps take K at element kb * 64; 3-D maps take K block kb (a
+        // block past the last is zero-filled and never multiplied)
+        const int32_t kx = pkc > 1 ? 0 : kb * 64;
+        const uint32_t dx = stage_at(stage), dy = stage_at(stage) + kStageX * (uint32_t)pkc;
+        if (elect_one()) {
           if constexpr (kPair) {
             const uint32_t fb = mapa(full_bar(stage), 0);  // both halves complete on the even CTA's barrier
             if (leader) mbar_arrive_expect_tx(full_bar(stage), 2 * tx);
             if (pkc > 1) {
-              tma_load_3d_pair(stage_at(stage), &pr->map_x, 0, xrow, (int32_t)kb, fb, px);
-              tma_load_3d_pair(stage_at(stage) + kStageX * (uint32_t)pkc, &pr->map_y, 0, yrow, (int32_t)kb, fb,
-                               pol_keep);
+              tma_load_3d_pair(dx, mx, 0, xrow, kb, fb, px);
+              tma_load_3d_pair(dy, my, 0, yrow, kb, fb, pol_keep);
             } else {
-              tma_load_2d_pair(stage_at(stage), &pr->map_x, kx, xrow, fb, px);
-              tma_load_2d_pair(stage_at(stage) + kStageX, &pr->map_y, kx, yrow, fb, pol_keep);
+              tma_load_2d_pair(dx, mx, kx, xrow, fb, px);
+              tma_load_2d_pair(dy, my, kx, yrow, fb, pol_keep);
             }
           } else {
             mbar_arrive_expect_tx(full_bar(stage), tx);
-            tma_load_2d(stage_at(stage), &pr->map_x, kx, xrow, full_bar(stage), px);
-            tma_load_2d(stage_at(stage) + kStageX, &pr->map_y, kx, yrow, full_bar(stage), pol_keep);
+            tma_load_2d(dx, mx, kx, xrow, full_bar(stage), px);
+            tma_load_2d(dy, my, kx, yrow, full_bar(stage), pol_keep);
           }
-          fills[stage]++;
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        ++filled;
+        if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
-      if (!ok && leader) {
-        for (int s2 = 0; s2 < kStages; ++s2)
-          if (fills[s2]) mbar_wait(full_bar(s2), (fills[s2] - 1u) & 1u, nullptr, nullptr, 200000000ull);
-      }
+    }
+    if (!ok && leader) {
+      for (uint32_t s2 = 0; s2 < (uint32_t)kStages && s2 < filled; ++s2)
+        mbar_wait(full_bar((int)s2), ((filled - s2 - 1u) / kStages) & 1u, nullptr, nullptr, 200000000ull);
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && leader) {
+    // ---------------- MMA issuer (the even CTA's warp 1, one elected lane)
+    if (leader) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
       for (int64_t j = 0; ok; ++j) {
         const int r = (int)(j % kRing);
-        if (!mbar_wait(rfull_bar(r), (uint32_t)((j / kRing) & 1), abort_flag, p.err)) { ok = false; break; }
-        const int64_t g = ring[r];
-        ring_release(r);
+        if (!mbar_wait_warp(rfull_bar(r), (uint32_t)((j / kRing) & 1), abort_flag, p.err)) { ok = false; break; }
+        const int64_t g = __shfl_sync(0xffffffffu, ring[r], 0);
+        if (lane == 0) ring_release(r);
         if (g < 0) break;
         const GroupedProblem* pr;
         int64_t tr, tc;
         decode(g, &pr, &tr, &tc);
         const int acc = (int)(j & 1);
         const uint32_t use = (uint32_t)((j >> 1) & 1);
-        if (!mbar_wait(tempty_bar(acc), use ^ 1u, abort_flag, p.err)) { ok = false; break; }
+        if (!mbar_wait_warp(tempty_bar(acc), use ^ 1u, abort_flag, p.err)) { ok = false; break; }
         tc_fence_after();
         const uint32_t idesc = idesc_f32acc(kPair ? 256 : 128, (uint32_t)pr->bn, false);
         const uint32_t d = tmem_base + (uint32_t)(acc * 256);
-        const int64_t nk = (pr->K + 63) / 64;
+        const int32_t nk = (int32_t)((pr->K + 63) / 64);
         const int32_t pkc = pr->kc;
         const uint32_t y_blk = (uint32_t)pr->box_y * 128u;  // one K block of the B operand
-        for (int64_t kb = 0; kb < nk; kb += pkc) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag, p.err)) { ok = false; break; }
+        for (int32_t kb = 0; kb < nk; kb += pkc) {
+          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.err)) { ok = false; break; }
           tc_fence_after();
+          const uint64_t ad0 = desc_kmajor_sw128(stage_at(stage));
+          const uint64_t bd0 = desc_kmajor_sw128(stage_at(stage) + kStageX * (uint32_t)pkc);
           // the stage's K blocks in K order (blocks past the last are not multiplied)
           for (int32_t jb = 0; jb < pkc && kb + jb < nk; ++jb) {
-            const uint64_t ad = desc_kmajor_sw128(stage_at(stage) + kStageX * (uint32_t)jb);
-            const uint64_t bd = desc_kmajor_sw128(stage_at(stage) + kStageX * (uint32_t)pkc + y_blk * (uint32_t)jb);
+            const uint64_t ad = ad0 + (uint64_t)((kStageX >> 4) * (uint32_t)jb);
+            const uint64_t bd = bd0 + (uint64_t)((y_blk >> 4) * (uint32_t)jb);
+            const uint32_t accum0 = kb + jb > 0 ? 1u : 0u;
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const uint32_t accum = (kb + jb > 0 || k > 0) ? 1u : 0u;
-              if constexpr (kPair) mma_pair<false>(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, accum);
-              else mma<false>(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, accum);
+              for (int k = 0; k < 4; ++k) {
+                const uint32_t accum = k > 0 ? 1u : accum0;
+                if constexpr (kPair) mma_pair<false>(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, accum);
+                else mma<false>(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, accum);
+              }
+            }
+            __syncwarp();
+          }
+          if (elect_one()) {
+            if constexpr (kPair) mma_commit_pair(empty_bar(stage), 0x3);
+            else mma_commit(empty_bar(stage));
+            if (kb + pkc >= nk) {
+              if constexpr (kPair) mma_commit_pair(tfull_bar(acc), 0x3);
+              else mma_commit(tfull_bar(acc));
             }
           }
-          if constexpr (kPair) mma_commit_pair(empty_bar(stage), 0x3);
-          else mma_commit(empty_bar(stage));
+          __syncwarp();
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        if constexpr (kPair) mma_commit_pair(tfull_bar(acc), 0x3);
-        else mma_commit(tfull_bar(acc));
       }
       if (!ok) {
-        if constexpr (kPair) mma_commit_pair(drain_bar, 0x1);
-        else mma_commit(drain_bar);
+        if (elect_one()) {
+          if constexpr (kPair) mma_commit_pair(drain_bar, 0x1);
+          else mma_commit(drain_bar);
+        }
+        __syncwarp();
         mbar_wait(drain_bar, 0, nullptr, nullptr, 200000000ull);
       }
     }

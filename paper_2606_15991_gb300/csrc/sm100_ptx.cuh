@@ -79,6 +79,28 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// One lane of a converged warp (the same lane on every call). The roles that
+// issue TMA copies and MMAs run their loops with the whole warp and put only
+// the issuing instructions behind this predicate: loop state, addresses and
+// descriptors then stay warp-uniform, the form those instructions take their
+// operands in, where a loop run by a single diverged lane has to move every
+// operand over for every instruction.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
+
+// mbar_wait by every lane of a converged warp; one outcome for the warp.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort, int* err,
+                                               uint64_t limit_ns = 2000000000ull) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, err, limit_ns)) != 0;
+}
+
 // -------------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
