@@ -1,8 +1,9 @@
 // Element-wise map kernels: one tile program per output tile (plain
 // partition, §3.4) or persistent programs walking a bounded sequence of tiles
 // (mapped partition, §3.6). The rank-1 path moves 16 bytes per load/store
-// (4 fp32 or 8 bf16) with streaming cache hints; other shapes use a scalar
-// path over the tile's elements. Each program stores only inside its tile.
+// (4 fp32 or 8 bf16) with streaming cache hints; other tilings move the rows
+// of a tile as runs of 16-byte slots; tensors whose alignments differ take a
+// scalar path. Each program stores only inside its tile.
 #include <cuda_bf16.h>
 
 #include "tile_claim.cuh"
@@ -28,6 +29,7 @@ struct MapArgs {
   int64_t shape[3];  // general path, padded to rank 3 (leading 1s)
   int64_t tshape[3];
   int64_t grid[3];
+  int32_t mis;           // elements from each base pointer down to a 16-byte boundary (segment path)
   uint32_t* claims;      // checked launch: tile-claim bitmap (null = release)
   unsigned* claim_done;  // checked launch: finished-CTA counter
   int* err;              // context error word
@@ -236,8 +238,122 @@ __global__ void __launch_bounds__(kThreads) map_vec_kernel(const __grid_constant
   finish_map_claims<CHECKED>(a);
 }
 
+// n / d and n % d of non-negative values, in 32 bits where both fit (a 64-bit
+// division costs hundreds of cycles).
+__device__ __forceinline__ void divmod(int64_t n, int64_t d, int64_t* q, int64_t* r) {
+  if (((n | d) >> 32) == 0) {
+    const uint32_t q32 = (uint32_t)n / (uint32_t)d;
+    *q = q32;
+    *r = (uint32_t)n - q32 * (uint32_t)d;
+  } else {
+    *q = n / d;
+    *r = n - *q * d;
+  }
+}
+
+// Tiles made of row segments: any rank-1..3 partition whose three tensors are
+// equally aligned (`mis` = elements from each base pointer down to a 16-byte
+// boundary). A tile row is one contiguous run of elements, the same run in
+// every tensor, so it is covered by 16-byte slots on the address grid: a slot
+// inside the run moves as one vector, a slot that the run only touches (at
+// its two ends) element by element, so a program still stores only inside its
+// tile. The slots of all rows of the tile are dealt to the threads in one
+// flat sequence, so rows shorter than a warp leave no lane idle; a thread's
+// (row, slot) advances by a fixed step, without a division per access.
+// Bound by HBM: y = gelu_tanh(x) * w over 4001 x 9728 bf16 in 128 x 256 tiles
+// (234 MB) takes a synchronous call of 67 us, of which the kernel is about 42
+// (5.5 TB/s); one element per access with two 64-bit divisions each took 299
+// us (kernel 267). Two (bf16) or four (f32) slots in flight per thread, as in
+// map_vec_kernel; that kernel stays for rank-1 tiles of whole vectors, where
+// it needs no run arithmetic (32 registers against 55-100).
+template <int OP, typename T, bool COUNT>
+__global__ void __launch_bounds__(kThreads) map_segment_kernel(const __grid_constant__ MapArgs a) {
+  using V = typename Vec<T>::V;
+  constexpr int W = Vec<T>::N;
+  constexpr int U = 16 / W > 1 ? 16 / W : 1;  // slots in flight per thread: 4 (f32), 2 (bf16)
+  __shared__ int64_t slot;
+  pdl_enter();
+  T* out = static_cast<T*>(a.out);
+  const T* x = static_cast<const T*>(a.x);
+  const T* y = static_cast<const T*>(a.y);
+  Schedule s;
+  for (int64_t t = s.first(a, &slot); t >= 0; t = s.next(a, &slot)) {
+    if (!claim_map_tile(a, t)) continue;
+    int64_t t0, t1, t2, q;
+    divmod(t, a.grid[2], &q, &t2);
+    divmod(q, a.grid[1], &t0, &t1);
+    // the tile clipped to the tensor: e0 x e1 rows of e2 elements
+    const int64_t b0 = t0 * a.tshape[0], b1 = t1 * a.tshape[1], b2 = t2 * a.tshape[2];
+    const int32_t e0 = (int32_t)min(a.tshape[0], a.shape[0] - b0), e1 = (int32_t)min(a.tshape[1], a.shape[1] - b1);
+    const int32_t e2 = (int32_t)min(a.tshape[2], a.shape[2] - b2);
+    const int64_t origin = (b0 * a.shape[1] + b1) * a.shape[2] + b2;
+    // slots a row may touch; every row starts at the same place of a slot
+    // when the row pitch is whole slots
+    const int32_t ph0 = (int32_t)((uint64_t)(origin + a.mis) % W);
+    const uint32_t per = (uint32_t)(a.shape[2] % W == 0 ? ph0 + e2 + W - 1 : e2 + 2 * W - 2) / W;
+    const uint32_t rows = (uint32_t)e0 * (uint32_t)e1;
+    const uint32_t dr = kThreads / per, dc = kThreads % per;
+    uint32_t r = threadIdx.x / per, c = threadIdx.x % per;
+    while (r < rows) {
+      int64_t at[U];   // the slot's first element (may lie before the run's)
+      int32_t i0[U], i1[U];  // its elements [i0, i1) are the run's; none when i0 >= i1
+      V xr[U], yr[U], cr[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        i0[u] = i1[u] = 0;
+        if (r < rows) {
+          const uint32_t r0 = e0 > 1 ? r / (uint32_t)e1 : 0u;
+          const uint32_t r1 = r - r0 * (uint32_t)e1;
+          const int64_t g = origin + ((int64_t)r0 * a.shape[1] + r1) * a.shape[2];  // the run's first element
+          const int32_t lo = (int32_t)c * W - (int32_t)((uint64_t)(g + a.mis) % W);
+          at[u] = g + lo;
+          i0[u] = max(-lo, 0);
+          i1[u] = min(W, e2 - lo);
+          if (i0[u] == 0 && i1[u] == W) {
+            xr[u] = __ldcs(reinterpret_cast<const V*>(x + at[u]));
+            yr[u] = __ldcs(reinterpret_cast<const V*>(y + at[u]));
+            if constexpr (OP == kMapAddAccum) cr[u] = *reinterpret_cast<const V*>(out + at[u]);
+          }
+        }
+        r += dr;
+        c += dc;
+        if (c >= per) {
+          c -= per;
+          ++r;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (i0[u] == 0 && i1[u] == W) {
+          float fx[W], fy[W], fc[W], fo[W];
+          unpack<T>(xr[u], fx);
+          unpack<T>(yr[u], fy);
+          if constexpr (OP == kMapAddAccum) unpack<T>(cr[u], fc);
+#pragma unroll
+          for (int i = 0; i < W; ++i) fo[i] = apply<OP>(fx[i], fy[i], OP == kMapAddAccum ? fc[i] : 0.f, a.alpha);
+          __stcs(reinterpret_cast<V*>(out + at[u]), pack<T>(fo));
+          if constexpr (COUNT) {
+#pragma unroll
+            for (int i = 0; i < W; ++i) count_write<COUNT>(a, at[u] + i);
+          }
+        } else {
+          for (int32_t i = i0[u]; i < i1[u]; ++i) {
+            const int64_t g = at[u] + i;
+            const float cv = OP == kMapAddAccum ? to_f<T>(out[g]) : 0.f;
+            out[g] = from_f<T>(apply<OP>(to_f<T>(x[g]), to_f<T>(y[g]), cv, a.alpha));
+            count_write<COUNT>(a, g);
+          }
+        }
+      }
+    }
+  }
+  finish_map_claims(a);
+}
+
 // General path: any rank-1..3 partition of a contiguous output, scalar
-// accesses, elements of the tile outside the tensor are skipped.
+// accesses, elements of the tile outside the tensor are skipped. Taken only
+// when the three tensors' base pointers differ in their offset from a 16-byte
+// boundary, so that no 16-byte access fits all of them.
 template <int OP, typename T, bool COUNT>
 __global__ void __launch_bounds__(kThreads) map_generic_kernel(const __grid_constant__ MapArgs a) {
   __shared__ int64_t slot;
@@ -282,9 +398,38 @@ cudaError_t launch_pdl(K kernel, const MapArgs& a, int64_t grid, cudaStream_t st
   return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
+// How a map's tiles are accessed, fastest first.
+enum Path : int {
+  kVector,   // rank 1, tiles of whole vectors from a 16-byte boundary on
+  kSegment,  // row segments on the 16-byte grid
+  kScalar,   // one element at a time
+};
+
+// The path for `a`. The segment path counts a tile's rows and slots in 32
+// bits, so tiles of 2^30 elements or more stay on the scalar path.
+template <typename T>
+Path map_path(MapArgs* a, bool rank1) {
+  constexpr int W = Vec<T>::N;
+  auto off = [](const void* p) { return reinterpret_cast<uintptr_t>(p) & 15u; };
+  const uintptr_t m = off(a->out);
+  if (off(a->x) != m || off(a->y) != m || m % sizeof(T)) return kScalar;
+  if (rank1 && m == 0 && a->tile % W == 0) return kVector;
+  int64_t elems = 1;
+  for (int i = 0; i < 3; ++i) {
+    const int64_t e = a->tshape[i] < a->shape[i] ? a->tshape[i] : a->shape[i];
+    if (e >= (int64_t(1) << 30) / elems) return kScalar;
+    elems *= e;
+  }
+  a->mis = (int32_t)(m / sizeof(T));
+  return kSegment;
+}
+
 template <int OP, typename T>
-cudaError_t launch_typed(const MapArgs& a, bool vec, bool count, int64_t grid, cudaStream_t st) {
+cudaError_t launch_typed(const MapArgs& a, Path path, bool count, int64_t grid, cudaStream_t st) {
   const bool checked = a.claims != nullptr;
+  const bool vec = path == kVector;
+  if (path == kSegment) return count ? launch_pdl(map_segment_kernel<OP, T, true>, a, grid, st)
+                                     : launch_pdl(map_segment_kernel<OP, T, false>, a, grid, st);
   if (vec && checked) return count ? launch_pdl(map_vec_kernel<OP, T, true, true>, a, grid, st)
                                    : launch_pdl(map_vec_kernel<OP, T, false, true>, a, grid, st);
   if (vec) return count ? launch_pdl(map_vec_kernel<OP, T, true, false>, a, grid, st)
@@ -294,12 +439,13 @@ cudaError_t launch_typed(const MapArgs& a, bool vec, bool count, int64_t grid, c
 }
 
 template <typename T>
-cudaError_t launch_op(int op, const MapArgs& a, bool vec, bool count, int64_t grid, cudaStream_t st) {
+cudaError_t launch_op(int op, MapArgs a, bool rank1, bool count, int64_t grid, cudaStream_t st) {
+  const Path path = map_path<T>(&a, rank1);
   switch (op) {
-    case kMapAxpy: return launch_typed<kMapAxpy, T>(a, vec, count, grid, st);
-    case kMapGeluMul: return launch_typed<kMapGeluMul, T>(a, vec, count, grid, st);
-    case kMapScale: return launch_typed<kMapScale, T>(a, vec, count, grid, st);
-    default: return launch_typed<kMapAddAccum, T>(a, vec, count, grid, st);
+    case kMapAxpy: return launch_typed<kMapAxpy, T>(a, path, count, grid, st);
+    case kMapGeluMul: return launch_typed<kMapGeluMul, T>(a, path, count, grid, st);
+    case kMapScale: return launch_typed<kMapScale, T>(a, path, count, grid, st);
+    default: return launch_typed<kMapAddAccum, T>(a, path, count, grid, st);
   }
 }
 
@@ -333,14 +479,11 @@ tp_status launch_map(tp_ctx* ctx, tp_partition* out, int op, float alpha, const 
     a.grid[i] = i < pad ? 1 : out->grid[i - pad];
   }
   if (a.n == 0 || a.ntiles == 0) return TP_OK;
-  const int w = out->t.dtype == TP_F32 ? 4 : 8;
-  auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
-  const bool vec = out->rank == 1 && (a.tile % w) == 0 && aligned(a.out) && aligned(a.x) && aligned(a.y);
   const int64_t grid = out->kind == TP_MAP_IDENTITY ? out->num_tiles : out->num_programs;
   if (grid > 0x7fffffff) return fail(TP_ERR_UNSUPPORTED, "more than 2^31-1 tile programs");
   const bool count = a.counts != nullptr;
-  cudaError_t e = out->t.dtype == TP_F32 ? launch_op<float>(op, a, vec, count, grid, stream)
-                                         : launch_op<__nv_bfloat16>(op, a, vec, count, grid, stream);
+  cudaError_t e = out->t.dtype == TP_F32 ? launch_op<float>(op, a, out->rank == 1, count, grid, stream)
+                                         : launch_op<__nv_bfloat16>(op, a, out->rank == 1, count, grid, stream);
   if (e != cudaSuccess) return cuda_fail(e, "map kernel launch");
   return TP_OK;
 }
@@ -381,8 +524,10 @@ tp_status noalloc_queue_address(void** out) {
   if (dev < 0 || dev >= kNoallocMaxDevices) return fail(TP_ERR_UNSUPPORTED, "device index above 63");
   std::lock_guard<std::mutex> lk(g_noalloc_mu);
   if (!g_noalloc_queue_addr[dev]) {
-    const void* kernels[4] = {reinterpret_cast<const void*>(map_vec_kernel<kMapAxpy, float, false, false>),
+    const void* kernels[6] = {reinterpret_cast<const void*>(map_vec_kernel<kMapAxpy, float, false, false>),
                               reinterpret_cast<const void*>(map_vec_kernel<kMapAxpy, __nv_bfloat16, false, false>),
+                              reinterpret_cast<const void*>(map_segment_kernel<kMapAxpy, float, false>),
+                              reinterpret_cast<const void*>(map_segment_kernel<kMapAxpy, __nv_bfloat16, false>),
                               reinterpret_cast<const void*>(map_generic_kernel<kMapAxpy, float, false>),
                               reinterpret_cast<const void*>(map_generic_kernel<kMapAxpy, __nv_bfloat16, false>)};
     for (const void* k : kernels) {
@@ -441,11 +586,8 @@ extern "C" tp_status tp_map_axpy_queue_noalloc(void* z, const void* x, const voi
     a.tshape[i] = i < 2 ? 1 : tile;
     a.grid[i] = i < 2 ? 1 : ntiles;
   }
-  const int w = dtype == TP_F32 ? 4 : 8;
-  auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
-  const bool vec = (tile % w) == 0 && aligned(z) && aligned(x) && aligned(y);
-  e = dtype == TP_F32 ? launch_op<float>(kMapAxpy, a, vec, false, num_programs, st)
-                      : launch_op<__nv_bfloat16>(kMapAxpy, a, vec, false, num_programs, st);
+  e = dtype == TP_F32 ? launch_op<float>(kMapAxpy, a, true, false, num_programs, st)
+                      : launch_op<__nv_bfloat16>(kMapAxpy, a, true, false, num_programs, st);
   if (e != cudaSuccess) return cuda_fail(e, "map kernel launch");
   return TP_OK;
 }

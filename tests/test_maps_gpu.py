@@ -350,3 +350,48 @@ def test_trace_log_lines():
     env.pop("TP_LOG")
     r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "[tp] " not in r.stderr
+
+
+@pytest.mark.parametrize("op", ["axpy", "gelu_mul", "scale", "add_accum"])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("shape,tile,kind,P,off", [
+    ((7, 64), (4, 32), "identity", 0, 0),        # whole slots
+    ((9, 257), (4, 100), "identity", 0, 0),      # rows starting at every place of a slot
+    ((3, 5, 31), (2, 2, 7), "strided", 4, 0),    # rank 3, runs shorter than a slot
+    ((130, 2049), (128, 2048), "queue", 3, 0),   # clipped tiles, runs longer than a block's round
+    ((10007,), (100,), "strided", 5, 0),         # rank 1, tiles not of whole vectors
+    ((4096 * 2 + 9,), (4096,), "identity", 0, 3),  # equally misaligned tensors
+    ((5, 40), (8, 64), "identity", 0, 1),        # one tile larger than the tensor, misaligned
+    ((1, 1), (1, 1), "identity", 0, 2),
+])
+def test_segment_tiles_equal_the_scalar_path(ctx, op, dt, shape, tile, kind, P, off):
+    """Row-segment tiles give the scalar path's bits (taken when the tensors'
+    alignments differ) and write each element once, nothing outside."""
+    n = int(np.prod(shape))
+    pad = 8 + off
+    kinds = {"identity": tp.MAP_IDENTITY, "strided": tp.MAP_STRIDED, "queue": tp.MAP_QUEUE}
+    xs, ys, cs = (t.reshape(-1) for t in _inputs(n, dt))
+    outs = []
+    for shift in (0, 1):   # shift 1: x is aligned differently from y and out
+        buf = [torch.full((n + 16 + pad,), 7.0, dtype=TORCH_DT[dt], device="cuda") for _ in range(3)]
+        views = []
+        for b, src, o in zip(buf, (xs, ys, cs), (off + shift, off, off)):
+            v = b[o:o + n]
+            v.copy_(src)
+            views.append(v.reshape(shape))
+        x, y, out = views
+        part = tp.tp_partition_create(ctx, out, tile)
+        if kind != "identity":
+            tp.tp_partition_map(part, kinds[kind], P)
+        counts = torch.zeros(n, dtype=torch.int32, device="cuda")
+        owner = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+        for ex in (None, tp.make_exec(write_counts=counts, write_owner=owner)):
+            out.reshape(-1).copy_(cs)
+            args = (ctx, part, ALPHA, x, y, ex) if op == "axpy" else (ctx, part, x, y, ex)
+            FN[op](*args)
+            outs.append(out.clone().reshape(-1))
+        assert opart.check_counts(counts.cpu().numpy())["ok"]
+        assert torch.all(buf[2][:off] == 7.0) and torch.all(buf[2][off + n:] == 7.0)
+        tp.tp_partition_destroy(part)
+    for o in outs[1:]:
+        assert torch.equal(outs[0].view(torch.uint8), o.view(torch.uint8))
