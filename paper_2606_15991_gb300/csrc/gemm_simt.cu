@@ -14,7 +14,19 @@
 namespace tp {
 namespace {
 
-constexpr int BM = 64, BN = 64, TH = 256;
+constexpr int BM = 64, BN = 64;
+
+constexpr int TM = 8, TN = 4;                   // elements per thread
+constexpr int TX = BN / TN, TY = BM / TM;       // threads along the columns and the rows
+constexpr int TH = TX * TY;                     // 128
+constexpr int KC = 32;                          // K elements per ring stage
+constexpr int kStages = 3;
+constexpr int kPitchA = KC + 4, kPitchB = BN + 4;  // floats per row of a stage's A (64 x KC) and B (KC x 64)
+constexpr int kStageA = BM * kPitchA;           // floats
+constexpr int kStage = kStageA + KC * kPitchB;
+constexpr size_t kSmem = (size_t)kStages * kStage * sizeof(float);
+constexpr int kCtas = 4;                        // CTAs that share an SM (128 registers a thread, 53 KB each)
+static_assert(kSmem >= BM * BN * sizeof(float), "a split program's partial block overlays the ring");
 
 struct SimtArgs {
   const float* a;
@@ -25,6 +37,7 @@ struct SimtArgs {
   int64_t gm, gn;              // tile grid
   int32_t kind, group_m;
   int32_t split;               // K slices per tile (cluster size); 1 = none
+  int32_t bk;                  // K granularity of the slices (cfg.bk)
   unsigned* queue;
   uint32_t* counts;
   int32_t* owner;
@@ -42,155 +55,233 @@ __device__ __forceinline__ void raster(int64_t s, int64_t gm, int64_t gn, int64_
   *tn = r / rows;
 }
 
-// Each of the 256 threads owns a 4 x 4 block of the tile: rows 4*ty..4*ty+3
-// and columns 4*tx..4*tx+3 (ty = tid / 16, tx = tid % 16). Shared memory
-// holds the A slice K-major (As[k][m]) and the B slice as stored (Bs[k][n]),
-// rows padded by 4 floats, so one 16-byte load gives a thread its 4 A or 4 B
-// values of a k step. The next K slice is loaded into registers while the
-// current one is multiplied (register-staged double buffering), so the
-// global-memory latency overlaps the FFMAs.
-// With split = S > 1 a tile program is a cluster of S CTAs: CTA r runs the
-// K slices [r*nk/S, (r+1)*nk/S) and keeps its partial 64 x 64 block in
+// Asynchronous copy of `bytes` (0..kBytes) from global to shared memory, the
+// rest of the kBytes zero-filled.
+template <int kBytes>
+__device__ __forceinline__ void copy_async(uint32_t dst, const float* src, int bytes) {
+  if constexpr (kBytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// Two FP32 fused multiply-adds, each rounded as fmaf rounds.
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+
+// How a block of an operand reaches shared memory.
+enum Fetch : int {
+  kRows16,  // 16-byte copies: contiguous block rows on 16-byte boundaries
+  kRows4,   // 4-byte copies, a warp along a block row
+  kCols4,   // 4-byte copies, a warp on 8 block rows x 4 columns: contiguous block columns
+};
+
+// Copies the valid part (nrows x ncols) of a kR x kC block at `src` (element
+// strides srow, scol) to `dst` (kPitch floats per row) and zero-fills the
+// rest. A warp's copies write distinct banks in every form (kPitch mod 32 = 4).
+template <int kFetch, int kR, int kC, int kPitch>
+__device__ __forceinline__ void fetch_block(uint32_t dst, const float* src, int64_t srow, int64_t scol, int nrows, int ncols) {
+  static_assert(kPitch % 32 == 4, "kCols4 writes 8 rows x 4 columns at once");
+  const int tid = threadIdx.x;
+  // opaque to the compiler, which would otherwise keep every copy's offset in
+  // registers across the K loop and spill the accumulators
+  asm volatile("" : "+l"(srow), "+l"(scol), "+r"(nrows));
+  if constexpr (kFetch == kRows16) {
+    constexpr int kQ = kC / 4;  // 16-byte pieces per row
+    const int c = tid % kQ * 4, r0 = tid / kQ;
+    const int valid = max(0, min(4, ncols - c)) * 4;
+    const float* at = src + r0 * srow + c;
+#pragma unroll
+    for (int e = 0; e < kR * kQ / TH; ++e) {
+      const int row = r0 + e * (TH / kQ);
+      const int bytes = row < nrows ? valid : 0;
+      copy_async<16>(dst + (uint32_t)(row * kPitch + c) * 4, bytes ? at : src, bytes);
+      at += (TH / kQ) * srow;
+    }
+  } else if constexpr (kFetch == kRows4) {
+    const int c = tid % kC, r0 = tid / kC;
+    const float* at = src + r0 * srow + c * scol;
+#pragma unroll
+    for (int e = 0; e < kR * kC / TH; ++e) {
+      const int row = r0 + e * (TH / kC);
+      const int bytes = row < nrows && c < ncols ? 4 : 0;
+      copy_async<4>(dst + (uint32_t)(row * kPitch + c) * 4, bytes ? at : src, bytes);
+      at += (TH / kC) * srow;
+    }
+  } else {
+    // warp w takes the 8 x 4 blocks w, w + 4, ... of the block, down the rows first
+    constexpr int kRB = kR / 8;
+#pragma unroll
+    for (int e = 0; e < kR * kC / TH; ++e) {
+      const int blk = e * (TH / 32) + tid / 32;
+      const int row = blk % kRB * 8 + (tid & 7), c = blk / kRB * 4 + (tid >> 3 & 3);
+      const int bytes = row < nrows && c < ncols ? 4 : 0;
+      copy_async<4>(dst + (uint32_t)(row * kPitch + c) * 4, bytes ? src + row * srow + c * scol : src, bytes);
+    }
+  }
+}
+
+// FP32 GEMM fed by asynchronous copies. Each of the 128 threads owns an 8 x 4
+// block of the tile and multiplies with the two-wide FMA, whose pairs are
+// neighbouring columns (one B load) times a duplicated A element: a single
+// FFMA stream peaks at 57-69 TFLOP/s on this chip for its register reads, the
+// two-wide form at 70-76. K arrives in chunks of 32 through a ring of three
+// stages, one block barrier per chunk; four CTAs share an SM, so their
+// barriers, shared-memory loads and tails overlap. A's rows stay as stored
+// (padded to 36 floats: the four rows a warp reads at once lie in different
+// banks), so a thread's four k of a row are one 16-byte load.
+// Bound by the FMA pipe (69 % busy at 2048^3, ncu) and the issue of what feeds
+// it: 49 TFLOP/s at 2048^3 aligned, 47 unaligned (the register-staged kernel
+// that this replaces, 256 threads of 4 x 4 at one CTA per SM: 41 fed by TMA,
+// 27 unaligned); 1000 x 3001 x 777, nothing aligned, 184 -> 113 us. Blocks of
+// 8 x 8 (64 threads) and 4 x 4 (256) ran 2048^3 at 45 and 43 TFLOP/s; pairs
+// along K, which need no duplication, leave no registers to load ahead: 35.
+// With split = S > 1 a tile program is a cluster of S CTAs: CTA r runs the K
+// steps [r*n/S, (r+1)*n/S) of cfg.bk and keeps its partial 64 x 64 block in
 // shared memory; after a cluster barrier CTA r adds, for rows
 // [r*64/S, (r+1)*64/S), the S partials in slice order 0..S-1 (reading the
-// others through distributed shared memory) and stores them, so every
-// element still has one writer and C is bit-reproducible.
-template <int BK, bool COUNT>
-__global__ void __launch_bounds__(TH, 1) gemm_f32_kernel(const __grid_constant__ SimtArgs p) {
-  constexpr int PA = BM * BK / TH;  // A elements per thread per K slice
-  constexpr int PB = BK * BN / TH;
-  // the operand buffers; a split program's partial block overlays them once
-  // its K loop has ended
-  constexpr int kAB = 2 * BK * (BM + 4) + 2 * BK * (BN + 4);
-  __shared__ __align__(16) float raw[kAB > BM * BN ? kAB : BM * BN];
-  auto As = reinterpret_cast<float(*)[BK][BM + 4]>(raw);
-  auto Bs = reinterpret_cast<float(*)[BK][BN + 4]>(raw + 2 * BK * (BM + 4));
-  auto Ps = reinterpret_cast<float(*)[BN]>(raw);
+// others through distributed shared memory) and stores them, so every element
+// still has one writer and C is bit-reproducible.
+template <int kFetchA, int kFetchB, bool COUNT>
+__global__ void __launch_bounds__(TH, kCtas) gemm_f32_kernel(const __grid_constant__ SimtArgs p) {
+  extern __shared__ __align__(16) float smem[];
   __shared__ int64_t slot;
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
+  const uint32_t base = sm100::smem_u32(smem);
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  // a warp is 8 threads along the columns x 4 along the rows; a thread's rows
+  // are ty + TY i and its columns 4 tx .. 4 tx + 3
+  const int tx = warp % (TX / 8) * 8 + (lane & 7), ty = warp / (TX / 8) * 4 + (lane >> 3);
   const int64_t T = p.gm * p.gn;
   const int S = p.split;
   const uint32_t r = S > 1 ? sm100::cluster_ctarank() : 0u;
+  // the operands may be the previous kernel's output, and C its input
+  sm100::grid_dependency_wait();
+  sm100::allow_dependents();
   int64_t s = S > 1 ? (int64_t)(blockIdx.x / S) : (int64_t)blockIdx.x;
   if (p.kind == TP_MAP_QUEUE) {
     if (tid == 0) slot = atomicAdd(p.queue, 1u);
     __syncthreads();
     s = slot;
   }
+  // this CTA's K slice, in whole steps of bk
+  const int64_t steps = (p.K + p.bk - 1) / p.bk;
+  const int64_t kbeg = S > 1 ? (int64_t)r * steps / S * p.bk : 0;
+  const int64_t kend = S > 1 ? min(p.K, (int64_t)(r + 1) * steps / S * p.bk) : p.K;
+  const int nch = kend > kbeg ? (int)((kend - kbeg + KC - 1) / KC) : 0;
   while (s < T) {
     int64_t tm, tn;
     raster(s, p.gm, p.gn, p.group_m, &tm, &tn);
     const int64_t m0 = tm * BM, n0 = tn * BN;
-    float acc[4][4] = {};
-    const int64_t nk_all = (p.K + BK - 1) / BK;
-    const int64_t kt0 = (int64_t)r * nk_all / S, kt1 = (int64_t)(r + 1) * nk_all / S;
-    const int64_t nk = kt1 - kt0;
-    float ra[PA], rb[PB];
-    // element e of this thread's share: A (row e*TH/BK + tid/BK, k tid%BK),
-    // B (k e*TH/BN + tid/BN, column tid%BN): consecutive threads read
-    // consecutive k of A and consecutive n of B
-    auto fetch = [&](int64_t k0) {
-#pragma unroll
-      for (int e = 0; e < PA; ++e) {
-        const int i = e * TH + tid;
-        const int64_t gm_ = m0 + i / BK, gk = k0 + i % BK;
-        ra[e] = (gm_ < p.M && gk < p.K) ? p.a[gm_ * p.sam + gk * p.sak] : 0.f;
-      }
-#pragma unroll
-      for (int e = 0; e < PB; ++e) {
-        const int i = e * TH + tid;
-        const int64_t gk = k0 + i / BN, gn_ = n0 + i % BN;
-        rb[e] = (gk < p.K && gn_ < p.N) ? p.b[gk * p.sbk + gn_ * p.sbn] : 0.f;
-      }
+    const int mrows = (int)min((int64_t)BM, p.M - m0), ncols = (int)min((int64_t)BN, p.N - n0);
+    // chunk ch of the slice into its ring stage
+    auto load = [&](int ch) {
+      const int64_t k0 = kbeg + (int64_t)ch * KC;
+      const int klen = (int)min((int64_t)KC, kend - k0);
+      const uint32_t sa = base + (uint32_t)((ch % kStages) * kStage * 4);
+      fetch_block<kFetchA, BM, KC, kPitchA>(sa, p.a + m0 * p.sam + k0 * p.sak, p.sam, p.sak, mrows, klen);
+      fetch_block<kFetchB, KC, BN, kPitchB>(sa + kStageA * 4, p.b + k0 * p.sbk + n0 * p.sbn, p.sbk, p.sbn, klen, ncols);
     };
-    auto stash = [&](int buf) {
+    uint64_t acc[TM][TN / 2];  // pairs of neighbouring columns
 #pragma unroll
-      for (int e = 0; e < PA; ++e) {
-        const int i = e * TH + tid;
-        As[buf][i % BK][i / BK] = ra[e];
-      }
+    for (int i = 0; i < TM; ++i) acc[i][0] = acc[i][1] = 0;
 #pragma unroll
-      for (int e = 0; e < PB; ++e) {
-        const int i = e * TH + tid;
-        Bs[buf][i / BN][i % BN] = rb[e];
-      }
-    };
-    if (nk > 0) {
-      fetch(kt0 * BK);
-      stash(0);
+    for (int ch = 0; ch < kStages - 1; ++ch) {
+      if (ch < nch) load(ch);
+      asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    __syncthreads();
-    for (int64_t kt = 0; kt < nk; ++kt) {
-      const int buf = kt & 1;
-      if (kt + 1 < nk) fetch((kt0 + kt + 1) * BK);
+    for (int ch = 0; ch < nch; ++ch) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+      __syncthreads();  // chunk ch has landed for every thread, and chunk ch - 1's stage is free
+      if (ch + kStages - 1 < nch) load(ch + kStages - 1);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      const float* As = smem + (ch % kStages) * kStage + ty * kPitchA;
+      const float* Bs = smem + (ch % kStages) * kStage + kStageA + 4 * tx;
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        const float4 a4 = *reinterpret_cast<const float4*>(&As[buf][kk][4 * ty]);
-        const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][kk][4 * tx]);
-        const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-        const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
+      for (int g = 0; g < KC / 4; ++g) {
+        float4 av[TM], bv[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(As + TY * i * kPitchA + 4 * g);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-      }
-      if (kt + 1 < nk) stash(buf ^ 1);  // the other buffer's readers passed the barrier below last step
-      __syncthreads();
-    }
-    bool mine = true;  // this thread's rows are stored by this CTA
-    if (S > 1) {
+        for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(Bs + (4 * g + j) * kPitchB);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<float4*>(&Ps[4 * ty + i][4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-      sm100::cluster_sync();  // every CTA's partial is in its shared memory
-      mine = (4 * ty) / (BM / S) == (int)r;
-      if (mine) {
-        float sum[4][4];
-        for (int src = 0; src < S; ++src) {
+        for (int j = 0; j < 4; ++j) {
+          const uint64_t b01 = pack2(bv[j].x, bv[j].y), b23 = pack2(bv[j].z, bv[j].w);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            float4 v;
-            if (src == (int)r) {
-              v = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-            } else {
-              const uint32_t at = sm100::mapa(sm100::smem_u32(&Ps[4 * ty + i][4 * tx]), (uint32_t)src);
-              asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                           : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                           : "r"(at)
-                           : "memory");
-            }
-            const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) sum[i][j] = src == 0 ? vv[j] : sum[i][j] + vv[j];
+          for (int i = 0; i < TM; ++i) {
+            const float a = j == 0 ? av[i].x : j == 1 ? av[i].y : j == 2 ? av[i].z : av[i].w;
+            const uint64_t aa = pack2(a, a);
+            fma2(acc[i][0], aa, b01);
+            fma2(acc[i][1], aa, b23);
           }
         }
+      }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    float4 out[TM];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i) {
+      const float2 lo = unpack2(acc[i][0]), hi = unpack2(acc[i][1]);
+      out[i] = make_float4(lo.x, lo.y, hi.x, hi.y);
+    }
+    __syncthreads();  // the ring is free (the next tile's loads, the partial block below)
+    // this thread's row i is stored by this CTA
+    auto mine = [&](int i) { return S == 1 || (ty + TY * i) / (BM / S) == (int)r; };
+    if (S > 1) {
+      // the partial blocks meet through distributed shared memory: CTA r adds
+      // rows [r*64/S, +64/S) of the S partials in slice order
+      float(*Ps)[BN] = reinterpret_cast<float(*)[BN]>(smem);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = sum[i][j];
+      for (int i = 0; i < TM; ++i) *reinterpret_cast<float4*>(&Ps[ty + TY * i][4 * tx]) = out[i];
+      sm100::cluster_sync();  // every CTA's partial is in its shared memory
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        if (!mine(i)) continue;
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int src = 0; src < S; ++src) {
+          float4 v = out[i];
+          if (src != (int)r) {
+            const uint32_t at = sm100::mapa(sm100::smem_u32(&Ps[ty + TY * i][4 * tx]), (uint32_t)src);
+            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                         : "r"(at)
+                         : "memory");
+          }
+          sum = src == 0 ? v : make_float4(sum.x + v.x, sum.y + v.y, sum.z + v.z, sum.w + v.w);
+        }
+        out[i] = sum;
       }
       sm100::cluster_sync();  // the peers' reads of this CTA's partial are done
     }
     const bool vec = (p.N % 4 == 0) && ((reinterpret_cast<uintptr_t>(p.c) & 15) == 0);
 #pragma unroll
-    for (int i = 0; i < 4 && mine; ++i) {
-      const int64_t r = m0 + 4 * ty + i;
-      if (r >= p.M) continue;
-      const int64_t c0 = n0 + 4 * tx;
-      if (vec && c0 + 4 <= p.N) {
-        *reinterpret_cast<float4*>(p.c + r * p.N + c0) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    for (int i = 0; i < TM; ++i) {
+      if (!mine(i) || ty + TY * i >= mrows) continue;
+      const int64_t e = (m0 + ty + TY * i) * p.N + n0 + 4 * tx;
+      const float f[4] = {out[i].x, out[i].y, out[i].z, out[i].w};
+      if (vec && 4 * tx + 4 <= ncols) {
+        *reinterpret_cast<float4*>(p.c + e) = out[i];
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (c0 + j < p.N) p.c[r * p.N + c0 + j] = acc[i][j];
+          if (4 * tx + j < ncols) p.c[e + j] = f[j];
       }
       if constexpr (COUNT) {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (c0 + j < p.N) {
-            atomicAdd(p.counts + r * p.N + c0 + j, 1u);
-            p.owner[r * p.N + c0 + j] = (int32_t)(blockIdx.x / S);
+          if (4 * tx + j < ncols) {
+            atomicAdd(p.counts + e + j, 1u);
+            p.owner[e + j] = (int32_t)(blockIdx.x / S);
           }
       }
     }
@@ -206,39 +297,75 @@ __global__ void __launch_bounds__(TH, 1) gemm_f32_kernel(const __grid_constant__
   }
 }
 
-template <int BK>
-cudaError_t launch_bk(const SimtArgs& p, bool count, int64_t grid, cudaStream_t st) {
+template <int kFetchA, int kFetchB, bool COUNT>
+cudaError_t launch_inst(const SimtArgs& p, int64_t programs, cudaStream_t st) {
+  auto k = gemm_f32_kernel<kFetchA, kFetchB, COUNT>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(grid * p.split));
+  cfg.gridDim = dim3((unsigned)(programs * p.split));
   cfg.blockDim = dim3(TH);
+  cfg.dynamicSmemBytes = kSmem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)p.split;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return count ? cudaLaunchKernelEx(&cfg, gemm_f32_kernel<BK, true>, p)
-               : cudaLaunchKernelEx(&cfg, gemm_f32_kernel<BK, false>, p);
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, k, p);
+}
+
+// The fetch of an operand whose block rows have element stride `row` and
+// whose block columns have stride `col`.
+int fetch_of(const float* ptr, int64_t row, int64_t col) {
+  if (col == 1 && row % 4 == 0 && (reinterpret_cast<uintptr_t>(ptr) & 15) == 0) return kRows16;
+  return row == 1 && col != 1 ? kCols4 : kRows4;
+}
+
+template <int kFetchA>
+cudaError_t launch_b(const SimtArgs& p, int fetch_b, int64_t programs, cudaStream_t st) {
+  switch (fetch_b) {
+    case kRows16: return launch_inst<kFetchA, kRows16, false>(p, programs, st);
+    case kRows4: return launch_inst<kFetchA, kRows4, false>(p, programs, st);
+    default: return launch_inst<kFetchA, kCols4, false>(p, programs, st);
+  }
+}
+
+cudaError_t launch_async(const SimtArgs& p, int64_t programs, cudaStream_t st) {
+  // instrumented launches: one form for every layout
+  if (p.counts) return launch_inst<kRows4, kRows4, true>(p, programs, st);
+  const int fb = fetch_of(p.b, p.sbk, p.sbn);
+  switch (fetch_of(p.a, p.sam, p.sak)) {
+    case kRows16: return launch_b<kRows16>(p, fb, programs, st);
+    case kRows4: return launch_b<kRows4>(p, fb, programs, st);
+    default: return launch_b<kCols4>(p, fb, programs, st);
+  }
 }
 
 // ------------------------------------------------ TMA-fed FP32 GEMM
-// The same tiles, thread blocking, K order and split-K reduction as
-// gemm_f32_kernel (so the same C bit for bit), with the operands brought by
-// TMA: a producer thread copies each 32-wide K chunk of the tile's A rows
-// (64 x 32 floats, 128-byte rows, 128-byte swizzle) and B columns (32 x 64
-// floats, 256-byte rows) into a ring of 16 KB stages while eight compute
-// warps multiply the chunks already landed; no register staging, no block
-// barrier per K step. Used for identity and strided maps with unit-stride,
-// 16-byte-aligned operands (and split-K only when each program holds one
-// tile); other launches take gemm_f32_kernel.
+// The same tiles, K order and split-K reduction as gemm_f32_kernel (so the
+// same C bit for bit) for launches that leave an SM one CTA at most: a
+// producer thread copies each 32-wide K chunk of the tile's A rows (64 x 32
+// floats, 128-byte rows, 128-byte swizzle) and B columns (32 x 64 floats,
+// 256-byte rows) into a ring of 16 KB stages while eight compute warps (4 x 4
+// elements per thread) multiply the chunks already landed, with no block
+// barrier per K step. Alone on its SM the eight warps hide each other's
+// latencies better than gemm_f32_kernel's four: 512^3 split in two (128 CTAs)
+// 11.9 us against 15.2, one tile of K = 512 17.5 against 18.4; with two CTAs
+// per SM and more the order turns (1024^3, 256 CTAs: 63.3 against 56.9).
+// Five stages and 96 registers, so that the next launch's CTAs could move in
+// early, were no faster (12.0 us).
 constexpr int kFChunk = 32;
 constexpr int kFStages = 8;
 constexpr uint32_t kFChunkA = BM * kFChunk * 4;  // 8 KB
 constexpr uint32_t kFChunkB = kFChunk * BN * 4;  // 8 KB
 constexpr uint32_t kFStageBytes = kFChunkA + kFChunkB;
-constexpr int kFThreads = TH + 32;               // eight compute warps + the producer warp
+constexpr int kFWarps = 8;                       // compute warps (4 x 4 elements per thread)
+constexpr int kFThreads = 32 * kFWarps + 32;     // + the producer warp
 constexpr size_t kFSmem = 1024 + (size_t)kFStages * kFStageBytes + BM * BN * 4 + 8 * (2 * kFStages) + 16;
 
 struct F32TmaArgs {
@@ -273,7 +400,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
   if (tid == 0) {
     for (int s = 0; s < kFStages; ++s) {
       mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), TH / 32);
+      mbar_init(empty_bar(s), kFWarps);
     }
     *abort_flag = 0;
     fence_mbar_init();
@@ -288,7 +415,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
   const int64_t s0 = (int64_t)(blockIdx.x / S);
   const int64_t step = p.kind == TP_MAP_IDENTITY ? T : (int64_t)(gridDim.x / S);
   const int32_t c0 = (int32_t)(((int64_t)r * p.nchunks) / S), c1 = (int32_t)(((int64_t)(r + 1) * p.nchunks) / S);
-  if (warp == TH / 32) {
+  if (warp == kFWarps) {
     // ---------------- producer
     if (lane == 0) {
       uint32_t fills[kFStages] = {};
@@ -322,7 +449,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     return;
   }
   // ---------------- compute warps: thread (tx, ty) owns rows 4ty..4ty+3 and
-  // columns 4tx..4tx+3 of the tile, as in gemm_f32_kernel
+  // columns 4tx..4tx+3 of the tile
   const int tx = tid % 16, ty = tid / 16;
   int stage = 0;
   uint32_t phase = 0;
@@ -520,21 +647,24 @@ tp_status launch_gemm_simt(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, con
   p.owner = ex->write_owner;
   if (p.M == 0 || p.N == 0) return TP_OK;
   const int64_t grid = c->kind == TP_MAP_IDENTITY ? c->num_tiles : c->num_programs;
-  const int bk = (cfg && cfg->bk > 0) ? cfg->bk : 32;  // 32: fewest barriers per K (fastest at 512^3)
+  const int bk = (cfg && cfg->bk > 0) ? cfg->bk : 32;
   p.split = (cfg && cfg->split_k > 1) ? cfg->split_k : 1;
   if (cfg && (cfg->split_k < 0 || cfg->split_k > 4 || (p.split & (p.split - 1))))
     return fail(TP_ERR_INVALID, "FP32 GEMM split_k must be 0, 1, 2 or 4");
   if (p.split > 1 && c->kind == TP_MAP_QUEUE)
     return fail(TP_ERR_UNSUPPORTED, "FP32 GEMM split_k with a queue map (each CTA would dequeue its own tile)");
+  if (bk != 8 && bk != 16 && bk != 32) return fail(TP_ERR_UNSUPPORTED, "FP32 GEMM bk must be 8, 16 or 32");
+  p.bk = bk;
   const bool count = p.counts != nullptr;
   cudaError_t e;
-  // TMA-fed kernel: unit-stride rows 16-byte aligned, K chunks of 32 (the
-  // bk = 32 schedule), identity or strided maps, split programs one tile each
+  // TMA-fed kernel: at most one CTA per SM (measured where the kernel is
+  // defined), unit-stride rows 16-byte aligned, K chunks of 32 (the bk = 32
+  // schedule), identity or strided maps, split programs one tile each
   const int64_t T = p.gm * p.gn;
   const bool tma_ok = bk == 32 && p.sak == 1 && p.sbn == 1 && p.sam % 4 == 0 && p.sbk % 4 == 0 &&
                       ((reinterpret_cast<uintptr_t>(p.a) | reinterpret_cast<uintptr_t>(p.b)) & 15) == 0 &&
                       p.K > 0 && p.K < ((int64_t)1 << 30) && p.M < ((int64_t)1 << 31) && p.N < ((int64_t)1 << 31) &&
-                      c->kind != TP_MAP_QUEUE && (p.split == 1 || grid >= T);
+                      c->kind != TP_MAP_QUEUE && (p.split == 1 || grid >= T) && grid * p.split <= ctx->sm_count;
   if (tma_ok) {
     CUtensorMap ma, mb;
     if (f32_map(&ma, p.a, p.M, p.K, p.sam, kFChunk, BM, true) && f32_map(&mb, p.b, p.K, p.N, p.sbk, BN, kFChunk, false)) {
@@ -558,12 +688,7 @@ tp_status launch_gemm_simt(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, con
       return TP_OK;
     }
   }
-  switch (bk) {
-    case 8: e = launch_bk<8>(p, count, grid, stream); break;
-    case 16: e = launch_bk<16>(p, count, grid, stream); break;
-    case 32: e = launch_bk<32>(p, count, grid, stream); break;
-    default: return fail(TP_ERR_UNSUPPORTED, "FP32 GEMM bk must be 8, 16 or 32");
-  }
+  e = launch_async(p, grid, stream);
   if (e != cudaSuccess) return cuda_fail(e, "FP32 GEMM launch");
   return TP_OK;
 }

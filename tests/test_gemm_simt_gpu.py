@@ -183,3 +183,44 @@ def test_tma_fed_kernel_equals_register_staged(ctx, m, n, k, split, kind, P, gro
     expect = (opart.gemm_owner_map(m, n, 64, 64) if kind == tp.MAP_IDENTITY
               else opart.gemm_owner_map(m, n, 64, 64, P, "strided", group_m))
     assert np.array_equal(owner.cpu().numpy(), expect)
+
+
+@pytest.mark.parametrize("m,n,k,split", [
+    (1, 1, 1, 1), (64, 64, 32, 1),               # one element; exactly one tile and one K chunk
+    (63, 65, 31, 1), (65, 63, 33, 1),            # one short of and one past a tile and a chunk
+    (130, 190, 97, 2), (128, 64, 100, 4),        # split slices of unequal and of whole chunks
+    (300, 260, 70, 1),
+])
+def test_operand_layouts_give_one_result(ctx, m, n, k, split):
+    """Every layout of A and B (rows on 16-byte boundaries, off them, or stored
+    transposed; a queue map keeps aligned operands off the TMA path) takes each
+    sum in the same order, so C is equal bit for bit, and within the FP32
+    summation bound k * 2^-24 * sum |a b| of the FP64 oracle."""
+    a = torch.from_numpy(synth.uniform(m * k, seed=m + 2 * k)).reshape(m, k).cuda()
+    b = torch.from_numpy(synth.uniform(k * n, seed=n + 5)).reshape(k, n).cuda()
+
+    def off(t):
+        buf = torch.empty(t.numel() + 1, device="cuda")
+        v = buf[1:].view(t.shape)
+        v.copy_(t)
+        return v
+
+    def padded(t):                               # row pitch a multiple of 4 floats
+        buf = torch.zeros(t.shape[0], (t.shape[1] + 7) // 4 * 4, device="cuda")
+        v = buf[:, :t.shape[1]]
+        v.copy_(t)
+        return v
+
+    def transposed(t):
+        return t.t().contiguous().t()
+
+    tiles = -(-m // 64) * -(-n // 64)
+    want, _, _ = _gemm(ctx, a, b, bk=32, split_k=split)
+    for fa in (padded, off, transposed):
+        for fb in (padded, off, transposed):
+            kind, P = (tp.MAP_QUEUE, min(2, tiles)) if split == 1 else (tp.MAP_STRIDED, 1)
+            c, _, _ = _gemm(ctx, fa(a), fb(b), kind, P, bk=32, split_k=split)
+            assert torch.equal(c, want)
+    an, bn_ = a.cpu().double().numpy(), b.cpu().double().numpy()
+    bound = (k + 4) * 2.0 ** -24 * (np.abs(an) @ np.abs(bn_)) + 1e-37
+    assert np.all(np.abs(want.cpu().double().numpy() - ogemm.gemm(a.cpu(), b.cpu())) <= bound)
