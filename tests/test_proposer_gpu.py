@@ -341,3 +341,45 @@ def test_swap_ab_search_is_opt_in(ctx):
         tp.tp_partition_destroy(p)
         outs.append(c)
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[1], outs[2])
+
+
+@pytest.mark.parametrize("f,h,c,b", [
+    (1, 1, 1, 1),            # one unit everywhere, half a CTA of rows
+    (5, 33, 9, 129),         # one past a block's columns, rows and batch chunk
+    (7, 130, 129, 3),        # more units than a row has threads
+    (5, 64, 72, 257),        # the proposer's network, three batch chunks
+    (3, 300, 20, 40),        # weights too large to be staged in shared memory
+])
+def test_mlp_sizes_match_oracle(ctx, f, h, c, b):
+    """Forward, loss, gradients and one Adam step at the edges of the kernels'
+    blocks, against the FP64 oracle (bounds as for the proposer's network)."""
+    p0 = proposer.init_params(f, h, c, seed=3)
+    X = synth.uniform(b * f, 1, 0, 4, dtype=np.float64).reshape(b, f).astype(np.float32)
+    T = synth.uniform(b * c, 2, 0, 1, dtype=np.float64).reshape(b, c).astype(np.float32)
+    V = (synth.uniform(b * c, 3, 0, 1, dtype=np.float64) > 0.2).astype(np.float32).reshape(b, c)
+    P, o = {}, 0
+    for k, shape in (("W1", (h, f)), ("b1", (h,)), ("W2", (h, h)), ("b2", (h,)), ("W3", (c, h)), ("b3", (c,))):
+        n = int(np.prod(shape))
+        P[k] = np.asarray(p0[o:o + n], np.float64).reshape(shape)
+        o += n
+    m = tp.tp_mlp_create(ctx, f, h, c, b, p0)
+    Xd, Td, Vd = (torch.from_numpy(a).cuda() for a in (X, T, V))
+    Y, G, loss = torch.empty(b, c, device="cuda"), torch.empty(len(p0), device="cuda"), torch.zeros(1, device="cuda")
+    tp.tp_mlp_forward(m, Xd, Y)
+    Yref, cache = omlp.forward(P, X.astype(np.float64))
+    assert np.max(np.abs(Y.cpu().numpy() - Yref)) <= 1e-5 * max(1.0, np.abs(Yref).max())
+    tp.tp_mlp_loss_grad(m, Xd, Td, Vd, loss, G)
+    assert abs(loss.item() - omlp.loss(Yref, T, V)) <= 1e-5 * max(1e-30, omlp.loss(Yref, T, V))
+    grads = omlp.backward(P, cache, Yref, T, V)
+    gref = _flat(grads)
+    assert np.linalg.norm(G.cpu().numpy() - gref) <= 1e-4 * np.linalg.norm(gref) + 1e-12
+    zeros = {k: np.zeros_like(v) for k, v in P.items()}
+    tp.tp_mlp_train_step(m, Xd, Td, Vd, 1e-3, loss)
+    want = _flat(omlp.adam_step(P, grads, zeros, {k: v.copy() for k, v in zeros.items()}, 1, 1e-3)[0])
+    # the first step is -lr g / (|g| + 1e-8): where |g| is well above its FP32
+    # error it is sign(g); elsewhere the step is bounded by lr
+    got = tp.tp_mlp_get_params(m)
+    sure = np.abs(gref) > 1e-3 * np.abs(gref).max() + 1e-6
+    assert np.max(np.abs(got - want)[sure], initial=0.0) <= 2e-5
+    assert np.max(np.abs(got - p0)) <= 1.01e-3
+    tp.tp_mlp_destroy(m)
