@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "sm100_ptx.cuh"
 #include "tp_internal.h"
@@ -131,6 +132,8 @@ template <int kEpi, int kParts, int kUnroll, bool kCount>
 __global__ void __launch_bounds__(kThreads) gemv_kernel(const __grid_constant__ GemvArgs p) {
   extern __shared__ float xs[];  // k floats (+ reduction scratch)
   float* red = xs + ((p.k + 3) & ~int64_t(3));
+  sm100::allow_dependents();
+  sm100::grid_dependency_wait();
   // stage x (optionally normalised) in shared memory
   float scale = 1.f;
   if (p.norm) scale = block_rms_scale(p.x, p.k, p.eps, red);
@@ -273,6 +276,8 @@ struct StreamArgs {
   int64_t units0, units;    // units of problem 0, total units
   int64_t rows0, rows1;
   int32_t epi0, epi1;       // kPlain / kSiluPair / kResidual (partial sums when slices > 1)
+  int32_t rgroups;          // 4-row groups of a plain unit: 8, or 4, 2, 1 with 8 / rgroups column blocks per stage
+  int32_t box3;             // rgroups < 8: a stage is one 3-D box (else a 2-D box per column block)
   float* y0;
   float* y1;
   float* partial;
@@ -286,7 +291,7 @@ struct StreamArgs {
   int32_t* owner;
 };
 
-template <bool kCount>
+template <bool kCount, int kRg, bool kBulkX>
 __global__ void __launch_bounds__(kSThreads, 1)
     gemv_stream_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
                        const __grid_constant__ StreamArgs p) {
@@ -314,7 +319,12 @@ __global__ void __launch_bounds__(kSThreads, 1)
   // values (warp w's at [4w, 4w + 4)), written to global memory kSOBuf units
   // at a time and at the end
   float* obuf = red + 16;
+  // rgroups < 8: the warps' sums of two consecutive units overlay it
+  float* psum = obuf;
   const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+  constexpr int rgroups = kRg, cblocks = kSConsumers / rgroups;
+  constexpr int urows = 4 * rgroups;             // rows of a plain unit
+  constexpr int stage_cols = kSCols * cblocks;   // columns of a stage
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) {
       mbar_init(full_bar(s), 1);
@@ -341,7 +351,15 @@ __global__ void __launch_bounds__(kSThreads, 1)
   auto consumers_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kSConsumers * 32) : "memory"); };
   if (warp < kSConsumers) {
     grid_dependency_wait();
-    if (p.slices == 1) {
+    if (kBulkX) {
+      // the producer copies the whole 16-byte pieces of x; the last k % 4
+      // elements are stored here
+      const int tail = (int)(p.k & 3);
+      if (threadIdx.x < tail) xsp[p.k - tail + threadIdx.x] = p.x[p.k - tail + threadIdx.x];
+      const bool got = p.k < 4 || mbar_wait(xfull_bar(0), 0, abort_flag, p.err, p.wait_ns);
+      (void)got;  // a timeout shows in the next stage's wait
+      consumers_sync();
+    } else if (p.slices == 1) {
       // The whole of x (normalised) in shared memory. Each consumer thread
       // loads its 16-byte pieces of x (and of gamma) at once, up to
       // kSXVec of them, so the prologue waits about one memory latency,
@@ -410,7 +428,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
       consumers_sync();
     }
   }
-  const int64_t stages_per_unit = (p.slice_cols + kSCols - 1) / kSCols;
+  const int64_t stages_per_unit = (p.slice_cols + stage_cols - 1) / stage_cols;
   // unit u -> problem, row block, K slice
   auto decode_unit = [&](int64_t u, bool* second, int64_t* rb, int32_t* slice) {
     *second = u >= p.units0;
@@ -439,19 +457,36 @@ __global__ void __launch_bounds__(kSThreads, 1)
         decode_unit(u, &second, &rb, &slice);
         const bool pair = (second ? p.epi1 : p.epi0) == kSiluPair;
         const CUtensorMap* m = second ? &map1 : &map0;
-        const int32_t r0 = (int32_t)(rb * (pair ? kSPairRows : kSRows));
+        const int32_t r0 = (int32_t)(rb * (pair ? kSPairRows : urows));
         auto issue = [&](int64_t st) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.err, p.wait_ns)) return false;
-          const int32_t c0 = (int32_t)(slice * p.slice_cols + st * kSCols);  // 512-byte aligned
+          const int32_t c0 = (int32_t)(slice * p.slice_cols + st * stage_cols);  // 512-byte aligned
           const uint32_t dst = base + (uint32_t)kSStage * stage;
           mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kSStage);
           if (pair) tma_load_3d(dst, m, c0, r0, 0, full_bar(stage), pol);  // g rows, then their u rows
-          else tma_load_2d(dst, m, c0, r0, full_bar(stage), pol);
+          else if (rgroups < 8 && p.box3) tma_load_3d(dst, m, 0, r0, c0 / kSCols, full_bar(stage), pol);
+          else
+            for (int cb = 0; cb < cblocks; ++cb)  // a block past the last column arrives as zeros
+              tma_load_2d(dst + (uint32_t)(cb * urows * kSCols * 2), m, c0 + cb * kSCols, r0, full_bar(stage), pol);
           fills[stage]++;
           if (++stage == nst) { stage = 0; phase ^= 1u; }
           return true;
         };
         int64_t st = 0;
+        if (kBulkX && t == 0) {
+          // weights first when they may go early, then the whole of x
+          if (p.early_weights) {
+            for (; st < stages_per_unit && st < nst && ok; ++st) ok = issue(st);
+            if (!ok) break;
+            grid_dependency_wait();  // x is the previous kernels' output
+          }
+          const uint32_t bytes = (uint32_t)(p.k / 4) * 16u;
+          if (bytes) {
+            mbar_arrive_expect_tx(xfull_bar(0), bytes);
+            bulk_copy_g2s(xs0, p.x, bytes, xfull_bar(0));
+            xfills[0]++;
+          }
+        }
         if (p.slices > 1) {
           if (t == 0) {
             // consumers start on x only after this copy, so at most a ring's
@@ -542,6 +577,13 @@ __global__ void __launch_bounds__(kSThreads, 1)
         const bool got = mbar_wait(xfull_bar(xb), (uint32_t)((t / xbufs) & 1), abort_flag, p.err, p.wait_ns);
         if (!__all_sync(0xffffffffu, got)) break;
       }
+      // rgroups < 8: warp 0 stores the unit's rows (lane = row); the values a
+      // residual adds to are fetched ahead
+      float y0 = 0.f;
+      if (rgroups < 8 && epi == kResidual && warp == 0 && lane < urows && rb * urows + lane < p.rows0)
+        y0 = p.y0[rb * urows + lane];
+      // this warp's row group and column block
+      const int wrow = rgroups == 8 ? warp : warp % rgroups, wcol = rgroups == 8 ? 0 : warp / rgroups;
       // acc[q][j]: q = row (plain) or 2 * half + pair (SiLU); j = lane slot
       float acc[4][4];
 #pragma unroll
@@ -550,7 +592,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
         for (int j = 0; j < 4; ++j) acc[q][j] = 0.f;
       for (int64_t st = 0; st < stages_per_unit; ++st) {
         // this lane's 8 columns of x (zero past the valid part of the buffer)
-        const int64_t cx = st * kSCols + lane * 8;
+        const int64_t cx = st * stage_cols + wcol * kSCols + lane * 8;
         float xv[8];
         if (cx + 8 <= lim) {
           const float4 a = *reinterpret_cast<const float4*>(xs + cx);
@@ -566,8 +608,9 @@ __global__ void __launch_bounds__(kSThreads, 1)
         const uint32_t src = base + (uint32_t)kSStage * stage;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          // smem row of slot q: plain row 4w + q; SiLU half q / 2, pair 2w + q % 2
-          const uint32_t row = pair ? (uint32_t)((q >> 1) * kSPairRows + 2 * warp + (q & 1)) : (uint32_t)(4 * warp + q);
+          // smem row of slot q: plain row 4 wrow + q of column block wcol; SiLU half q / 2, pair 2w + q % 2
+          const uint32_t row = pair ? (uint32_t)((q >> 1) * kSPairRows + 2 * warp + (q & 1))
+                                    : (uint32_t)(wcol * urows + 4 * wrow + q);
           uint32_t w4[4];
           ld_shared_v4(src + row * (kSCols * 2) + (uint32_t)lane * 16u, w4);
           const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(w4);
@@ -596,6 +639,39 @@ __global__ void __launch_bounds__(kSThreads, 1)
         for (int o = 16; o > 0; o >>= 1) tq += __shfl_xor_sync(0xffffffffu, tq, o);
         sum[q] = tq;
       }
+      if constexpr (rgroups < 8) {
+        // psum[unit parity][column block][row], handed to warp 0 (which adds
+        // the blocks in order and stores) and back by two of the barriers
+        // that only K slices use otherwise; the other warps go on
+        const int par = (int)(t & 1);
+        const uint32_t use = (uint32_t)((t >> 1) & 1);
+        const uint32_t ps_full = xempty_bar(par), ps_empty = xfull_bar(2 + par);
+        float* ps = psum + par * kSRows;
+        bool got = mbar_wait(ps_empty, use ^ 1u, abort_flag, p.err, p.wait_ns);
+        if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+        if (lane == 0) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) ps[wcol * urows + 4 * wrow + q] = sum[q];
+          mbar_arrive(ps_full);
+        }
+        if (warp == 0) {
+          got = mbar_wait(ps_full, use, abort_flag, p.err, p.wait_ns);
+          if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+          const int64_t r = rb * urows + lane;
+          if (lane < urows && r < p.rows0) {
+            float v = 0.f;
+            for (int cb = 0; cb < cblocks; ++cb) v += ps[cb * urows + lane];
+            p.y0[r] = y0 + v;
+            if constexpr (kCount) {
+              atomicAdd(p.counts + r, 1u);
+              p.owner[r] = (int32_t)blockIdx.x;
+            }
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(ps_empty);
+        }
+        continue;
+      }
       if (lane == 0) {
         float* ob = obuf + (t % kSOBuf) * kSRows + 4 * warp;
         if (pair && p.slices == 1) {
@@ -619,28 +695,98 @@ struct VecArgs {
   float* y;
   int64_t n;
   float eps;
-  int32_t op;  // 0 rmsnorm (a = h, b = gamma), 1 silu_mul (a = gu), 2 residual add (y += a)
+  int32_t op;  // 1 silu_mul (a = gu), 2 residual add (y += a)
   uint32_t* counts;
   int32_t* owner;
 };
 
 template <bool kCount>
+__device__ __forceinline__ void count_elem(const VecArgs& p, int64_t i) {
+  if constexpr (kCount) {
+    atomicAdd(p.counts + i, 1u);
+    p.owner[i] = (int32_t)blockIdx.x;
+  }
+}
+
+template <bool kCount>
 __global__ void __launch_bounds__(kThreads) vec_kernel(const __grid_constant__ VecArgs p) {
-  __shared__ float red[kWarps];
-  float scale = 1.f;
-  if (p.op == 0) scale = block_rms_scale(p.a, p.n, p.eps, red);
+  sm100::allow_dependents();
+  sm100::grid_dependency_wait();
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < p.n; i += stride) {
-    float v;
-    if (p.op == 0) v = p.a[i] * scale * (p.b ? p.b[i] : 1.f);
-    else if (p.op == 1) v = silu(p.a[i]) * p.a[i + p.n];
-    else v = p.y[i] + p.a[i];
-    p.y[i] = v;
-    if constexpr (kCount) {
-      atomicAdd(p.counts + i, 1u);
-      p.owner[i] = (int32_t)blockIdx.x;
-    }
+    p.y[i] = p.op == 1 ? silu(p.a[i]) * p.a[i + p.n] : p.y[i] + p.a[i];
+    count_elem<kCount>(p, i);
   }
+}
+
+// y = a / sqrt(mean(a^2) + eps) * b (b null: 1) by one CTA: the scale needs
+// the whole vector, a hidden size of a few thousand. Latency-bound: up to
+// kRmsHeld elements per thread, and their gammas, are fetched in one round
+// trip and kept in registers (the rest is read twice). 5120 elements took
+// 4.4 us (ncu) with 256 threads reading the vector twice, one element at a
+// time.
+constexpr int kRmsThreads = 1024;
+constexpr int kRmsHeld = 8;
+
+template <bool kCount>
+__global__ void __launch_bounds__(kRmsThreads) rmsnorm_kernel(const __grid_constant__ VecArgs p) {
+  __shared__ float red[kRmsThreads / 32];
+  sm100::allow_dependents();
+  sm100::grid_dependency_wait();
+  constexpr int64_t kHeld = (int64_t)kRmsThreads * kRmsHeld;
+  float v[kRmsHeld], g[kRmsHeld];
+#pragma unroll
+  for (int j = 0; j < kRmsHeld; ++j) {
+    const int64_t i = threadIdx.x + (int64_t)j * kRmsThreads;
+    v[j] = i < p.n ? p.a[i] : 0.f;
+    g[j] = i < p.n && p.b ? p.b[i] : 1.f;
+  }
+  float s = 0.f;
+#pragma unroll
+  for (int j = 0; j < kRmsHeld; ++j) s = fmaf(v[j], v[j], s);
+  for (int64_t i = kHeld + threadIdx.x; i < p.n; i += kRmsThreads) s = fmaf(p.a[i], p.a[i], s);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = s;
+  __syncthreads();
+  float t = red[threadIdx.x & 31];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  const float scale = rsqrtf(t / (float)p.n + p.eps);
+#pragma unroll
+  for (int j = 0; j < kRmsHeld; ++j) {
+    const int64_t i = threadIdx.x + (int64_t)j * kRmsThreads;
+    if (i >= p.n) continue;
+    p.y[i] = v[j] * scale * g[j];
+    count_elem<kCount>(p, i);
+  }
+  for (int64_t i = kHeld + threadIdx.x; i < p.n; i += kRmsThreads) {
+    p.y[i] = p.a[i] * scale * (p.b ? p.b[i] : 1.f);
+    count_elem<kCount>(p, i);
+  }
+}
+
+// Launch of a kernel that waits for its grid dependency itself.
+template <typename K, typename A>
+cudaError_t launch_dependent(K kernel, int grid, int threads, size_t smem, cudaStream_t st, const A& a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+cudaError_t launch_vec(const VecArgs& a, int sms, cudaStream_t st) {
+  if (a.n == 0) return cudaSuccess;
+  const int grid = (int)std::min<int64_t>((a.n + kThreads - 1) / kThreads, 4 * sms);
+  return a.counts ? launch_dependent(vec_kernel<true>, grid, kThreads, 0, st, a)
+                  : launch_dependent(vec_kernel<false>, grid, kThreads, 0, st, a);
 }
 
 bool vec_f32(const tp_tensor* t, int64_t n) {
@@ -662,8 +808,7 @@ cudaError_t launch_gemv(const GemvArgs& a, int grid, cudaStream_t st) {
   auto k = a.counts ? gemv_kernel<kEpi, kParts, kUnroll, true> : gemv_kernel<kEpi, kParts, kUnroll, false>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<grid, kThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(k, grid, kThreads, smem, st, a);
 }
 
 int gemv_grid(tp_ctx* ctx, int64_t k) {
@@ -692,15 +837,25 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 // past the edges. A SiLU-pair matrix ([2 n, k]: g rows, then u rows) is seen
 // as 3-D {k, n, 2} and boxed {256, 16, 2}, so one copy brings 16 g rows and
 // their 16 u partners (16 KB, g first).
-tp_status weight_map(CUtensorMap* map, const tp_tensor* w, bool pair) {
+// A plain matrix with units of fewer rows (rgroups < 8) is boxed {256, 4
+// rgroups}, or, when its rows are whole blocks of 256 columns, seen as 3-D
+// {256, rows, k / 256} and boxed {256, 4 rgroups, 8 / rgroups}: one copy per
+// stage.
+tp_status weight_map(CUtensorMap* map, const tp_tensor* w, bool pair, int rgroups, bool box3) {
   auto fn = encode_fn();
   if (!fn) return fail(TP_ERR_CUDA, "cuTensorMapEncodeTiled unavailable from the driver");
   const int64_t half = w->shape[0] / 2;
   cuuint64_t dims[3] = {(cuuint64_t)w->shape[1], (cuuint64_t)(pair ? half : w->shape[0]), 2};
   cuuint64_t strides[2] = {(cuuint64_t)(w->strides[0] * 2), (cuuint64_t)(half * w->strides[0] * 2)};
-  cuuint32_t box[3] = {(cuuint32_t)kSCols, (cuuint32_t)(pair ? kSPairRows : kSRows), 2};
+  cuuint32_t box[3] = {(cuuint32_t)kSCols, (cuuint32_t)(pair ? kSPairRows : 4 * rgroups), 2};
+  if (box3) {
+    dims[0] = kSCols;
+    dims[2] = (cuuint64_t)(w->shape[1] / kSCols);
+    strides[1] = kSCols * 2;
+    box[2] = (cuuint32_t)(kSConsumers / rgroups);
+  }
   cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, pair ? 3 : 2, w->ptr, dims, strides, box, estr,
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, pair || box3 ? 3 : 2, w->ptr, dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(TP_ERR_CUDA, "cuTensorMapEncodeTiled (weights) failed (" + std::to_string((int)r) + ")");
@@ -714,6 +869,45 @@ tp_status weight_map(CUtensorMap* map, const tp_tensor* w, bool pair) {
 constexpr int kSRingStages = 10;
 int stream_stages() { return kSRingStages; }
 
+// Ring stages that fit beside the whole of a k-element x (0: fewer than four,
+// too few to stream with).
+int whole_x_stages(int64_t k) {
+  const int64_t left = (int64_t)kSSmemMax - (int64_t)kSSmemFixed - (k + 3) / 4 * 16;
+  const int64_t n = left / kSStage;
+  return n < 4 ? 0 : (int)std::min<int64_t>(n, kSRingStages);
+}
+
+// Shape of the units of a single plain rows x k product with x whole in shared
+// memory: the one with the least work for the busiest CTA, counted in weight
+// elements plus what a unit costs beyond them (the cross-warp sum; the partly
+// filled last stage of a row), fitted to the times below. Units of 32 rows
+// leave a matrix of few rows unevenly spread (10240 rows: 320 units for 152
+// SMs), short ones pay their overhead often. Measured in graph replays, us
+// (10240 x 5120 / 5120 x 5120 / 5120 x 25600 / 51200 x 5120):
+//   32 rows 22.3 / 15.7 / 63.5 / 75.2   16 rows 19.6 / 12.8 / 48.2 / 75.7
+//    8 rows 20.3 / 12.5 / 42.0 / 83.5    4 rows 26.8 / 15.3 / 41.9 / 124
+//   per-lane gemv_kernel 21.3 / 14.0 / 62.5 / 78.3
+void unit_rows(StreamArgs* a, int64_t rows, int64_t k, int sms) {
+  a->rgroups = 8;
+  a->box3 = 0;
+  const bool blocks = k % kSCols == 0;
+  double best = 0;
+  for (int rg = 8; rg >= 1; rg /= 2) {
+    // a stage is 8 / rg column blocks: one 3-D box, or for rg = 4 two 2-D ones
+    const int64_t stage_cols = (int64_t)kSCols * (kSConsumers / rg);
+    if (rg < 8 && (k < stage_cols || (!blocks && rg < 4))) break;
+    const int64_t units = (rows + 4 * rg - 1) / (4 * rg);
+    const double per_unit = rg == 8 ? 0.0 : rg == 4 ? 4e3 : rg == 2 ? 7e3 : 14e3;
+    const double cost = (double)((units + sms - 1) / sms) * (4.0 * rg * (double)k + per_unit);
+    if (rg == 8 || cost < best) {
+      best = cost;
+      a->rgroups = rg;
+      a->box3 = rg < 8 && blocks ? 1 : 0;
+    }
+  }
+  a->units0 = a->units = (rows + 4 * a->rgroups - 1) / (4 * a->rgroups);
+}
+
 // The longest K slice (whole stages) of which two x buffers fit beside the ring.
 int64_t stream_max_slice_cols() {
   const size_t fixed = kSSmemFixed + (size_t)kSStage * stream_stages();
@@ -726,19 +920,30 @@ tp_status launch_stream(tp_ctx* ctx, StreamArgs a, const tp_tensor* w0, bool pai
                         cudaStream_t st) {
   // a problem without units has no map (and its descriptor is never touched)
   CUtensorMap m0 = {}, m1 = {};
-  tp_status s = a.units0 > 0 ? weight_map(&m0, w0, pair0) : TP_OK;
-  if (s == TP_OK && a.units > a.units0) s = weight_map(&m1, w1, pair1);
+  tp_status s = a.units0 > 0 ? weight_map(&m0, w0, pair0, a.rgroups, a.box3 != 0) : TP_OK;
+  if (s == TP_OK && a.units > a.units0) s = weight_map(&m1, w1, pair1, a.rgroups, false);
   if (s != TP_OK) return s;
   a.err = ctx->d_err;
   a.wait_ns = 2000000000ull;
   // x: one buffer, or with K slices as many (2..kSMaxXBufs) as fit
-  a.stages = stream_stages();
-  const size_t fixed = kSSmemFixed + (size_t)kSStage * a.stages;
   const size_t xbuf = (size_t)((a.slice_cols + 3) & ~int64_t(3)) * 4;
+  a.stages = a.slices > 1 ? stream_stages() : whole_x_stages(a.slice_cols);
+  const size_t fixed = kSSmemFixed + (size_t)kSStage * a.stages;
   a.xbufs = a.slices > 1 ? (int32_t)std::min<size_t>(kSMaxXBufs, (kSSmemMax - fixed) / xbuf) : 1;
   if (a.slices > 1 && a.xbufs < 2) return fail(TP_ERR_INVALID, "streaming matrix-vector kernel: K slice too long");
   const size_t smem = fixed + xbuf * (size_t)a.xbufs;
-  auto k = a.counts ? gemv_stream_kernel<true> : gemv_stream_kernel<false>;
+  // x by a bulk copy when it has more columns than the registers stage (never
+  // with norm: that takes at most kSMaxXCols)
+  auto pick = [&](auto count, auto bulk) {
+    constexpr bool kC = decltype(count)::value, kB = decltype(bulk)::value;
+    return a.rgroups == 8   ? gemv_stream_kernel<kC, 8, kB>
+           : a.rgroups == 4 ? gemv_stream_kernel<kC, 4, kB>
+           : a.rgroups == 2 ? gemv_stream_kernel<kC, 2, kB>
+                            : gemv_stream_kernel<kC, 1, kB>;
+  };
+  const bool bulk_x = a.slices == 1 && a.slice_cols > kSMaxXCols;
+  auto k = a.counts ? (bulk_x ? pick(std::true_type{}, std::true_type{}) : pick(std::true_type{}, std::false_type{}))
+                    : (bulk_x ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{}));
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return cuda_fail(e, "streaming matrix-vector kernel attributes");
   // the fewest CTAs (at most one per SM) that take as many units each as
@@ -771,6 +976,22 @@ tp_status launch_stream(tp_ctx* ctx, StreamArgs a, const tp_tensor* w0, bool pai
 // shared memory in bulk, read in 16-byte pieces).
 bool stream_ok(const tp_tensor* x) { return ((uintptr_t)x->ptr & 15) == 0; }
 
+// One plain product y = W x (or y += W x) with x whole in shared memory.
+StreamArgs whole_x_args(tp_ctx* ctx, const GemvArgs& g, int epi) {
+  StreamArgs a{};
+  a.k = g.k;
+  a.slices = 1;
+  a.slice_cols = g.k;
+  a.rows0 = a.rows1 = g.rows;
+  a.epi0 = a.epi1 = epi;
+  a.y0 = a.y1 = g.y;
+  a.x = g.x;
+  a.counts = g.counts;
+  a.owner = g.owner;
+  unit_rows(&a, g.rows, g.k, ctx->sm_count);
+  return a;
+}
+
 tp_status check_counts(const tp_exec* ex) {
   if ((ex->write_counts == nullptr) != (ex->write_owner == nullptr))
     return fail(TP_ERR_INVALID, "write_counts and write_owner must be given together");
@@ -797,12 +1018,11 @@ tp_status tp_rmsnorm(tp_ctx* ctx, tp_partition* n_out, const tp_tensor* h, const
   if (s != TP_OK) return s;
   VecArgs a{h ? static_cast<const float*>(h->ptr) : nullptr, gamma ? static_cast<const float*>(gamma->ptr) : nullptr,
             static_cast<float*>(n_out->t.ptr), d, eps, 0, ex->write_counts, ex->write_owner};
-  // the scale needs the whole vector: one CTA (d is a hidden size, tiny)
-  if (d > 0) {
-    if (a.counts) vec_kernel<true><<<1, kThreads, 0, o.stream>>>(a);
-    else vec_kernel<false><<<1, kThreads, 0, o.stream>>>(a);
-  }
-  return o.end(cudaGetLastError());
+  cudaError_t e = cudaSuccess;
+  if (d > 0)
+    e = a.counts ? launch_dependent(rmsnorm_kernel<true>, 1, kRmsThreads, 0, o.stream, a)
+                 : launch_dependent(rmsnorm_kernel<false>, 1, kRmsThreads, 0, o.stream, a);
+  return o.end(e);
 }
 
 tp_status tp_gemv(tp_ctx* ctx, tp_partition* y, const tp_tensor* w, const tp_tensor* x, const tp_exec* ex) {
@@ -825,7 +1045,25 @@ tp_status tp_gemv(tp_ctx* ctx, tp_partition* y, const tp_tensor* w, const tp_ten
   a.counts = ex->write_counts;
   a.owner = ex->write_owner;
   cudaError_t e = cudaSuccess;
-  if (rows > 0 && k > 0) e = launch_gemv<kPlain, 1, 4>(a, gemv_grid(ctx, k), o.stream);
+  if (rows > 0 && k > 0) {
+    // Streamed, but for matrices of a few boxes, where the stream's set-up
+    // shows (32 x 64: 2.8 us streamed, 2.0 per lane; 1000 x 1000: 3.2 and
+    // 3.6), for few rows that are not whole column blocks, whose units can't
+    // be cut below 16 rows (300 x 4104: 5.5 and 4.8), and for x that the bulk
+    // copies or shared memory cannot take.
+    StreamArgs sa = whole_x_args(ctx, a, kPlain);
+    const bool few = k % kSCols != 0 && sa.units < ctx->sm_count / 4;
+    if (stream_ok(x) && whole_x_stages(k) > 0 && rows * k >= (int64_t(1) << 16) && !few) {
+      o.check_err = true;  // its waits are bounded
+      tp_status ls = launch_stream(ctx, sa, w, false, w, false, o.stream);
+      if (ls != TP_OK) {
+        o.abort();
+        return ls;
+      }
+    } else {
+      e = launch_gemv<kPlain, 1, 4>(a, gemv_grid(ctx, k), o.stream);
+    }
+  }
   return o.end(e);
 }
 
@@ -840,12 +1078,7 @@ tp_status tp_silu_mul(tp_ctx* ctx, tp_partition* a_out, const tp_tensor* gu, con
   if (s != TP_OK) return s;
   VecArgs a{static_cast<const float*>(gu->ptr), nullptr, static_cast<float*>(a_out->t.ptr), n, 0.f, 1,
             ex->write_counts, ex->write_owner};
-  if (n > 0) {
-    const int grid = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, 4 * ctx->sm_count);
-    if (a.counts) vec_kernel<true><<<grid, kThreads, 0, o.stream>>>(a);
-    else vec_kernel<false><<<grid, kThreads, 0, o.stream>>>(a);
-  }
-  return o.end(cudaGetLastError());
+  return o.end(launch_vec(a, ctx->sm_count, o.stream));
 }
 
 tp_status tp_residual_add(tp_ctx* ctx, tp_partition* h, const tp_tensor* d, const tp_exec* ex) {
@@ -859,12 +1092,7 @@ tp_status tp_residual_add(tp_ctx* ctx, tp_partition* h, const tp_tensor* d, cons
   if (s != TP_OK) return s;
   VecArgs a{static_cast<const float*>(d->ptr), nullptr, static_cast<float*>(h->t.ptr), n, 0.f, 2,
             ex->write_counts, ex->write_owner};
-  if (n > 0) {
-    const int grid = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, 4 * ctx->sm_count);
-    if (a.counts) vec_kernel<true><<<grid, kThreads, 0, o.stream>>>(a);
-    else vec_kernel<false><<<grid, kThreads, 0, o.stream>>>(a);
-  }
-  return o.end(cudaGetLastError());
+  return o.end(launch_vec(a, ctx->sm_count, o.stream));
 }
 
 tp_status tp_decode_norm_qkv_gu(tp_ctx* ctx, tp_partition* qkv, tp_partition* a_out, const tp_tensor* h,
@@ -915,6 +1143,7 @@ tp_status tp_decode_norm_qkv_gu(tp_ctx* ctx, tp_partition* qkv, tp_partition* a_
       sa.rows1 = ni;
       sa.epi0 = kPlain;
       sa.epi1 = kSiluPair;
+      sa.rgroups = 8;
       sa.y0 = a.y;
       sa.y1 = a.y2;
       sa.x = a.x;
@@ -958,12 +1187,25 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
   a.counts = ex->write_counts;
   a.owner = ex->write_owner;
   cudaError_t e = cudaSuccess;
+  if (d > 0 && ni > 0 && stream_ok(a_in) && ni <= kSMaxXCols) {
+    // x whole in shared memory and units shaped to the matrix: one launch,
+    // each row summed in one place (4096 x 4096: 11.1 us in two K slices and
+    // a finish kernel, 8.4 so; 5120 x 5120: 15.6 and 12.5)
+    o.check_err = true;  // the streaming kernel's waits are bounded
+    StreamArgs sa = whole_x_args(ctx, a, kResidual);
+    sa.early_weights = (ex->flags & TP_EXEC_STATIC_WEIGHTS) ? 1 : 0;
+    tp_status ls = launch_stream(ctx, sa, w_down, false, w_down, false, o.stream);
+    if (ls != TP_OK) {
+      o.abort();
+      return ls;
+    }
+    return o.end(e);
+  }
   // Streamed in K slices as long as two x buffers of one fit beside the
   // ring, and more of them (down to 2048 columns) while the units (32-row
   // block x slice) number under four per SM; slices of equal whole stages.
   // Few long units beat many short ones (measured: a 5120 x 25600 product
-  // takes 43.4 us in 4 slices, 44.7 us in 10, 52 us in 15). One slice (x
-  // whole in shared memory, no finish kernel) when that is all it takes.
+  // takes 43.4 us in 4 slices, 44.7 us in 10, 52 us in 15).
   const int64_t row_blocks = (d + kSRows - 1) / kSRows;
   const int64_t max_cols = stream_max_slice_cols();
   int64_t slices64 = (ni + max_cols - 1) / max_cols;
@@ -987,6 +1229,7 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
     sa.rows1 = d;
     sa.epi0 = kResidual;
     sa.epi1 = kResidual;
+    sa.rgroups = 8;
     sa.y0 = a.y;
     sa.y1 = a.y;
     sa.partial = ctx->d_partial;

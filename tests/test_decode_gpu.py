@@ -314,3 +314,39 @@ def test_static_weights_flag_is_for_the_decode_products(ctx):
     href, qref = odecode.chain(h0.cpu(), [(a.cpu(), b.cpu(), c.cpu()) for a, b, c in layers])
     assert ogemm.rel_frobenius(h.cpu(), href) <= 1e-5
     ch.close()
+
+
+@pytest.mark.parametrize("rows,k,pitch", [
+    (16, 25600, 25600),     # units of 4 rows (8 column blocks a stage), x by bulk copy, the last stage half full
+    (5, 2048, 2048),        # ... one stage a row, a clipped unit
+    (5120, 5120, 5120),     # units of 8 rows
+    (10241, 2048, 2048),    # units of 16 rows, one 3-D box a stage, a clipped last unit
+    (6001, 1000, 1000),     # ... as two 2-D boxes (rows not of whole column blocks)
+    (77, 9001, 9008),       # x of an odd length, longer than the registers stage
+    (300, 33000, 33000),    # the longest x but for a few
+    (70, 1024, 1024), (63, 1024, 1024),  # just streamed, and just left to the per-lane kernel
+])
+def test_gemv_unit_shapes_within_summation_bound(ctx, rows, k, pitch):
+    """Every unit shape of the streamed product, and the residual form of it,
+    within the kernel's summation bound; each row is written once."""
+    w = _w(rows, pitch, rows + k)[:, :k]
+    x = _vec(k, 5)
+    y = torch.full((rows,), float("nan"), device="cuda")
+    p = tp.tp_partition_create(ctx, y, (rows,))
+    counts = torch.zeros(rows, dtype=torch.int32, device="cuda")
+    owner = torch.full((rows,), -1, dtype=torch.int32, device="cuda")
+    tp.tp_gemv(ctx, p, w, x, tp.make_exec(write_counts=counts, write_owner=owner))
+    assert opart.check_counts(counts.cpu().numpy())["ok"]
+    ref, bound = _f(w) @ _f(x), _gemv_bound(w, x)
+    assert np.all(np.abs(_f(y) - ref) <= bound)
+    counted = y.clone()
+    y.fill_(float("nan"))
+    tp.tp_gemv(ctx, p, w, x)
+    assert torch.equal(y, counted)
+    tp.tp_partition_destroy(p)
+    h = _vec(rows, 6)
+    h0 = _f(h)
+    p = tp.tp_partition_create(ctx, h, (rows,))
+    tp.tp_decode_down_residual(ctx, p, w, x)
+    assert np.all(np.abs(_f(h) - (h0 + ref)) <= bound + 2 * U32 * (np.abs(h0) + np.abs(ref) + bound))
+    tp.tp_partition_destroy(p)
