@@ -722,9 +722,8 @@ __global__ void __launch_bounds__(kThreads) vec_kernel(const __grid_constant__ V
 // y = a / sqrt(mean(a^2) + eps) * b (b null: 1) by one CTA: the scale needs
 // the whole vector, a hidden size of a few thousand. Latency-bound: up to
 // kRmsHeld elements per thread, and their gammas, are fetched in one round
-// trip and kept in registers (the rest is read twice). 5120 elements took
-// 4.4 us (ncu) with 256 threads reading the vector twice, one element at a
-// time.
+// trip and kept in registers (the rest is read twice): 5120 elements take 4.1
+// us (ncu, cold), 4.4 with 256 threads reading the vector twice.
 constexpr int kRmsThreads = 1024;
 constexpr int kRmsHeld = 8;
 

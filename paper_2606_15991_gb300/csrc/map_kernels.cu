@@ -261,9 +261,8 @@ __device__ __forceinline__ void divmod(int64_t n, int64_t d, int64_t* q, int64_t
 // flat sequence, so rows shorter than a warp leave no lane idle; a thread's
 // (row, slot) advances by a fixed step, without a division per access.
 // Bound by HBM: y = gelu_tanh(x) * w over 4001 x 9728 bf16 in 128 x 256 tiles
-// (234 MB) takes a synchronous call of 67 us, of which the kernel is about 42
-// (5.5 TB/s); one element per access with two 64-bit divisions each took 299
-// us (kernel 267). Two (bf16) or four (f32) slots in flight per thread, as in
+// (234 MB) takes 36.8 us (6.3 TB/s; a synchronous call of 67 us); one element
+// per access with two 64-bit divisions each took 267 (299 us). Two (bf16) or four (f32) slots in flight per thread, as in
 // map_vec_kernel; that kernel stays for rank-1 tiles of whole vectors, where
 // it needs no run arithmetic (32 registers against 55-100).
 template <int OP, typename T, bool COUNT>

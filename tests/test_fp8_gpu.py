@@ -196,3 +196,43 @@ def test_multi_block_stages_bit_identical(ctx, bm, bn, bk):
         out.append(c)
     assert torch.equal(out[0], out[1])
     assert np.array_equal(out[1].cpu().double().numpy(), lowp.round_bf16(ogemm.gemm(a, bt.t())))
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("n,tile,P,off", [
+    (1 << 20, 1 << 20, 0, 0),       # one program, several CTAs on its tile
+    (16 * 4096 + 16, 32768, 0, 0),  # a last round of one vector
+    (100_003, 40_000, 2, 0),        # ragged, two strided programs
+    (100_003, 50_000, 0, 1),        # off 16-byte boundaries: one element at a time
+    (5000, 17, 7, 0),               # tiles that are not whole vectors
+    (3_000_001, 8192, 0, 0),        # more tiles than the chip holds CTAs
+])
+def test_amax_and_codes_at_round_edges(ctx, dt, n, tile, P, off):
+    """The largest magnitude placed at each end and in the middle is found, and
+    every code is the oracle's, however a tile is shared among CTAs; each code
+    is written once, by its tile's program."""
+    buf = _x(n + off, 5, dt).cuda()
+    x = buf[off:]
+    ends = torch.tensor([0, n // 2, n - 1])
+    for i, at in enumerate(ends.tolist()):
+        x[at] = -(100.0 + i)
+        amax = torch.full((1,), 1e9, device="cuda")
+        tp.tp_amax(ctx, x, amax)
+        assert amax.item() == 100.0 + i
+    scale = torch.zeros(1, device="cuda")
+    qb = torch.zeros(n + 16 + off, dtype=torch.uint8, device="cuda")
+    q = qb[off:off + n]
+    p = tp.tp_partition_create(ctx, q, (tile,))
+    if P:
+        tp.tp_partition_map(p, tp.MAP_STRIDED, P)
+    counts = torch.zeros(n, dtype=torch.int32, device="cuda")
+    owner = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+    tp.tp_quantize_fp8(ctx, p, x, amax, scale, tp.make_exec(write_counts=counts, write_owner=owner))
+    first = q.clone()
+    q.zero_()
+    tp.tp_quantize_fp8(ctx, p, x, amax, scale)
+    assert torch.equal(q, first) and not qb[off + n:].any() and not qb[:off].any()
+    assert np.array_equal(q.cpu().numpy(), ogemm.fp8_quantize(x.cpu(), np.float32(scale.item())))
+    assert opart.check_counts(counts.cpu().numpy())["ok"]
+    assert np.array_equal(owner.cpu().numpy(), opart.owner_map((n,), (tile,), P or None, "strided" if P else "identity"))
+    tp.tp_partition_destroy(p)
