@@ -622,7 +622,7 @@ tp_status tp_propose(tp_ctx* ctx, tp_mlp* mlp, int64_t M, int64_t N, int64_t K, 
  * mbarrier with the same bounded wait those kernels' roles use. With
  * arrive != 0 the barrier is signalled first and the wait completes (TP_OK).
  * With arrive == 0 nothing ever signals it: the wait gives up after
- * `limit_ns` of GPU wall time (1e3..2e9), records a timeout in the context's
+ * `limit_ns` of GPU wall time (1e3..2e9), records a timeout in the operation's
  * error word and the kernel returns, so the operation reports TP_ERR_TIMEOUT
  * where it reports device errors (SYNC: on return; ASYNC: from
  * tp_event_query / tp_event_wait; graph: from the replay) and the context

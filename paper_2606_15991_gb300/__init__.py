@@ -9,6 +9,7 @@ raise.
 from __future__ import annotations
 
 import ctypes
+import struct
 
 import torch
 
@@ -52,15 +53,27 @@ def _i64(vals):
     return arr
 
 
+# tp_tensor as bytes, by rank: ptr, dtype, rank, shape[8], strides[8]
+_TENSOR_PACK = [struct.Struct("<Qii" + f"{r}q{64 - 8 * r}x" * 2).pack for r in range(9)]
+assert struct.calcsize("<Qii8q8q") == ctypes.sizeof(tp_tensor)
+
+
 def tensor_desc(t) -> tp_tensor:
-    """tp_tensor view of a torch tensor (or a tp_tensor passed through)."""
+    """tp_tensor view of a torch tensor (or a tp_tensor passed through).
+
+    Packed here rather than by tp_tensor_init: a torch tensor's extents and
+    dtype need none of its checks but the rank's, and a call to it, with its two
+    ctypes arrays, cost more than everything else a small operation marshals."""
     if isinstance(t, tp_tensor):
         return t
-    if t.dtype not in _DTYPES:
+    code = _DTYPES.get(t.dtype)
+    if code is None:
         raise TypeError(f"unsupported dtype {t.dtype}")
+    r = t.dim()
+    if r <= 8:
+        return tp_tensor.from_buffer_copy(_TENSOR_PACK[r](t.data_ptr(), code, r, *t.shape, *t.stride()))
     d = tp_tensor()
-    call("tp_tensor_init", ctypes.byref(d), ctypes.c_void_p(t.data_ptr()), _DTYPES[t.dtype], t.dim(),
-         _i64(t.shape), _i64(t.stride()))
+    call("tp_tensor_init", ctypes.byref(d), ctypes.c_void_p(t.data_ptr()), code, r, _i64(t.shape), _i64(t.stride()))
     return d
 
 
@@ -176,8 +189,14 @@ def tp_event_destroy(ev: Event) -> None:
         ev.handle = ctypes.c_void_p()
 
 
+# the current stream's handle without the Stream object around it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_handle(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -226,15 +245,17 @@ def make_exec(mode: int = SYNC, stream=None, event: Event | None = None, write_c
     GEMM's failure-path test hook (TP_EXEC_INJECT_TIMEOUT). static_weights:
     the decode products may start reading their weights before the work
     queued ahead of them on the stream finishes (TP_EXEC_STATIC_WEIGHTS)."""
-    ex = tp_exec()
-    ex.mode = mode
-    ex.flags = ((_lib.EXEC_CHECKED if checked else 0) | (_lib.EXEC_INJECT_TIMEOUT if inject_timeout else 0) |
-                (_lib.EXEC_STATIC_WEIGHTS if static_weights else 0))
-    ex.stream = _stream_handle(stream)
-    ex.event = event.handle.value if event is not None else None
-    ex.write_counts = write_counts.data_ptr() if write_counts is not None else None
-    ex.write_owner = write_owner.data_ptr() if write_owner is not None else None
-    return ex
+    flags = ((_lib.EXEC_CHECKED if checked else 0) | (_lib.EXEC_INJECT_TIMEOUT if inject_timeout else 0) |
+             (_lib.EXEC_STATIC_WEIGHTS if static_weights else 0))
+    return tp_exec.from_buffer_copy(_EXEC_PACK(
+        mode, flags, _stream_handle(stream), event.handle.value or 0 if event is not None else 0,
+        write_counts.data_ptr() if write_counts is not None else 0,
+        write_owner.data_ptr() if write_owner is not None else 0))
+
+
+# tp_exec as bytes: mode, flags, stream, event, write_counts, write_owner
+_EXEC_PACK = struct.Struct("<iiQQQQ").pack
+assert struct.calcsize("<iiQQQQ") == ctypes.sizeof(tp_exec)
 
 
 def gemm_config(bm=0, bn=0, bk=0, stages=0, group_m=0, num_programs=0, swap_ab=0, split_k=0, cut_limit=0):

@@ -168,7 +168,7 @@ def lib():
 
 def call(name: str, *args) -> None:
     """Call a tp_* entry point and raise TPError on a non-OK status."""
-    L = lib()
+    L = _lib if _lib is not None else lib()
     st = getattr(L, name)(*args)
     if st != OK:
         raise TPError(st, L.tp_last_error_detail().decode(), name)

@@ -916,13 +916,13 @@ int64_t stream_max_slice_cols() {
 // The streaming kernel on w0 (problem 0) and w1 (problem 1, may equal w0):
 // one persistent CTA per SM, or one per unit when there are fewer units.
 tp_status launch_stream(tp_ctx* ctx, StreamArgs a, const tp_tensor* w0, bool pair0, const tp_tensor* w1, bool pair1,
-                        cudaStream_t st) {
+                        cudaStream_t st, int* err) {
   // a problem without units has no map (and its descriptor is never touched)
   CUtensorMap m0 = {}, m1 = {};
   tp_status s = a.units0 > 0 ? weight_map(&m0, w0, pair0, a.rgroups, a.box3 != 0) : TP_OK;
   if (s == TP_OK && a.units > a.units0) s = weight_map(&m1, w1, pair1, a.rgroups, false);
   if (s != TP_OK) return s;
-  a.err = ctx->d_err;
+  a.err = err;
   a.wait_ns = 2000000000ull;
   // x: one buffer, or with K slices as many (2..kSMaxXBufs) as fit
   const size_t xbuf = (size_t)((a.slice_cols + 3) & ~int64_t(3)) * 4;
@@ -1054,7 +1054,7 @@ tp_status tp_gemv(tp_ctx* ctx, tp_partition* y, const tp_tensor* w, const tp_ten
     const bool few = k % kSCols != 0 && sa.units < ctx->sm_count / 4;
     if (stream_ok(x) && whole_x_stages(k) > 0 && rows * k >= (int64_t(1) << 16) && !few) {
       o.check_err = true;  // its waits are bounded
-      tp_status ls = launch_stream(ctx, sa, w, false, w, false, o.stream);
+      tp_status ls = launch_stream(ctx, sa, w, false, w, false, o.stream, o.err);
       if (ls != TP_OK) {
         o.abort();
         return ls;
@@ -1152,7 +1152,7 @@ tp_status tp_decode_norm_qkv_gu(tp_ctx* ctx, tp_partition* qkv, tp_partition* a_
       sa.counts = a.counts;
       sa.owner = a.owner;
       sa.early_weights = (ex->flags & TP_EXEC_STATIC_WEIGHTS) ? 1 : 0;
-      tp_status ls = launch_stream(ctx, sa, w_qkv, false, w_gu, true, o.stream);
+      tp_status ls = launch_stream(ctx, sa, w_qkv, false, w_gu, true, o.stream, o.err);
       if (ls != TP_OK) {
         o.abort();
         return ls;
@@ -1193,7 +1193,7 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
     o.check_err = true;  // the streaming kernel's waits are bounded
     StreamArgs sa = whole_x_args(ctx, a, kResidual);
     sa.early_weights = (ex->flags & TP_EXEC_STATIC_WEIGHTS) ? 1 : 0;
-    tp_status ls = launch_stream(ctx, sa, w_down, false, w_down, false, o.stream);
+    tp_status ls = launch_stream(ctx, sa, w_down, false, w_down, false, o.stream, o.err);
     if (ls != TP_OK) {
       o.abort();
       return ls;
@@ -1236,7 +1236,7 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
     sa.early_weights = (ex->flags & TP_EXEC_STATIC_WEIGHTS) ? 1 : 0;
     sa.counts = sa.slices > 1 ? nullptr : a.counts;
     sa.owner = sa.slices > 1 ? nullptr : a.owner;
-    tp_status ls = launch_stream(ctx, sa, w_down, false, w_down, false, o.stream);
+    tp_status ls = launch_stream(ctx, sa, w_down, false, w_down, false, o.stream, o.err);
     if (ls != TP_OK) {
       o.abort();
       return ls;

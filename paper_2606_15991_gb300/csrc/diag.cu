@@ -1,6 +1,6 @@
 // Diagnostic of the failure path shared by the pipelined kernels: a role
 // that waits on an mbarrier gives up after a wall-time limit, records
-// kDevTimeout in the context's error word and returns, so the launch ends and
+// kDevTimeout in the operation's error word and returns, so the launch ends and
 // the host reports TP_ERR_TIMEOUT instead of the GPU hanging.
 #include "sm100_ptx.cuh"
 #include "tp_internal.h"
@@ -37,6 +37,6 @@ extern "C" tp_status tp_diag_bounded_wait(tp_ctx* ctx, int64_t limit_ns, int32_t
   tp_status s = o.begin(ctx, ex, {}, {});
   if (s != TP_OK) return s;
   o.check_err = true;
-  bounded_wait_kernel<<<1, 32, 0, o.stream>>>(ctx->d_err, (uint64_t)limit_ns, arrive != 0);
+  bounded_wait_kernel<<<1, 32, 0, o.stream>>>(o.err, (uint64_t)limit_ns, arrive != 0);
   return o.end(cudaGetLastError());
 }

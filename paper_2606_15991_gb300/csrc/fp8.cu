@@ -300,7 +300,7 @@ tp_status tp_gemm_fp8(tp_ctx* ctx, tp_partition* c, const tp_tensor* qa, const t
   tp_status s = o.begin(ctx, ex, {c}, {qa, qb});
   if (s != TP_OK) return s;
   o.check_err = true;
-  s = launch_gemm_tc_impl(ctx, c, qa, qb, cfg, ex, o.stream, 1, scale_a, scale_b);
+  s = launch_gemm_tc_impl(ctx, c, qa, qb, cfg, ex, o.stream, 1, scale_a, scale_b, o.err);
   if (s != TP_OK) {
     o.abort();
     return s;

@@ -621,7 +621,7 @@ bool f32_map(CUtensorMap* map, const float* ptr, int64_t rows, int64_t cols, int
 
 tp_status launch_gemm_simt(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_tensor* b,
                            const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream,
-                           unsigned* queue) {
+                           unsigned* queue, int* err) {
   if (c->tile[0] != BM || c->tile[1] != BN)
     return fail(TP_ERR_UNSUPPORTED, "the FP32 GEMM uses 64 x 64 output tiles");
   if ((ex->write_counts == nullptr) != (ex->write_owner == nullptr))
@@ -681,7 +681,7 @@ tp_status launch_gemm_simt(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, con
       t.nchunks = (int32_t)((p.K + kFChunk - 1) / kFChunk);
       t.counts = p.counts;
       t.owner = p.owner;
-      t.err = ctx->d_err;
+      t.err = err;
       t.wait_ns = 2000000000ull;
       e = count ? launch_f32_tma<true>(ma, mb, t, grid, stream) : launch_f32_tma<false>(ma, mb, t, grid, stream);
       if (e != cudaSuccess) return cuda_fail(e, "FP32 GEMM launch");

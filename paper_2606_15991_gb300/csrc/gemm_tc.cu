@@ -72,7 +72,7 @@ struct TcArgs {
   __nv_bfloat16* c;
   const float* scale_a; // optional (FP8): C = acc * 1 / (*scale_a * *scale_b)
   const float* scale_b;
-  int* err;             // context error word
+  int* err;             // the operation's error word
   uint32_t* counts;     // write-count instrumentation (optional)
   int32_t* owner;
   uint32_t* claims;     // checked launch: tile-claim bitmap (kChecked)
@@ -894,7 +894,7 @@ tp_status make_map_c(CUtensorMap* map, void* ptr, int64_t M, int64_t N, int cols
 // Shared by the BF16 and FP8 entry points. esize = 2 (bf16) or 1 (fp8).
 tp_status launch_gemm_tc_impl(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_tensor* b,
                               const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream, int esize,
-                              const float* scale_a, const float* scale_b) {
+                              const float* scale_a, const float* scale_b, int* err) {
   const int64_t M = a->shape[0], K = a->shape[1], N = b->shape[1];
   if ((ex->write_counts == nullptr) != (ex->write_owner == nullptr))
     return fail(TP_ERR_INVALID, "write_counts and write_owner must be given together");
@@ -986,7 +986,7 @@ tp_status launch_gemm_tc_impl(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, 
   p.c = static_cast<__nv_bfloat16*>(c->t.ptr);
   p.scale_a = scale_a;
   p.scale_b = scale_b;
-  p.err = ctx->d_err;
+  p.err = err;
   p.counts = ex->write_counts;
   p.owner = ex->write_owner;
   int cols = 32;
@@ -1098,9 +1098,8 @@ tp_status gemm_tc_resident(tp_ctx* ctx, const tp_gemm_config* cfg, int32_t* prog
 }
 
 tp_status launch_gemm_tc(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_tensor* b,
-                         const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream, unsigned* queue) {
-  (void)queue;
-  return launch_gemm_tc_impl(ctx, c, a, b, cfg, ex, stream, 2, nullptr, nullptr);
+                         const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream, int* err) {
+  return launch_gemm_tc_impl(ctx, c, a, b, cfg, ex, stream, 2, nullptr, nullptr, err);
 }
 
 }  // namespace tp

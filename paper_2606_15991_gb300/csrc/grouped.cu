@@ -785,7 +785,7 @@ tp_status tp_grouped_gemm(tp_ctx* ctx, tp_grouped_plan* plan, int32_t num_progra
   a.n = plan->n;
   a.total = plan->total_tiles;
   a.queue = q;
-  a.err = ctx->d_err;
+  a.err = o.err;
   a.counts = ex->write_counts;
   a.owner = ex->write_owner;
   const bool pair = plan->pair;

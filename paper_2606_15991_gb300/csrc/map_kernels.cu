@@ -32,7 +32,7 @@ struct MapArgs {
   int32_t mis;           // elements from each base pointer down to a 16-byte boundary (segment path)
   uint32_t* claims;      // checked launch: tile-claim bitmap (null = release)
   unsigned* claim_done;  // checked launch: finished-CTA counter
-  int* err;              // context error word
+  int* err;              // the operation's error word
 };
 
 // 2^a by the hardware base-2 exponential (flush-to-zero).
@@ -451,7 +451,7 @@ cudaError_t launch_op(int op, MapArgs a, bool rank1, bool count, int64_t grid, c
 }  // namespace
 
 tp_status launch_map(tp_ctx* ctx, tp_partition* out, int op, float alpha, const tp_tensor* x,
-                     const tp_tensor* y, const tp_exec* ex, cudaStream_t stream, unsigned* queue) {
+                     const tp_tensor* y, const tp_exec* ex, cudaStream_t stream, unsigned* queue, int* err) {
   MapArgs a{};
   a.out = out->t.ptr;
   a.x = x->ptr;
@@ -469,7 +469,7 @@ tp_status launch_map(tp_ctx* ctx, tp_partition* out, int op, float alpha, const 
   if (ex->flags & TP_EXEC_CHECKED) {
     tp_status cs = claims_for(ctx, out->num_tiles, &a.claims, &a.claim_done);
     if (cs != TP_OK) return cs;
-    a.err = ctx->d_err;
+    a.err = err;
   }
   const int pad = 3 - out->rank;
   for (int i = 0; i < 3; ++i) {

@@ -151,13 +151,13 @@ tp_status tp_permute_heads_unchecked(tp_ctx* ctx, void* dst, const void* src, in
   int32_t* wo = ex->write_owner;
   if (wc && checked)
     permute_raw_kernel<true, true><<<grid, kThreads, 0, o.stream>>>(d, sp, B, H, M, D, BM, swap_bug, wc, wo, claims,
-                                                                     done, ctx->d_err);
+                                                                     done, o.err);
   else if (wc)
     permute_raw_kernel<true, false><<<grid, kThreads, 0, o.stream>>>(d, sp, B, H, M, D, BM, swap_bug, wc, wo, nullptr,
                                                                       nullptr, nullptr);
   else if (checked)
     permute_raw_kernel<false, true><<<grid, kThreads, 0, o.stream>>>(d, sp, B, H, M, D, BM, swap_bug, nullptr,
-                                                                      nullptr, claims, done, ctx->d_err);
+                                                                      nullptr, claims, done, o.err);
   else
     permute_raw_kernel<false, false><<<grid, kThreads, 0, o.stream>>>(d, sp, B, H, M, D, BM, swap_bug, nullptr,
                                                                        nullptr, nullptr, nullptr, nullptr);

@@ -2,7 +2,7 @@
 // a tile it claims the tile's bit in the context's claim bitmap. A bit that
 // is already set means a second program is about to write the same
 // sub-tensor (a data race in the sense of Appendix A); the claim fails and
-// the context's error word records kDevRace. Off-map tiles record kDevRace as
+// the operation's error word records kDevRace. Off-map tiles record kDevRace as
 // well. The bitmap starts a launch all clear: every checked launch counts its
 // claimants (CTAs, or the GEMM's epilogue warps) as they make their last
 // claim, and the last one clears the bits the launch could have set, so the

@@ -16,7 +16,7 @@
 
 namespace tp {
 
-// Device-side error codes written to the context's error word.
+// Device-side error codes written to an error word (tp_ctx::words).
 enum DeviceError : int {
   kDevOk = 0,
   kDevTimeout = 1,     // a bounded wait ran out of iterations
@@ -62,15 +62,21 @@ struct tp_ctx {
   std::unordered_map<tp::HoldKey, int64_t, tp::HoldKeyHash> busy;
   tp_graph* capturing = nullptr;    // graph being captured, if any
   // Device workspace, allocated once at creation.
-  int* d_err = nullptr;             // device error word (tp::DeviceError)
+  // Error words (tp::DeviceError) in pinned host memory that kernels write to
+  // directly, and only when something failed: an operation that went well
+  // moves nothing to report so. words[0] is the context's (launches that no
+  // operation reports for), the next kSyncWords serve SYNC operations in turn,
+  // the rest are lent to events and graphs.
+  int* words = nullptr;
+  std::atomic<uint32_t> sync_word{0};
+  std::vector<int> free_words;      // indices to lend, under mu
+  static constexpr int kSyncWords = 256;
+  static constexpr int kWords = 4096;
   unsigned* d_queue = nullptr;      // tile-queue counters (kQueueSlots)
   float* d_scratch = nullptr;       // small float scratch (kScratchFloats)
   float* d_partial = nullptr;       // matrix-vector partial sums (kPartialFloats)
   uint32_t* d_claims = nullptr;     // tile-claim bitmap of checked launches (kClaimBits), all clear
   unsigned* d_claim_done = nullptr; // CTAs of the running checked launch that finished
-  int* h_err_slots = nullptr;       // pinned host copies of the error word (kErrSlots)
-  std::atomic<uint32_t> err_slot{0};
-  static constexpr int kErrSlots = 256;
   std::atomic<uint32_t> queue_slot{0};
   static constexpr int kQueueSlots = 256;
   static constexpr int kScratchFloats = 4096;
@@ -98,7 +104,8 @@ struct tp_event {
   bool recorded = false;
   bool check_err = false;
   cudaStream_t stream = nullptr;  // stream of the last record
-  int* h_err = nullptr;           // pinned copy of the error word, staged behind the work
+  int* err = nullptr;             // error word of the operations recorded into it
+  std::vector<int*> graph_errs;   // error words of the graphs replayed into it
   std::vector<tp::Hold> held;   // holds released when the event completes (appended per op)
 };
 
@@ -109,6 +116,7 @@ struct tp_graph {
   cudaGraphExec_t exec = nullptr;
   bool ended = false;
   bool check_err = false;
+  int* err = nullptr;                // error word of the recorded operations
   std::vector<tp_partition*> parts;  // partitions written by recorded nodes
 };
 
@@ -154,7 +162,8 @@ struct Op {
   const tp_exec* ex = nullptr;
   cudaStream_t stream = nullptr;
   std::vector<tp_partition*> outs;
-  bool check_err = false;   // kernel may write the device error word
+  bool check_err = false;   // kernel may write the error word
+  int* err = nullptr;       // error word for this operation's kernels (set by begin)
   bool marked = false;
   bool allow_checked = false;  // the op implements TP_EXEC_CHECKED (set before begin)
   bool allow_inject = false;   // the op implements TP_EXEC_INJECT_TIMEOUT (set before begin)
@@ -174,13 +183,12 @@ struct Op {
   bool capturing() const { return ex->mode == TP_CAPTURE; }
 };
 
-tp_status read_device_error(tp_ctx* ctx);
-// Enqueue a copy of the device error word into pinned `slot` on `stream`
-// (behind the work already queued there).
-cudaError_t stage_device_error(tp_ctx* ctx, cudaStream_t stream, int* slot);
-// Status for a staged error word `h` (read after the stream or event
-// completed); clears the device word when it is set.
-tp_status take_device_error(tp_ctx* ctx, int h);
+// Status of the error in `word` (or, when it holds none, in the context's
+// word), read after the work that may write it has completed; clears it.
+tp_status take_error(tp_ctx* ctx, int* word);
+// An error word to lend (ctx->mu held); the context's own when none is left.
+int* lend_word_locked(tp_ctx* ctx);
+void return_word_locked(tp_ctx* ctx, int* word);
 // An ASYNC launch may record `ev` on `stream`: OK when the event tracks no
 // unfinished work on another stream (completed work is released first).
 tp_status event_claim(tp_event* ev, cudaStream_t stream);
@@ -193,13 +201,12 @@ tp_status queue_counter(tp_ctx* ctx, cudaStream_t stream, unsigned** out);
 // Kernel launchers (defined in the kernel translation units).
 enum MapOp : int { kMapAxpy = 0, kMapGeluMul = 1, kMapScale = 2, kMapAddAccum = 3 };
 tp_status launch_map(tp_ctx* ctx, tp_partition* out, int op, float alpha, const tp_tensor* x,
-                     const tp_tensor* y, const tp_exec* ex, cudaStream_t stream, unsigned* queue);
+                     const tp_tensor* y, const tp_exec* ex, cudaStream_t stream, unsigned* queue, int* err);
 tp_status launch_gemm_simt(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_tensor* b,
                            const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream,
-                           unsigned* queue);
+                           unsigned* queue, int* err);
 tp_status launch_gemm_tc(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_tensor* b,
-                         const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream,
-                         unsigned* queue);
+                         const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream, int* err);
 
 // Programs of the tensor-core GEMM (CTA pairs for 256-row tiles, CTAs
 // otherwise) that can be resident at once for `cfg`.
@@ -211,6 +218,6 @@ bool autotune_config_runs(const tp_ctx* ctx, int64_t M, int64_t N, int64_t K, in
 
 tp_status launch_gemm_tc_impl(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_tensor* b,
                               const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream, int esize,
-                              const float* scale_a, const float* scale_b);
+                              const float* scale_a, const float* scale_b, int* err);
 
 }  // namespace tp

@@ -135,22 +135,14 @@ static tp_status error_status(int h) {
   return fail(TP_ERR_INVALID, "device bounds check failed");
 }
 
-tp_status read_device_error(tp_ctx* ctx) {
-  int h = 0;
-  cudaError_t e = cudaMemcpy(&h, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "reading device error word");
-  return take_device_error(ctx, h);
-}
+// The word's error, cleared; kernels write it from the device, so the read is
+// an atomic exchange.
+static int take_word(int* word) { return __atomic_exchange_n(word, 0, __ATOMIC_ACQ_REL); }
 
-cudaError_t stage_device_error(tp_ctx* ctx, cudaStream_t stream, int* slot) {
-  *slot = 0;
-  return cudaMemcpyAsync(slot, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, stream);
-}
-
-tp_status take_device_error(tp_ctx* ctx, int h) {
+tp_status take_error(tp_ctx* ctx, int* word) {
+  int h = take_word(word);
+  if (h == kDevOk && word != ctx->words) h = take_word(ctx->words);
   if (h == kDevOk) return TP_OK;
-  int zero = 0;
-  cudaMemcpy(ctx->d_err, &zero, sizeof(int), cudaMemcpyHostToDevice);
   // a checked launch that gave up part-way may have left claim state
   // behind; the next launch must start from zero
   if (h == kDevTimeout) {
@@ -158,6 +150,18 @@ tp_status take_device_error(tp_ctx* ctx, int h) {
     cudaMemset(ctx->d_claims, 0, (size_t)tp_ctx::kClaimBits / 8);
   }
   return error_status(h);
+}
+
+int* lend_word_locked(tp_ctx* ctx) {
+  if (ctx->free_words.empty()) return ctx->words;
+  int* w = ctx->words + ctx->free_words.back();
+  ctx->free_words.pop_back();
+  *w = kDevOk;
+  return w;
+}
+
+void return_word_locked(tp_ctx* ctx, int* word) {
+  if (word != ctx->words) ctx->free_words.push_back((int)(word - ctx->words));
 }
 
 tp_status claims_for(tp_ctx* ctx, int64_t bits, uint32_t** claims, unsigned** done) {
@@ -282,6 +286,12 @@ tp_status Op::begin_impl(tp_ctx* c, const tp_exec* e, const std::vector<tp_parti
       if (held.hit(r.first, r.second))
         return fail(TP_ERR_BUSY, "an input reads bytes of a partition with work in flight on another stream");
   }
+  if (ex->mode == TP_SYNC) {
+    err = ctx->words + 1 + ctx->sync_word.fetch_add(1) % tp_ctx::kSyncWords;
+    *err = kDevOk;
+  } else {
+    err = ex->mode == TP_ASYNC ? ex->event->err : ctx->capturing->err;
+  }
   if (ex->mode == TP_CAPTURE) {
     for (auto* p : outs) {
       auto& v = ctx->capturing->parts;
@@ -316,21 +326,13 @@ tp_status Op::end_impl(cudaError_t launch_err) {
     return TP_OK;
   }
   if (ex->mode == TP_SYNC) {
-    int* slot = nullptr;
-    cudaError_t e = cudaSuccess;
-    if (check_err) {
-      slot = ctx->h_err_slots + ctx->err_slot.fetch_add(1) % tp_ctx::kErrSlots;
-      e = stage_device_error(ctx, stream, slot);
-    }
-    cudaError_t e2 = cudaStreamSynchronize(stream);
+    const cudaError_t e = cudaStreamSynchronize(stream);
     release(ctx, outs, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "staging the device error word");
-    if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamSynchronize");
-    return check_err ? take_device_error(ctx, *slot) : TP_OK;
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    return check_err ? take_error(ctx, err) : TP_OK;
   }
   tp_event* ev = ex->event;
-  cudaError_t e = check_err ? stage_device_error(ctx, stream, ev->h_err) : cudaSuccess;
-  if (e == cudaSuccess) e = cudaEventRecord(ev->ev, stream);
+  const cudaError_t e = cudaEventRecord(ev->ev, stream);
   if (e != cudaSuccess) {
     release(ctx, outs, stream);
     return cuda_fail(e, "cudaEventRecord");
@@ -397,7 +399,7 @@ tp_status tp_ctx_create(int32_t device, tp_ctx** out) {
     delete c;
     return fail(TP_ERR_UNSUPPORTED, "this library is built for sm_103a (Blackwell) only");
   }
-  e = cudaMalloc(&c->d_err, sizeof(int));
+  e = cudaMallocHost(&c->words, sizeof(int) * tp_ctx::kWords);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_queue, sizeof(unsigned) * tp_ctx::kQueueSlots);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_scratch, sizeof(float) * tp_ctx::kScratchFloats);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_partial, sizeof(float) * tp_ctx::kPartialFloats);
@@ -405,20 +407,19 @@ tp_status tp_ctx_create(int32_t device, tp_ctx** out) {
   if (e == cudaSuccess) e = cudaMalloc(&c->d_claim_done, 256);
   if (e == cudaSuccess) e = cudaMemset(c->d_claims, 0, (size_t)tp_ctx::kClaimBits / 8);
   if (e == cudaSuccess) e = cudaMemset(c->d_claim_done, 0, 256);
-  if (e == cudaSuccess) e = cudaMallocHost(&c->h_err_slots, sizeof(int) * tp_ctx::kErrSlots);
-  if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(c->d_queue, 0, sizeof(unsigned) * tp_ctx::kQueueSlots);
   if (e != cudaSuccess) {
-    cudaFree(c->d_err);
     cudaFree(c->d_queue);
     cudaFree(c->d_scratch);
     cudaFree(c->d_partial);
     cudaFree(c->d_claims);
     cudaFree(c->d_claim_done);
-    cudaFreeHost(c->h_err_slots);
+    cudaFreeHost(c->words);
     delete c;
     return cuda_fail(e, "allocating context workspace");
   }
+  std::fill(c->words, c->words + tp_ctx::kWords, (int)kDevOk);
+  for (int i = tp_ctx::kWords - 1; i > tp_ctx::kSyncWords; --i) c->free_words.push_back(i);
   *out = c;
   return TP_OK;
 }
@@ -430,13 +431,14 @@ tp_status tp_ctx_destroy(tp_ctx* ctx) {
     if (!ctx->busy.empty()) return fail(TP_ERR_BUSY, "context still has work in flight");
     if (ctx->capturing) return fail(TP_ERR_BUSY, "context is capturing a graph");
   }
-  cudaFree(ctx->d_err);
+  // the frees wait for the device, so no kernel is left that could still write
+  // an error word
   cudaFree(ctx->d_queue);
   cudaFree(ctx->d_scratch);
   cudaFree(ctx->d_partial);
   cudaFree(ctx->d_claims);
   cudaFree(ctx->d_claim_done);
-  cudaFreeHost(ctx->h_err_slots);
+  cudaFreeHost(ctx->words);
   delete ctx;
   return TP_OK;
 }
@@ -570,29 +572,32 @@ tp_status tp_event_create(tp_ctx* ctx, tp_event** out) {
     delete ev;
     return cuda_fail(e, "cudaEventCreate");
   }
-  e = cudaMallocHost(&ev->h_err, sizeof(int));
-  if (e != cudaSuccess) {
-    cudaEventDestroy(ev->ev);
-    delete ev;
-    return cuda_fail(e, "cudaMallocHost");
-  }
-  *ev->h_err = 0;
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  ev->err = lend_word_locked(ctx);
   *out = ev;
   return TP_OK;
 }
 
 static tp_status event_complete(tp_event* ev) {
   std::vector<Hold> held;
+  std::vector<int*> errs;
   bool chk;
   {
     std::lock_guard<std::mutex> lk(ev->ctx->mu);
     held.swap(ev->held);
+    errs.swap(ev->graph_errs);
     chk = ev->check_err;
     ev->check_err = false;
     ev->recorded = false;
     for (auto& h : held) release_locked(ev->ctx, h.p, h.stream, h.count);
   }
-  return chk ? take_device_error(ev->ctx, *ev->h_err) : TP_OK;
+  if (!chk) return TP_OK;
+  tp_status s = take_error(ev->ctx, ev->err);
+  for (int* w : errs) {
+    const tp_status gs = take_error(ev->ctx, w);
+    if (s == TP_OK) s = gs;
+  }
+  return s;
 }
 
 }  // extern "C"
@@ -642,7 +647,10 @@ tp_status tp_event_destroy(tp_event* ev) {
     event_complete(ev);
   }
   cudaEventDestroy(ev->ev);
-  cudaFreeHost(ev->h_err);
+  {
+    std::lock_guard<std::mutex> lk(ev->ctx->mu);
+    return_word_locked(ev->ctx, ev->err);
+  }
   delete ev;
   return TP_OK;
 }
@@ -661,6 +669,7 @@ tp_status tp_graph_begin(tp_ctx* ctx, void* stream, tp_graph** out) {
     delete g;
     return cuda_fail(e, "cudaStreamBeginCapture");
   }
+  g->err = lend_word_locked(ctx);
   ctx->capturing = g;
   *out = g;
   return TP_OK;
@@ -713,19 +722,12 @@ tp_status tp_graph_replay(tp_graph* g, const tp_exec* ex) {
     return cuda_fail(e, "cudaGraphLaunch");
   }
   if (ex->mode == TP_SYNC) {
-    int* slot = nullptr;
-    if (g->check_err) {
-      slot = ctx->h_err_slots + ctx->err_slot.fetch_add(1) % tp_ctx::kErrSlots;
-      e = stage_device_error(ctx, stream, slot);
-    }
-    cudaError_t e2 = cudaStreamSynchronize(stream);
+    e = cudaStreamSynchronize(stream);
     release(ctx, g->parts, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "staging the device error word");
-    if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamSynchronize");
-    return g->check_err ? take_device_error(ctx, *slot) : TP_OK;
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    return g->check_err ? take_error(ctx, g->err) : TP_OK;
   }
-  e = g->check_err ? stage_device_error(ctx, stream, ex->event->h_err) : cudaSuccess;
-  if (e == cudaSuccess) e = cudaEventRecord(ex->event->ev, stream);
+  e = cudaEventRecord(ex->event->ev, stream);
   if (e != cudaSuccess) {
     release(ctx, g->parts, stream);
     return cuda_fail(e, "cudaEventRecord");
@@ -734,6 +736,8 @@ tp_status tp_graph_replay(tp_graph* g, const tp_exec* ex) {
   ex->event->recorded = true;
   ex->event->stream = stream;
   ex->event->check_err |= g->check_err;
+  auto& errs = ex->event->graph_errs;
+  if (g->check_err && std::find(errs.begin(), errs.end(), g->err) == errs.end()) errs.push_back(g->err);
   for (auto* p : g->parts) ex->event->held.push_back({p, stream, 1});
   return TP_OK;
 }
@@ -765,6 +769,7 @@ tp_status tp_graph_destroy(tp_graph* g) {
     for (auto* p : g->parts)
       if (p->busy.load()) return fail(TP_ERR_BUSY, "graph replay still in flight");
     if (g->ctx->capturing == g) return fail(TP_ERR_BUSY, "graph still capturing; call tp_graph_end");
+    return_word_locked(g->ctx, g->err);
   }
   if (g->exec) cudaGraphExecDestroy(g->exec);
   if (g->graph) cudaGraphDestroy(g->graph);
@@ -806,7 +811,7 @@ static tp_status map_op(tp_ctx* ctx, tp_partition* out, int op, float alpha, con
       return s;
     }
   }
-  s = launch_map(ctx, out, op, alpha, x, y, ex, o.stream, q);
+  s = launch_map(ctx, out, op, alpha, x, y, ex, o.stream, q, o.err);
   if (s != TP_OK) {
     o.abort();
     return s;
@@ -859,8 +864,8 @@ tp_status tp_gemm(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_ten
     }
   }
   o.check_err = true;  // the tensor-core and TMA-fed FP32 kernels' waits are bounded
-  s = simt ? launch_gemm_simt(ctx, c, a, b, cfg, ex, o.stream, q)
-           : launch_gemm_tc(ctx, c, a, b, cfg, ex, o.stream, q);
+  s = simt ? launch_gemm_simt(ctx, c, a, b, cfg, ex, o.stream, q, o.err)
+           : launch_gemm_tc(ctx, c, a, b, cfg, ex, o.stream, o.err);
   if (s != TP_OK) {
     o.abort();
     return s;
@@ -914,7 +919,7 @@ tp_status tp_gemm_unchecked(tp_ctx* ctx, void* c, const tp_tensor* a, const tp_t
   tp_exec ex{};
   ex.mode = TP_SYNC;
   ex.stream = stream;
-  return launch_gemm_tc(ctx, &p, a, b, cfg, &ex, static_cast<cudaStream_t>(stream), nullptr);
+  return launch_gemm_tc(ctx, &p, a, b, cfg, &ex, static_cast<cudaStream_t>(stream), ctx->words);
 }
 
 }  // extern "C"

@@ -112,3 +112,33 @@ def test_injected_timeout_is_refused_where_not_implemented(ctx):
         tp.tp_map_axpy(ctx, pz, 1.0, x, x, tp.make_exec(inject_timeout=True))
     assert e.value.status == tp._lib.ERR_UNSUPPORTED
     tp.tp_partition_destroy(pz)
+
+
+def test_each_operation_reports_its_own_failure(ctx):
+    """Failed and successful operations interleaved on one stream: each event
+    and replay reports exactly its own work, also when several graphs and
+    operations complete into one event, and events can be reused."""
+    s = torch.cuda.Stream()
+    bad, good, both = (tp.tp_event_create(ctx) for _ in range(3))
+    graphs = []
+    for arrive in (False, True):
+        g = tp.tp_graph_begin(ctx, s)
+        tp.tp_diag_bounded_wait(ctx, 1_000_000, arrive, tp.make_exec(tp.CAPTURE, s))
+        tp.tp_graph_end(g)
+        graphs.append(g)
+    for _ in range(2):
+        tp.tp_diag_bounded_wait(ctx, 1_000_000, False, tp.make_exec(tp.ASYNC, s, bad))
+        tp.tp_diag_bounded_wait(ctx, 1_000_000, True, tp.make_exec(tp.ASYNC, s, good))
+        tp.tp_graph_replay(graphs[0], tp.make_exec(tp.ASYNC, s, both))
+        tp.tp_graph_replay(graphs[1], tp.make_exec(tp.ASYNC, s, both))
+        tp.tp_diag_bounded_wait(ctx, 1_000_000, True, tp.make_exec(stream=s))       # SYNC: its own result
+        tp.tp_event_wait(good)
+        for ev in (bad, both):
+            with pytest.raises(tp.TPError) as e:
+                tp.tp_event_wait(ev)
+            assert e.value.status == tp._lib.ERR_TIMEOUT
+        tp.tp_graph_replay(graphs[1], tp.make_exec(stream=s))
+    for ev in (bad, good, both):
+        tp.tp_event_destroy(ev)
+    for g in graphs:
+        tp.tp_graph_destroy(g)
