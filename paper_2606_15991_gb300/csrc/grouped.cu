@@ -17,7 +17,7 @@
 // of column j, while their B slab is still in L2. The tail then costs MMA
 // columns for its rows rounded up to 32 instead of a full 256-row tile.
 //
-// Roles per CTA (192 threads): warp 0 dequeues slots, publishes them through
+// Roles per CTA (192 threads): warp 0 dequeues slots, publishes them, decoded, through
 // a 4-entry shared-memory ring and streams the tile's K slices with TMA;
 // warp 1 issues tcgen05.mma into two TMEM accumulators; warps 2-5 drain TMEM
 // and store. Every wait is bounded and reports TP_ERR_TIMEOUT.
@@ -91,7 +91,12 @@ template <bool kPair> struct Ring {
   static constexpr int kKc = kPair ? TP_GROUPED_PAIR_KC : 1;
   static constexpr int kStages = kPair ? 6 / TP_GROUPED_PAIR_KC : 4;
 };
-constexpr size_t kWordsBytes = 8 + 8 * kRing;
+// A ring entry: the queue slot (-1: the queue is empty) and what the roles need
+// of its tile, so that none of them starts a tile with a chain of global loads.
+//   0 slot   1 problem | tile row << 32   2 tile column | K blocks << 32
+//   3 K blocks per stage | MMA columns << 32   4 B-operand rows per CTA | stream_x << 32
+constexpr int kEntry = 5;  // 64-bit words
+constexpr size_t kWordsBytes = 8 + 8 * kEntry * kRing;
 constexpr int kWideKc = 3;  // K blocks per stage of a swap problem with few B rows (pairs)
 constexpr uint32_t kStageC = 4u * 2u * 4096u;  // epilogue staging: 4 warps x 2 buffers x (32 rows x 128 B)
 // Longest partial last 256-row band of a normal problem that CTA pairs run
@@ -147,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
   uint8_t* words = gbase + (bars - base) + 232u;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(words);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(words + 4);
-  volatile int64_t* ring = reinterpret_cast<volatile int64_t*>(words + 8);          // kRing slots
+  volatile int64_t* ring = reinterpret_cast<volatile int64_t*>(words + 8);          // kRing entries
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -183,16 +188,6 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  // decode a queue slot into (problem, tile row, tile column) through the
-  // plan's slot map; a problem's tiles are column-major over its tile grid so
-  // consecutive tiles share a B slab while the problem's A stays in L2
-  auto decode = [&](int64_t g, const GroupedProblem** pr, int64_t* tr, int64_t* tc) {
-    const int64_t e = p.slot_map[g];
-    *pr = p.probs + (e >> 32);
-    const int64_t local = e & 0xffffffffll;
-    *tr = local % (*pr)->tiles_r;
-    *tc = local / (*pr)->tiles_r;
-  };
   // wait for a ring slot's value; on a pair it may come from the peer CTA
   auto ring_wait = [&](uint32_t bar, uint32_t parity) {
     return kPair ? mbar_wait_cluster(bar, parity, abort_flag, p.err) : mbar_wait(bar, parity, abort_flag, p.err);
@@ -214,43 +209,88 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
-    for (int64_t j = 0; ok; ++j) {
+    // The leader dequeues tile j + 1 while it still streams tile j, in steps
+    // spread over tile j's last stages: the counter's atomic, the slot map's
+    // entry and the problem's fields are each in flight while a stage is
+    // issued. (A slot's tiles are column-major over the problem's tile grid,
+    // so consecutive ones share a B slab while the problem's A stays in L2.)
+    // Dequeuing and decoding at the start of each tile instead left a bubble
+    // of about 1.5 us there, longer than the ring covers. @@DEQ@@
+    int64_t nxt_slot = 0, nxt_entry = 0;
+    int32_t nxt_tiles_r = 1, nxt_nk = 0, nxt_kc = 1, nxt_bn = 0, nxt_box = 0, nxt_stream = 0;
+    auto dequeue = [&](int step, int64_t j) -> bool {
       const int r = (int)(j % kRing);
-      const uint32_t par = (uint32_t)((j / kRing) & 1);
-      int64_t g = 0;
-      if (leader) {
-        if (!ring_wait_warp(rempty_bar(r), par ^ 1u)) { ok = false; break; }
+      if (step == 0) {
+        if (!ring_wait_warp(rempty_bar(r), (uint32_t)((j / kRing) & 1) ^ 1u)) return false;
+        if (lane == 0) nxt_slot = (int64_t)atomicAdd(p.queue, 1u);
+      } else if (step == 1) {
+        nxt_slot = __shfl_sync(0xffffffffu, nxt_slot, 0);
+        if (nxt_slot >= p.total) nxt_slot = -1;
+        if (nxt_slot >= 0) nxt_entry = p.slot_map[nxt_slot];
+      } else if (step == 2) {
+        if (nxt_slot >= 0) {
+          // (problem << 32) | tile
+          const GroupedProblem* q = p.probs + (nxt_entry >> 32);
+          nxt_tiles_r = (int32_t)q->tiles_r;
+          nxt_nk = (int32_t)((q->K + 63) / 64);
+          nxt_kc = q->kc;
+          nxt_bn = q->bn;
+          nxt_box = q->box_y;
+          nxt_stream = q->stream_x;
+        }
+      } else {
+        int64_t w[kEntry] = {nxt_slot, 0, 0, 0, 0};
+        if (nxt_slot >= 0) {
+          const uint32_t prob = (uint32_t)(nxt_entry >> 32), local = (uint32_t)nxt_entry;
+          const uint32_t tc = local / (uint32_t)nxt_tiles_r, tr = local - tc * (uint32_t)nxt_tiles_r;
+          w[1] = (int64_t)prob | ((int64_t)tr << 32);
+          w[2] = (int64_t)tc | ((int64_t)nxt_nk << 32);
+          w[3] = (int64_t)nxt_kc | ((int64_t)nxt_bn << 32);
+          w[4] = (int64_t)nxt_box | ((int64_t)nxt_stream << 32);
+        }
         if (lane == 0) {
-          const int64_t d = (int64_t)atomicAdd(p.queue, 1u);
-          g = d < p.total ? d : -1;
-          ring[r] = g;
-          if constexpr (kPair) {
-            st_cluster_u64(mapa(smem_u32(const_cast<int64_t*>(ring + r)), 1), g);
-            mbar_arrive(rfull_bar(r));
-            mbar_arrive_cluster(mapa(rfull_bar(r), 1));
-          } else {
-            mbar_arrive(rfull_bar(r));
+#pragma unroll
+          for (int i = 0; i < kEntry; ++i) {
+            ring[kEntry * r + i] = w[i];
+            if constexpr (kPair) st_cluster_u64(mapa(smem_u32(const_cast<int64_t*>(ring + kEntry * r + i)), 1), w[i]);
+          }
+          mbar_arrive(rfull_bar(r));
+          if constexpr (kPair) mbar_arrive_cluster(mapa(rfull_bar(r), 1));
+          if (nxt_slot >= 0) {
+            tma_prefetch_desc(&p.probs[nxt_entry >> 32].map_x);
+            tma_prefetch_desc(&p.probs[nxt_entry >> 32].map_y);
           }
         }
-        g = __shfl_sync(0xffffffffu, g, 0);
-      } else {
-        if (!ring_wait_warp(rfull_bar(r), par)) { ok = false; break; }
-        g = __shfl_sync(0xffffffffu, ring[r], 0);
-        if (lane == 0) ring_release(r);
+        __syncwarp();
       }
+      return true;
+    };
+    constexpr int kSteps = 4;
+    if (leader)
+      for (int i = 0; i < kSteps && ok; ++i) ok = dequeue(i, 0);
+    for (int64_t j = 0; ok; ++j) {
+      const int r = (int)(j % kRing);
+      // the leader's own entry is already written (read back below); the odd
+      // CTA waits for it
+      if (!leader && !ring_wait_warp(rfull_bar(r), (uint32_t)((j / kRing) & 1))) { ok = false; break; }
+      const int64_t g = __shfl_sync(0xffffffffu, ring[kEntry * r], 0);
+      const int64_t w1 = __shfl_sync(0xffffffffu, ring[kEntry * r + 1], 0);
+      const int64_t w2 = __shfl_sync(0xffffffffu, ring[kEntry * r + 2], 0);
+      const int64_t w3 = __shfl_sync(0xffffffffu, ring[kEntry * r + 3], 0);
+      const int64_t w4 = __shfl_sync(0xffffffffu, ring[kEntry * r + 4], 0);
+      if (!leader && lane == 0) ring_release(r);
       if (g < 0) break;
-      const GroupedProblem* pr;
-      int64_t tr, tc;
-      decode(g, &pr, &tr, &tc);
-      const int32_t xrow = (int32_t)(tr * pr->tile_rows + rank * 128);
-      const int32_t yrow = (int32_t)(tc * pr->bn + rank * pr->box_y);
-      const int32_t pkc = pr->kc;
-      const uint32_t tx = (kStageX + (uint32_t)pr->box_y * 128u) * (uint32_t)pkc;
-      const int32_t nk = (int32_t)((pr->K + 63) / 64);
+      const GroupedProblem* pr = p.probs + (int32_t)w1;
+      const int32_t tr = (int32_t)(w1 >> 32), tc = (int32_t)w2, nk = (int32_t)(w2 >> 32);
+      const int32_t pkc = (int32_t)w3, bn = (int32_t)(w3 >> 32), box_y = (int32_t)w4;
+      const int32_t xrow = tr * (kPair ? 256 : 128) + (int32_t)rank * 128;
+      const int32_t yrow = tc * bn + (int32_t)rank * box_y;
+      const uint32_t tx = (kStageX + (uint32_t)box_y * 128u) * (uint32_t)pkc;
       // streamed swap: x = B_i slab (read once), y = A_i (reused by every tile)
-      const uint64_t px = pr->stream_x ? pol_stream : pol_keep;
+      const uint64_t px = (w4 >> 32) ? pol_stream : pol_keep;
       const CUtensorMap* mx = &pr->map_x;
       const CUtensorMap* my = &pr->map_y;
+      int step = 0;
       for (int32_t kb = 0; kb < nk; kb += pkc) {
         if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.err)) { ok = false; break; }
         // 2-D maps take K at element kb * 64; 3-D maps take K block kb (a
@@ -277,7 +317,14 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
         __syncwarp();
         ++filled;
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        // a step per stage over the last ones: late, so that a tile is not
+        // taken from a program that would start it sooner
+        if (leader && kb + (kSteps + 2) * pkc >= nk && step < kSteps) {
+          if (!dequeue(step++, j + 1)) { ok = false; break; }
+        }
       }
+      if (leader)
+        for (; step < kSteps && ok; ++step) ok = dequeue(step, j + 1);
     }
     if (!ok && leader) {
       for (uint32_t s2 = 0; s2 < (uint32_t)kStages && s2 < filled; ++s2)
@@ -293,21 +340,20 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
       for (int64_t j = 0; ok; ++j) {
         const int r = (int)(j % kRing);
         if (!mbar_wait_warp(rfull_bar(r), (uint32_t)((j / kRing) & 1), abort_flag, p.err)) { ok = false; break; }
-        const int64_t g = __shfl_sync(0xffffffffu, ring[r], 0);
+        const int64_t g = __shfl_sync(0xffffffffu, ring[kEntry * r], 0);
+        const int32_t nk = (int32_t)(__shfl_sync(0xffffffffu, ring[kEntry * r + 2], 0) >> 32);
+        const int64_t w3 = __shfl_sync(0xffffffffu, ring[kEntry * r + 3], 0);
+        const int32_t box_y = (int32_t)__shfl_sync(0xffffffffu, ring[kEntry * r + 4], 0);
         if (lane == 0) ring_release(r);
         if (g < 0) break;
-        const GroupedProblem* pr;
-        int64_t tr, tc;
-        decode(g, &pr, &tr, &tc);
         const int acc = (int)(j & 1);
         const uint32_t use = (uint32_t)((j >> 1) & 1);
         if (!mbar_wait_warp(tempty_bar(acc), use ^ 1u, abort_flag, p.err)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t idesc = idesc_f32acc(kPair ? 256 : 128, (uint32_t)pr->bn, false);
+        const uint32_t idesc = idesc_f32acc(kPair ? 256 : 128, (uint32_t)(w3 >> 32), false);
         const uint32_t d = tmem_base + (uint32_t)(acc * 256);
-        const int32_t nk = (int32_t)((pr->K + 63) / 64);
-        const int32_t pkc = pr->kc;
-        const uint32_t y_blk = (uint32_t)pr->box_y * 128u;  // one K block of the B operand
+        const int32_t pkc = (int32_t)w3;
+        const uint32_t y_blk = (uint32_t)box_y * 128u;  // one K block of the B operand
         for (int32_t kb = 0; kb < nk; kb += pkc) {
           if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.err)) { ok = false; break; }
           tc_fence_after();
@@ -359,13 +405,12 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
       const int r = (int)(j % kRing);
       const bool got = ring_wait(rfull_bar(r), (uint32_t)((j / kRing) & 1));
       if (!__all_sync(0xffffffffu, got)) break;  // leave together (tcgen05.ld below is warp-collective)
-      const int64_t g = ring[r];
+      const int64_t g = ring[kEntry * r], w1 = ring[kEntry * r + 1], w2 = ring[kEntry * r + 2];
       __syncwarp();
       if (lane == 0) ring_release(r);
       if (g < 0) break;
-      const GroupedProblem* pr;
-      int64_t tr, tc;
-      decode(g, &pr, &tr, &tc);
+      const GroupedProblem* pr = p.probs + (int32_t)w1;
+      const int64_t tr = w1 >> 32, tc = (int32_t)w2;
       const int acc = (int)(j & 1);
       const uint32_t use = (uint32_t)((j >> 1) & 1);
       const bool ready = mbar_wait(tfull_bar(acc), use, abort_flag, p.err);
