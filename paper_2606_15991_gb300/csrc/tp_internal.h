@@ -204,7 +204,7 @@ tp_status launch_map(tp_ctx* ctx, tp_partition* out, int op, float alpha, const 
                      const tp_tensor* y, const tp_exec* ex, cudaStream_t stream, unsigned* queue, int* err);
 tp_status launch_gemm_simt(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_tensor* b,
                            const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream,
-                           unsigned* queue, int* err);
+                           unsigned* queue);
 tp_status launch_gemm_tc(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_tensor* b,
                          const tp_gemm_config* cfg, const tp_exec* ex, cudaStream_t stream, int* err);
 
