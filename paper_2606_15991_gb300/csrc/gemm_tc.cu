@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
 
-  const int warp = threadIdx.x / 32;
+  const int warp = warp_index();
   const int lane = threadIdx.x % 32;
   // A CTA pair computes a 256-row tile: this CTA holds rows [rank*128, +128)
   // of A and of the accumulator, and B rows (tile columns) [rank*bn/2, +bn/2).
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if constexpr (kPair) cluster_sync();  // peer barriers initialised before any remote signal
   else __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   // The prologue above touches no global memory, so it may overlap the tail
   // of the grid this launch depends on (programmatic dependent launch).
   grid_dependency_wait();
@@ -296,11 +296,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer (the even CTA's warp 1; one elected lane
-    // issues). With the loop on one diverged lane, each MMA of a 128 x 64
-    // tile (32 tensor-core cycles at N = 64) took 60 cycles to issue: 1024^3
-    // on those tiles 6.29 us, 5.81 us converged; a single tile of K = 16384
-    // 46.4 and 41.7 us, now bound by the SM's operand stream (150 GB/s)
-    // rather than by issue.
+    // issues). What a stage costs this warp bounds tiles narrower than 128
+    // columns: the wait on the full barrier (95 cycles), the MMAs (23 each)
+    // and the commit (200) are a serial chain of 390 cycles for one K block of
+    // 64, so stages of several blocks cost less per block. It rests on the
+    // loop being warp-uniform: with one diverged lane running it an MMA took
+    // 60 cycles to issue, and with the warp's role not known to be uniform the
+    // chain was 580. One 128 x 64 tile of K = 16384 with 64 / 128 / 256
+    // elements a stage: 76.2 / 52.8 / 41.3 us before, 51.3 / 39.6 / 38.1 us
+    // (165 GB/s into the one SM); 1024^3 on such tiles 7.67 / 6.22 / 5.70 and
+    // 5.94 / 5.32 / 5.35 us.
     if (leader) {
       const uint32_t idesc_full = idesc_f32acc((uint32_t)tile_m, (uint32_t)p.bn, kF8);
       const uint32_t idesc_cut = idesc_f32acc((uint32_t)tile_m, (uint32_t)p.bn_cut, kF8);

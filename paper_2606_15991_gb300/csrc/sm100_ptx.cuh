@@ -79,12 +79,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// This thread's warp in the block, taken from lane 0 so that the compiler sees
+// one value per warp: a role selected by it is known to run converged, and its
+// loop state, addresses and descriptors stay in uniform registers (the form
+// copies and MMAs take their operands in). With threadIdx.x / 32 the same
+// loops moved every operand of every instruction over: four MMAs of a K block
+// took 237 cycles to issue, 92 with this (see the MMA issuer of the tile GEMM).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x / 32), 0); }
+
 // One lane of a converged warp (the same lane on every call). The roles that
-// issue TMA copies and MMAs run their loops with the whole warp and put only
-// the issuing instructions behind this predicate: loop state, addresses and
-// descriptors then stay warp-uniform, the form those instructions take their
-// operands in, where a loop run by a single diverged lane has to move every
-// operand over for every instruction.
+// issue copies and MMAs run their loops with the whole warp and put only the
+// issuing instructions behind this predicate, so that everything else stays
+// warp-uniform (warp_index).
 __device__ __forceinline__ bool elect_one() {
   uint32_t ok;
   asm volatile(
@@ -95,10 +101,24 @@ __device__ __forceinline__ bool elect_one() {
   return ok != 0;
 }
 
-// mbar_wait by every lane of a converged warp; one outcome for the warp.
+// mbar_wait by every lane of a converged warp; one outcome for the warp. Each
+// attempt is voted on, so that the loop's branches are the warp's and not the
+// lanes'.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort, int* err,
                                                uint64_t limit_ns = 2000000000ull) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, err, limit_ns)) != 0;
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const uint64_t t0 = global_timer_ns();
+  for (uint32_t i = 1;; ++i) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((i & 63) == 0) {
+      if (abort && __any_sync(0xffffffffu, *abort)) return false;
+      if (__any_sync(0xffffffffu, global_timer_ns() - t0 > limit_ns)) {
+        if (abort) *abort = 1;
+        if (err) atomicExch(err, 1);
+        return false;
+      }
+    }
+  }
 }
 
 // -------------------------------------------------------------------- TMA
