@@ -395,3 +395,42 @@ def test_segment_tiles_equal_the_scalar_path(ctx, op, dt, shape, tile, kind, P, 
         tp.tp_partition_destroy(part)
     for o in outs[1:]:
         assert torch.equal(outs[0].view(torch.uint8), o.view(torch.uint8))
+
+
+@pytest.mark.parametrize("op,dt", [("axpy", "f32"), ("axpy", "bf16"), ("add_accum", "f32"), ("add_accum", "bf16")])
+@pytest.mark.parametrize("kind,P", [("identity", 0), ("strided", 3), ("strided", 700), ("queue", 2), ("queue", 700)])
+@pytest.mark.parametrize("shape,tile", [
+    ((100003,), (1,)), ((100003,), (100,)),           # tiles below a warp's round, odd and whole slots
+    ((100003,), (1000,)), ((100008,), (2048,)),       # whole vectors, several groups of threads per block
+    ((300007,), (16384,)),                            # a block of more than 256 threads per tile
+    ((4001, 131), (16, 20)), ((700, 264), (16, 64)),  # rows ending inside slots, rows of whole slots
+    ((9, 130, 72), (2, 16, 24)),
+])
+def test_tile_groups_equal_one_tile(ctx, op, dt, kind, P, shape, tile):
+    """Tiles dealt to groups of threads give the bits of one tile that is the
+    whole tensor, each element written once and by the program that owns it."""
+    n = int(np.prod(shape))
+    xs, ys, cs = (t.reshape(shape) for t in _inputs(n, dt))
+    tiles = opart.num_tiles(shape, tile)
+    P = min(P, tiles)
+    kinds = {"identity": tp.MAP_IDENTITY, "strided": tp.MAP_STRIDED, "queue": tp.MAP_QUEUE}
+    counts = torch.zeros(n, dtype=torch.int32, device="cuda")
+    owner = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+    outs = []
+    for t, ex in ((shape, None), (tile, None), (tile, tp.make_exec(write_counts=counts, write_owner=owner))):
+        out = cs.clone()
+        part = tp.tp_partition_create(ctx, out, t)
+        if t is tile and kind != "identity":
+            tp.tp_partition_map(part, kinds[kind], P)
+        args = (ctx, part, ALPHA, xs, ys, ex) if op == "axpy" else (ctx, part, xs, ys, ex)
+        FN[op](*args)
+        outs.append(out)
+        tp.tp_partition_destroy(part)
+    for o in outs[1:]:
+        assert torch.equal(outs[0].view(torch.uint8), o.view(torch.uint8))
+    assert opart.check_counts(counts.cpu().numpy())["ok"]
+    own = owner.cpu().numpy()
+    if kind == "queue":
+        assert own.min() >= 0 and own.max() < P
+    else:
+        assert np.array_equal(own, opart.owner_map(shape, tile, P or None, kind).reshape(-1))
