@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
   float* obuf = red + 16;
   // rgroups < 8: the warps' sums of two consecutive units overlay it
   float* psum = obuf;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   constexpr int rgroups = kRg, cblocks = kSConsumers / rgroups;
   constexpr int urows = 4 * rgroups;             // rows of a plain unit
   constexpr int stage_cols = kSCols * cblocks;   // columns of a stage
@@ -437,13 +437,16 @@ __global__ void __launch_bounds__(kSThreads, 1)
     *slice = p.slices > 1 ? (int32_t)(ub % p.slices) : 0;
   };
   if (warp == kSConsumers) {
-    // ---------------- producer: one thread issues every copy. With K
-    // slices, unit t's x slice goes to buffer t mod xbufs; the first unit's
-    // weight stages (as many as the ring holds) are issued before the
-    // dependency wait, the x slices only after it.
-    if (lane == 0) {
-      uint32_t fills[kSStages] = {};
-      uint32_t xfills[kSMaxXBufs] = {};
+    // ---------------- producer: the warp walks the schedule, one elected lane
+    // issues every copy (elect_one). With K slices, unit t's x slice goes to
+    // buffer t mod xbufs; the first unit's weight stages (as many as the ring
+    // holds) are issued before the dependency wait, the x slices only after
+    // it. With this loop on one diverged lane and per-lane waits in every role,
+    // what a copy cost to issue bounded the stream: 5120 x 25600 41.9 us, 20896
+    // x 2848 23.1, 10240 x 5120 19.2, a fused layer of d = 5120 133.1; so 38.3
+    // (6.85 TB/s), 19.7, 17.5 and 128.1 us (6.96 TB/s).
+    {
+      uint32_t filled = 0, xfilled = 0;  // ring stages and x buffers filled so far
       int stage = 0;
       uint32_t phase = 0;
       int64_t t = 0;  // units taken by this CTA
@@ -459,16 +462,19 @@ __global__ void __launch_bounds__(kSThreads, 1)
         const CUtensorMap* m = second ? &map1 : &map0;
         const int32_t r0 = (int32_t)(rb * (pair ? kSPairRows : urows));
         auto issue = [&](int64_t st) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.err, p.wait_ns)) return false;
+          if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.err, p.wait_ns)) return false;
           const int32_t c0 = (int32_t)(slice * p.slice_cols + st * stage_cols);  // 512-byte aligned
           const uint32_t dst = base + (uint32_t)kSStage * stage;
-          mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kSStage);
-          if (pair) tma_load_3d(dst, m, c0, r0, 0, full_bar(stage), pol);  // g rows, then their u rows
-          else if (rgroups < 8 && p.box3) tma_load_3d(dst, m, 0, r0, c0 / kSCols, full_bar(stage), pol);
-          else
-            for (int cb = 0; cb < cblocks; ++cb)  // a block past the last column arrives as zeros
-              tma_load_2d(dst + (uint32_t)(cb * urows * kSCols * 2), m, c0 + cb * kSCols, r0, full_bar(stage), pol);
-          fills[stage]++;
+          if (elect_one()) {
+            mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kSStage);
+            if (pair) tma_load_3d(dst, m, c0, r0, 0, full_bar(stage), pol);  // g rows, then their u rows
+            else if (rgroups < 8 && p.box3) tma_load_3d(dst, m, 0, r0, c0 / kSCols, full_bar(stage), pol);
+            else
+              for (int cb = 0; cb < cblocks; ++cb)  // a block past the last column arrives as zeros
+                tma_load_2d(dst + (uint32_t)(cb * urows * kSCols * 2), m, c0 + cb * kSCols, r0, full_bar(stage), pol);
+          }
+          __syncwarp();
+          ++filled;
           if (++stage == nst) { stage = 0; phase ^= 1u; }
           return true;
         };
@@ -482,9 +488,12 @@ __global__ void __launch_bounds__(kSThreads, 1)
           }
           const uint32_t bytes = (uint32_t)(p.k / 4) * 16u;
           if (bytes) {
-            mbar_arrive_expect_tx(xfull_bar(0), bytes);
-            bulk_copy_g2s(xs0, p.x, bytes, xfull_bar(0));
-            xfills[0]++;
+            if (elect_one()) {
+              mbar_arrive_expect_tx(xfull_bar(0), bytes);
+              bulk_copy_g2s(xs0, p.x, bytes, xfull_bar(0));
+            }
+            __syncwarp();
+            ++xfilled;
           }
         }
         if (p.slices > 1) {
@@ -498,24 +507,27 @@ __global__ void __launch_bounds__(kSThreads, 1)
           }
           // this unit's slice of x (whole 8-float pieces: k is a multiple of 8)
           const int xb = (int)(t % xbufs);
-          if (!mbar_wait(xempty_bar(xb), (uint32_t)(((t / xbufs) & 1) ^ 1), abort_flag, p.err, p.wait_ns)) {
+          if (!mbar_wait_warp(xempty_bar(xb), (uint32_t)(((t / xbufs) & 1) ^ 1), abort_flag, p.err, p.wait_ns)) {
             ok = false;
             break;
           }
           const int64_t c0 = (int64_t)slice * p.slice_cols;
           const uint32_t bytes = (uint32_t)(min(p.slice_cols, p.k - c0) * 4);
-          mbar_arrive_expect_tx(xfull_bar(xb), bytes);
-          bulk_copy_g2s(xs0 + 4u * xstride * (uint32_t)xb, p.x + c0, bytes, xfull_bar(xb));
-          xfills[xb]++;
+          if (elect_one()) {
+            mbar_arrive_expect_tx(xfull_bar(xb), bytes);
+            bulk_copy_g2s(xs0 + 4u * xstride * (uint32_t)xb, p.x + c0, bytes, xfull_bar(xb));
+          }
+          __syncwarp();
+          ++xfilled;
         }
         for (; st < stages_per_unit && ok; ++st) ok = issue(st);
       }
       if (!ok) {
-        // every copy this thread issued lands before the CTA retires
-        for (int s2 = 0; s2 < nst; ++s2)
-          if (fills[s2]) mbar_wait(full_bar(s2), (fills[s2] - 1u) & 1u, nullptr, nullptr, 200000000ull);
-        for (int b = 0; b < kSMaxXBufs; ++b)
-          if (xfills[b]) mbar_wait(xfull_bar(b), (xfills[b] - 1u) & 1u, nullptr, nullptr, 200000000ull);
+        // every copy this warp issued lands before the CTA retires
+        for (uint32_t s2 = 0; s2 < (uint32_t)nst && s2 < filled; ++s2)
+          mbar_wait(full_bar((int)s2), ((filled - s2 - 1u) / (uint32_t)nst) & 1u, nullptr, nullptr, 200000000ull);
+        for (uint32_t b = 0; b < (uint32_t)xbufs && b < xfilled; ++b)
+          mbar_wait(xfull_bar((int)b), ((xfilled - b - 1u) / (uint32_t)xbufs) & 1u, nullptr, nullptr, 200000000ull);
       }
     }
     __syncwarp();
@@ -574,8 +586,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
       const float* xs = xsp + (size_t)xstride * xb;
       const int64_t lim = min(p.k - (int64_t)slice * p.slice_cols, p.slice_cols);  // valid x in this slice
       if (p.slices > 1) {
-        const bool got = mbar_wait(xfull_bar(xb), (uint32_t)((t / xbufs) & 1), abort_flag, p.err, p.wait_ns);
-        if (!__all_sync(0xffffffffu, got)) break;
+        if (!mbar_wait_warp(xfull_bar(xb), (uint32_t)((t / xbufs) & 1), abort_flag, p.err, p.wait_ns)) break;
       }
       // rgroups < 8: warp 0 stores the unit's rows (lane = row); the values a
       // residual adds to are fetched ahead
@@ -603,8 +614,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
 #pragma unroll
           for (int j = 0; j < 8; ++j) xv[j] = cx + j < lim ? xs[cx + j] : 0.f;
         }
-        const bool got = mbar_wait(full_bar(stage), phase, abort_flag, p.err, p.wait_ns);
-        if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+        if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
         const uint32_t src = base + (uint32_t)kSStage * stage;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -647,16 +657,14 @@ __global__ void __launch_bounds__(kSThreads, 1)
         const uint32_t use = (uint32_t)((t >> 1) & 1);
         const uint32_t ps_full = xempty_bar(par), ps_empty = xfull_bar(2 + par);
         float* ps = psum + par * kSRows;
-        bool got = mbar_wait(ps_empty, use ^ 1u, abort_flag, p.err, p.wait_ns);
-        if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+        if (!mbar_wait_warp(ps_empty, use ^ 1u, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
         if (lane == 0) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) ps[wcol * urows + 4 * wrow + q] = sum[q];
           mbar_arrive(ps_full);
         }
         if (warp == 0) {
-          got = mbar_wait(ps_full, use, abort_flag, p.err, p.wait_ns);
-          if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+          if (!mbar_wait_warp(ps_full, use, abort_flag, p.err, p.wait_ns)) { ok = false; break; }
           const int64_t r = rb * urows + lane;
           if (lane < urows && r < p.rows0) {
             float v = 0.f;
@@ -886,6 +894,8 @@ int whole_x_stages(int64_t k) {
 //   32 rows 22.3 / 15.7 / 63.5 / 75.2   16 rows 19.6 / 12.8 / 48.2 / 75.7
 //    8 rows 20.3 / 12.5 / 42.0 / 83.5    4 rows 26.8 / 15.3 / 41.9 / 124
 //   per-lane gemv_kernel 21.3 / 14.0 / 62.5 / 78.3
+// and, since the producer's warp runs converged, 17.5 / 11.1 / 38.3 / 73.8 with
+// the shapes that the rule takes.
 void unit_rows(StreamArgs* a, int64_t rows, int64_t k, int sms) {
   a->rgroups = 8;
   a->box3 = 0;
@@ -1189,7 +1199,7 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
   if (d > 0 && ni > 0 && stream_ok(a_in) && ni <= kSMaxXCols) {
     // x whole in shared memory and units shaped to the matrix: one launch,
     // each row summed in one place (4096 x 4096: 11.1 us in two K slices and
-    // a finish kernel, 8.4 so; 5120 x 5120: 15.6 and 12.5)
+    // a finish kernel, 8.4 so; 5120 x 5120: 15.6 and 11.3)
     o.check_err = true;  // the streaming kernel's waits are bounded
     StreamArgs sa = whole_x_args(ctx, a, kResidual);
     sa.early_weights = (ex->flags & TP_EXEC_STATIC_WEIGHTS) ? 1 : 0;
@@ -1204,7 +1214,8 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
   // ring, and more of them (down to 2048 columns) while the units (32-row
   // block x slice) number under four per SM; slices of equal whole stages.
   // Few long units beat many short ones (measured: a 5120 x 25600 product
-  // takes 43.4 us in 4 slices, 44.7 us in 10, 52 us in 15).
+  // takes 43.4 us in 4 slices, 44.7 us in 10, 52 us in 15; 40.8 in 4 since the
+  // producer runs converged).
   const int64_t row_blocks = (d + kSRows - 1) / kSRows;
   const int64_t max_cols = stream_max_slice_cols();
   int64_t slices64 = (ni + max_cols - 1) / max_cols;
