@@ -254,7 +254,7 @@ constexpr int kSMaxXCols = 8192;                  // x (or a slice of it) kept i
 constexpr int kSXVec = kSMaxXCols / (kSConsumers * 32 * 4);  // 16-byte pieces of x per consumer thread
 constexpr int kSMaxXBufs = 4;                     // x slice buffers (sliced mode)
 constexpr int kSOBuf = 32;                        // units whose outputs are held in shared memory
-constexpr size_t kSSmemMax = 232448;              // opt-in shared memory per CTA
+constexpr size_t kSSmemMax = kSmemOptin;
 // shared memory beside the x buffers: alignment slack, ring, barriers, abort word, reduction scratch
 // alignment slack, barriers, abort word, reduction scratch, output buffer (+ the ring and x)
 constexpr size_t kSSmemFixed = 1024 + 8 * (2 * kSStages + 2 * kSMaxXBufs) + 16 + 64 + (size_t)kSOBuf * kSRows * 4;
@@ -812,10 +812,12 @@ bool vec_out(const tp_partition* p, int64_t n) {
 template <int kEpi, int kParts, int kUnroll>
 cudaError_t launch_gemv(const GemvArgs& a, int grid, cudaStream_t st) {
   const size_t smem = (((a.k + 3) & ~int64_t(3)) + 16 + 2 * kWarps) * sizeof(float);
-  auto k = a.counts ? gemv_kernel<kEpi, kParts, kUnroll, true> : gemv_kernel<kEpi, kParts, kUnroll, false>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > (size_t)kSmemOptin) return cudaErrorInvalidValue;
+  constexpr auto counted = gemv_kernel<kEpi, kParts, kUnroll, true>;
+  constexpr auto plain = gemv_kernel<kEpi, kParts, kUnroll, false>;
+  cudaError_t e = a.counts ? allow_smem<counted>(kSmemOptin) : allow_smem<plain>(kSmemOptin);
   if (e != cudaSuccess) return e;
-  return launch_dependent(k, grid, kThreads, smem, st, a);
+  return launch_dependent(a.counts ? counted : plain, grid, kThreads, smem, st, a);
 }
 
 int gemv_grid(tp_ctx* ctx, int64_t k) {
@@ -943,17 +945,21 @@ tp_status launch_stream(tp_ctx* ctx, StreamArgs a, const tp_tensor* w0, bool pai
   const size_t smem = fixed + xbuf * (size_t)a.xbufs;
   // x by a bulk copy when it has more columns than the registers stage (never
   // with norm: that takes at most kSMaxXCols)
+  cudaError_t e = cudaSuccess;
+  auto instance = [&](auto count, auto rgroups, auto bulk) {
+    constexpr auto k = gemv_stream_kernel<decltype(count)::value, decltype(rgroups)::value, decltype(bulk)::value>;
+    e = allow_smem<k>((int)kSSmemMax);
+    return k;
+  };
   auto pick = [&](auto count, auto bulk) {
-    constexpr bool kC = decltype(count)::value, kB = decltype(bulk)::value;
-    return a.rgroups == 8   ? gemv_stream_kernel<kC, 8, kB>
-           : a.rgroups == 4 ? gemv_stream_kernel<kC, 4, kB>
-           : a.rgroups == 2 ? gemv_stream_kernel<kC, 2, kB>
-                            : gemv_stream_kernel<kC, 1, kB>;
+    return a.rgroups == 8   ? instance(count, std::integral_constant<int, 8>{}, bulk)
+           : a.rgroups == 4 ? instance(count, std::integral_constant<int, 4>{}, bulk)
+           : a.rgroups == 2 ? instance(count, std::integral_constant<int, 2>{}, bulk)
+                            : instance(count, std::integral_constant<int, 1>{}, bulk);
   };
   const bool bulk_x = a.slices == 1 && a.slice_cols > kSMaxXCols;
   auto k = a.counts ? (bulk_x ? pick(std::true_type{}, std::true_type{}) : pick(std::true_type{}, std::false_type{}))
                     : (bulk_x ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{}));
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return cuda_fail(e, "streaming matrix-vector kernel attributes");
   // the fewest CTAs (at most one per SM) that take as many units each as
   // one per SM would: every CTA gets the same count, give or take one
@@ -1279,8 +1285,8 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
     else {
       const int64_t slice = ((ni / 8 + parts - 1) / parts) * 8 + 8;
       const size_t smem = (size_t)((slice + 3) & ~int64_t(3)) * sizeof(float);
-      auto k = gemv_partial_kernel<8>;
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      constexpr auto k = gemv_partial_kernel<8>;
+      e = smem > (size_t)kSmemOptin ? cudaErrorInvalidValue : allow_smem<k>(kSmemOptin);
       if (e == cudaSuccess) {
         const int grid = ctx->sm_count * 4;  // a multiple of `parts` on every GB300 SM count used (152)
         k<<<(grid / parts) * parts, kThreads, smem, o.stream>>>(a, parts, ctx->d_partial);

@@ -337,12 +337,13 @@ __global__ void __launch_bounds__(TH, kCtas) gemm_f32_kernel(const __grid_consta
 
 template <int kFetchA, int kFetchB, bool kSplit, bool COUNT>
 cudaError_t launch_inst(const SimtArgs& p, int64_t programs, int sms, cudaStream_t st) {
-  auto k = gemm_f32_kernel<kFetchA, kFetchB, kSplit, COUNT>;
+  constexpr auto k = gemm_f32_kernel<kFetchA, kFetchB, kSplit, COUNT>;
   // Clusters are packed onto as few SMs as hold them: a split launch asks for
   // enough shared memory that no SM takes more CTAs than an even spread needs.
   const int64_t per_sm = (programs * p.split + sms - 1) / sms;
-  const size_t smem = p.split == 1 || per_sm >= kCtas ? kSmem : std::max(kSmem, kSmemSm / (size_t)(per_sm + 1) + 1024);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto spread = [](int64_t ctas) { return std::max(kSmem, kSmemSm / (size_t)(ctas + 1) + 1024); };
+  const size_t smem = p.split == 1 || per_sm >= kCtas ? kSmem : spread(per_sm);
+  cudaError_t e = allow_smem<k>((int)(kSplit ? spread(1) : kSmem));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(programs * p.split));

@@ -758,13 +758,9 @@ struct Maps {
 
 template <bool kF8, bool kPair, bool kCount, bool kChecked, bool kSwap = false>
 cudaError_t launch_kernel(const Maps& m, const TcArgs& p, int grid, int csize, size_t smem, cudaStream_t st) {
-  auto k = gemm_tc_kernel<kF8, kPair, kCount, kChecked, kSwap>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  constexpr auto k = gemm_tc_kernel<kF8, kPair, kCount, kChecked, kSwap>;
+  const cudaError_t e = allow_smem<k>(kSmemOptin);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kThreads);
@@ -811,8 +807,8 @@ cudaError_t launch_any(bool pair, bool count, bool checked, const Maps& m, const
 // the kernel that can be resident at once (0 when the query fails).
 template <bool kPair>
 int max_active_clusters(int csize, size_t smem) {
-  auto k = gemm_tc_kernel<false, kPair, false, false>;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448) != cudaSuccess) return 0;
+  constexpr auto k = gemm_tc_kernel<false, kPair, false, false>;
+  if (allow_smem<k>(kSmemOptin) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)csize);
   cfg.blockDim = dim3(kThreads);

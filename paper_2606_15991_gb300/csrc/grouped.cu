@@ -28,6 +28,7 @@
 #include <algorithm>
 #include <cstring>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "sm100_ptx.cuh"
@@ -847,8 +848,9 @@ tp_status tp_grouped_gemm(tp_ctx* ctx, tp_grouped_plan* plan, int32_t num_progra
   const int grid = (int)(pair ? 2 * programs : programs);
   size_t smem;
   cudaError_t e;
-  auto launch = [&](auto kernel, size_t bytes, int cluster) {
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  auto launch = [&](auto pairs, auto counted, size_t bytes, int cluster) {
+    constexpr auto kernel = grouped_kernel<decltype(pairs)::value, decltype(counted)::value>;
+    cudaError_t err = allow_smem<kernel>((int)bytes);  // the same for every launch of the instance
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)grid);
@@ -864,14 +866,16 @@ tp_status tp_grouped_gemm(tp_ctx* ctx, tp_grouped_plan* plan, int32_t num_progra
     lc.numAttrs = 1;
     return cudaLaunchKernelEx(&lc, kernel, a);
   };
+  constexpr std::true_type yes;
+  constexpr std::false_type no;
   if (pair) {
     smem = 1024 + (kStageX + Ring<true>::kStageY) * Ring<true>::kKc * Ring<true>::kStages + kStageC + 232 +
            kWordsBytes;
-    e = a.counts ? launch(grouped_kernel<true, true>, smem, 2) : launch(grouped_kernel<true, false>, smem, 2);
+    e = a.counts ? launch(yes, yes, smem, 2) : launch(yes, no, smem, 2);
   } else {
     smem = 1024 + (kStageX + Ring<false>::kStageY) * Ring<false>::kKc * Ring<false>::kStages + kStageC + 232 +
            kWordsBytes;
-    e = a.counts ? launch(grouped_kernel<false, true>, smem, 1) : launch(grouped_kernel<false, false>, smem, 1);
+    e = a.counts ? launch(no, yes, smem, 1) : launch(no, no, smem, 1);
   }
   return o.end(e);
 }

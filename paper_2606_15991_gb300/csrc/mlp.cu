@@ -364,10 +364,13 @@ __global__ void __launch_bounds__(kGradThreads) grads_kernel(const __grid_consta
   }
 }
 
-template <typename K, typename A>
-cudaError_t launch_pdl(K kernel, const A& a, int grid, int threads, size_t smem, cudaStream_t st) {
+// Shared memory of the rows kernel that the weights may take part in.
+constexpr size_t kRowsSmem = 200 * 1024;
+
+template <auto K, typename A>
+cudaError_t launch_pdl(const A& a, int grid, int threads, size_t smem, cudaStream_t st) {
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem<K>((int)kRowsSmem);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
@@ -380,7 +383,7 @@ cudaError_t launch_pdl(K kernel, const A& a, int grid, int threads, size_t smem,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, a);
+  return cudaLaunchKernelEx(&cfg, K, a);
 }
 
 int row_ctas(int B) { return (B + kRowsPerCta - 1) / kRowsPerCta; }
@@ -403,15 +406,15 @@ cudaError_t launch_rows(tp_mlp* n, const float* X, const float* T, const float* 
   a.dy = n->dy;
   a.part = n->part;
   // the weights stay in global memory when they do not fit beside the
-  // activations in 200 KB
+  // activations (32 KB at most)
   const int64_t params = rows_params(a.F, a.H, a.C), acts = rows_acts(a.H, a.C);
-  a.staged = (params + acts) * (int64_t)sizeof(float) <= 200 * 1024 ? 1 : 0;
+  a.staged = (params + acts) * sizeof(float) <= kRowsSmem ? 1 : 0;
   a.ld1 = a.staged ? a.F | 1 : a.F;
   a.ld2 = a.staged ? a.H | 1 : a.H;
   const size_t smem = (size_t)(acts + (a.staged ? params : 0)) * sizeof(float);
   const int threads = kRowThreads * kRowsPerCta;
-  return T ? launch_pdl(rows_kernel<true>, a, row_ctas(B), threads, smem, st)
-           : launch_pdl(rows_kernel<false>, a, row_ctas(B), threads, smem, st);
+  return T ? launch_pdl<rows_kernel<true>>(a, row_ctas(B), threads, smem, st)
+           : launch_pdl<rows_kernel<false>>(a, row_ctas(B), threads, smem, st);
 }
 
 tp_status launch_forward(tp_mlp* n, const float* X, int B, float* Y, cudaStream_t st) {
@@ -450,7 +453,7 @@ tp_status launch_loss_grad(tp_mlp* n, const float* X, const float* T, const floa
   }
   auto blocks = [](int rows, int cols) { return (rows + kGradRows - 1) / kGradRows * ((cols + kGradCols - 1) / kGradCols); };
   const int grid = blocks(a.C, a.H) + blocks(a.H, a.H) + blocks(a.H, a.F);
-  e = launch_pdl(grads_kernel, a, grid, kGradThreads, 0, st);
+  e = launch_pdl<grads_kernel>(a, grid, kGradThreads, 0, st);
   return e == cudaSuccess ? TP_OK : cuda_fail(e, "mlp backward");
 }
 

@@ -189,6 +189,25 @@ tp_status take_error(tp_ctx* ctx, int* word);
 // An error word to lend (ctx->mu held); the context's own when none is left.
 int* lend_word_locked(tp_ctx* ctx);
 void return_word_locked(tp_ctx* ctx, int* word);
+// Dynamic shared memory a CTA may opt in to (sm_103).
+constexpr int kSmemOptin = 232448;
+// Lets launches of kernel K ask for up to `bytes` of dynamic shared memory.
+// The limit is the process's, so `bytes` is a constant of the instance, the
+// most that any launch of it needs: a launch that set its own size could lower
+// the limit under another thread's launch. Set once per device.
+template <auto K>
+cudaError_t allow_smem(int bytes) {
+  static std::atomic<uint64_t> done{0};  // a bit per device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? uint64_t(1) << dev : 0;
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
+
 // An ASYNC launch may record `ev` on `stream`: OK when the event tracks no
 // unfinished work on another stream (completed work is released first).
 tp_status event_claim(tp_event* ev, cudaStream_t stream);

@@ -224,3 +224,40 @@ def test_operand_layouts_give_one_result(ctx, m, n, k, split):
     an, bn_ = a.cpu().double().numpy(), b.cpu().double().numpy()
     bound = (k + 4) * 2.0 ** -24 * (np.abs(an) @ np.abs(bn_)) + 1e-37
     assert np.all(np.abs(want.cpu().double().numpy() - ogemm.gemm(a.cpu(), b.cpu())) <= bound)
+
+
+def test_split_products_of_two_sizes_from_two_threads(ctx):
+    """Split programs ask for shared memory by the size of their grid (here 64
+    and 256 CTAs, 114 and 76 KB of one instance): launches of two host threads
+    do not get in each other's way."""
+    import threading
+
+    errors = []
+    want = {}
+    ops = {}
+    for m in (256, 512):
+        a = torch.from_numpy(synth.uniform(m * 64, seed=m)).reshape(m, 64).cuda()
+        b = torch.from_numpy(synth.uniform(64 * m, seed=m + 1)).reshape(64, m).cuda()
+        ops[m] = a, b, torch.zeros(m, m, device="cuda")
+        want[m] = _gemm(ctx, a, b, bk=32, split_k=4)[0]
+    torch.cuda.synchronize()
+
+    def body(m):
+        try:
+            a, b, c = ops[m]
+            ex = tp.make_exec(stream=torch.cuda.Stream())
+            p = tp.tp_partition_create(ctx, c, (64, 64))
+            for _ in range(1500):
+                tp.tp_gemm(ctx, p, a, b, tp.gemm_config(bk=32, split_k=4), ex)
+            tp.tp_partition_destroy(p)
+        except Exception as e:  # noqa: BLE001 - reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=body, args=(m,)) for m in ops]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert errors == []
+    for m in ops:
+        assert torch.equal(ops[m][2], want[m])

@@ -1,0 +1,73 @@
+"""Host code of the library on a CUDA runtime that runs nothing
+(fake_cudart.cpp): what launches ask for and what they share, without a GPU."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2606_15991_gb300 as tp
+from paper_2606_15991_gb300 import _lib, build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def host_path(built_lib, tmp_path_factory):
+    """libtp linked with the fake runtime."""
+    out = tmp_path_factory.mktemp("host")
+    obj, so = str(out / "fake.o"), str(out / "libtp_host.so")
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-I" + inc, "-c", os.path.join(HERE, "fake_cudart.cpp"),
+                    "-o", obj], check=True)
+    subprocess.run([build.nvcc(), "-shared", "--cudart", "none", "-Xlinker", "-Bsymbolic", "-o", so, obj] +
+                   sorted(glob.glob(os.path.join(build.BUILD, "*.o"))), check=True)
+    return so
+
+
+@pytest.fixture
+def host(host_path, monkeypatch):
+    L = ctypes.CDLL(host_path)
+    for name, args in _lib._PROTOS.items():
+        f = getattr(L, name)
+        f.argtypes, f.restype = args, _lib._RESTYPES.get(name, ctypes.c_int32)
+    monkeypatch.setattr(_lib, "_lib", L)
+    yield L
+    L.fake_finish()
+
+
+S1, S2 = 0x100, 0x200  # streams
+
+
+def _exec(mode=_lib.SYNC, stream=S1, event=None):
+    return tp.make_exec(mode, stream, event)
+
+
+def test_shared_memory_limits_are_never_lowered(host):
+    """A kernel's dynamic shared-memory limit belongs to the process: a launch
+    that set it to its own size would fail a larger launch of another thread
+    made between that thread's set and its launch."""
+    ctx = tp.tp_ctx_create(0)
+    for m, n, split in ((512, 512, 2), (1024, 512, 4), (512, 512, 4), (2048, 2048, 2), (64, 64, 2)):
+        a, b, c = torch.zeros(m, 64), torch.zeros(64, n), torch.zeros(m, n)
+        p = tp.tp_partition_create(ctx, c, (64, 64))
+        tp.tp_gemm(ctx, p, a, b, tp.gemm_config(split_k=split), _exec())
+        tp.tp_partition_destroy(p)
+    for hidden in (160, 96, 128):
+        m = tp.tp_mlp_create(ctx, 5, hidden, 72, 4, np.zeros(5 * hidden + hidden * hidden + 74 * hidden + 72, np.float32))
+        tp.tp_mlp_forward(m, torch.zeros(4, 5), torch.zeros(4, 72), _exec())
+        tp.tp_mlp_destroy(m)
+    for k in (40000, 16384, 24576, 512, 20480):
+        buf = torch.zeros(k + 8)
+        at = -buf.data_ptr() // 4 % 4
+        for off in (at, at + 1):      # streamed, where it fits, and per lane
+            w, x, y = torch.zeros(256, k, dtype=torch.bfloat16), buf[off:off + k], torch.zeros(256)
+            p = tp.tp_partition_create(ctx, y, (256,))
+            tp.tp_gemv(ctx, p, w, x, _exec())
+            tp.tp_decode_down_residual(ctx, p, w, x, _exec())
+            tp.tp_partition_destroy(p)
+    tp.tp_ctx_destroy(ctx)
+    assert host.fake_lowered() == 0
