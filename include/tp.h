@@ -237,7 +237,8 @@ tp_status tp_version(int32_t* major, int32_t* minor);
  * word, queue counters, scale scratch) once, so later calls can be captured.
  * Errors: TP_ERR_INVALID (null out), TP_ERR_CUDA (no such device / no sm_103). */
 tp_status tp_ctx_create(int32_t device, tp_ctx** out);
-/* Frees the context and its workspace. TP_ERR_BUSY if work is still in flight. */
+/* Frees the context and its workspace. TP_ERR_BUSY if work is still in flight.
+ * Its events and graphs may be destroyed before or after it. */
 tp_status tp_ctx_destroy(tp_ctx* ctx);
 /* Number of SMs and compute capability of the context's device. */
 tp_status tp_ctx_info(tp_ctx* ctx, int32_t* sm_count, int32_t* cc_major, int32_t* cc_minor);
@@ -286,7 +287,8 @@ tp_status tp_event_create(tp_ctx* ctx, tp_event** ev);
 tp_status tp_event_query(tp_event* ev, int32_t* done);
 /* Blocks until completion, releases the held partitions, reports errors. */
 tp_status tp_event_wait(tp_event* ev);
-/* TP_ERR_BUSY if it still holds partitions of unfinished work. */
+/* TP_ERR_BUSY if it still holds partitions of unfinished work; waits for
+ * unfinished work that holds none but may still report an error. */
 tp_status tp_event_destroy(tp_event* ev);
 
 /* ----------------------------------------------------------------- graphs */
@@ -304,6 +306,9 @@ tp_status tp_graph_replay(tp_graph* g, const tp_exec* ex);
  * kernels). TP_ERR_INVALID before tp_graph_end; TP_ERR_CUDA if the graph
  * cannot be walked. */
 tp_status tp_graph_kernel_count(tp_graph* g, int64_t* count);
+/* TP_ERR_BUSY while the graph is being captured or a replay of it holds its
+ * partitions. A replay in flight that holds none runs on, and the event it was
+ * recorded into still reports its errors. */
 tp_status tp_graph_destroy(tp_graph* g);
 
 /* ----------------------------------------------------- element-wise maps */

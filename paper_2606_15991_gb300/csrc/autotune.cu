@@ -255,12 +255,12 @@ tp_status time_config(tp_ctx* ctx, TuneState* st, const TuneProblem& pb, const t
   part.num_programs = std::min<int64_t>(part.num_tiles, cap);
   if (c.num_programs > 0) part.num_programs = std::min<int64_t>(part.num_tiles, c.num_programs);
   if (c.split_k > 1) part.num_programs = part.num_tiles;  // a split program holds one tile
-  tp_status ls = launch_gemm_tc_impl(ctx, &part, &pb.a, &pb.b, &c, &pb.ex, st->stream, pb.esize, pb.one, pb.one, ctx->words);
+  tp_status ls = launch_gemm_tc_impl(ctx, &part, &pb.a, &pb.b, &c, &pb.ex, st->stream, pb.esize, pb.one, pb.one, ctx->own->err);
   if (ls != TP_OK) return ls;
   delay_kernel<<<1, 32, 0, st->stream>>>(20000ull + 30000ull * (uint64_t)r);
   cudaEventRecord(e0, st->stream);
   for (int j = 0; j < r && ls == TP_OK; ++j)
-    ls = launch_gemm_tc_impl(ctx, &part, &pb.a, &pb.b, &c, &pb.ex, st->stream, pb.esize, pb.one, pb.one, ctx->words);
+    ls = launch_gemm_tc_impl(ctx, &part, &pb.a, &pb.b, &c, &pb.ex, st->stream, pb.esize, pb.one, pb.one, ctx->own->err);
   cudaEventRecord(e1, st->stream);
   cudaError_t e = cudaEventSynchronize(e1);
   if (e != cudaSuccess) return cuda_fail(e, "autotune timing");
@@ -334,7 +334,7 @@ tp_status tp_autotune(tp_ctx* ctx, int64_t M, int64_t N, int64_t K, int32_t dtyp
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  tp_status es = take_error(ctx, ctx->words);
+  tp_status es = take_error(ctx, ctx->own->err);
   if (es != TP_OK) return es;
   if (best_i < 0) return fail(TP_ERR_CUDA, "no configuration ran");
   st->cache[TuneKey{M, N, K, dtype, flags}] = {cfgs[best_i], best_tf};
@@ -364,7 +364,7 @@ tp_status tp_autotune_time(tp_ctx* ctx, int64_t M, int64_t N, int64_t K, int32_t
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (s != TP_OK) return s;
-  tp_status es = take_error(ctx, ctx->words);
+  tp_status es = take_error(ctx, ctx->own->err);
   if (es != TP_OK) return es;
   std::sort(tf.begin(), tf.end());
   *tflops_median = repeats % 2 ? tf[repeats / 2] : 0.5f * (tf[repeats / 2 - 1] + tf[repeats / 2]);

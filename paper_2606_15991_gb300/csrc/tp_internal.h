@@ -5,7 +5,9 @@
 
 #include <atomic>
 #include <cstdint>
+#include <deque>
 #include <functional>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <unordered_map>
@@ -16,7 +18,7 @@
 
 namespace tp {
 
-// Device-side error codes written to an error word (tp_ctx::words).
+// Device-side error codes written to an error word (Workspace::err).
 enum DeviceError : int {
   kDevOk = 0,
   kDevTimeout = 1,     // a bounded wait ran out of iterations
@@ -49,6 +51,34 @@ struct HoldKeyHash {
     return std::hash<const void*>()(k.first) * 31u ^ std::hash<const void*>()(k.second);
   }
 };
+
+// What the kernels of an operation, an event's operations or a graph report to
+// as long as any of them may run.
+struct Workspace {
+  // Error word (DeviceError) in pinned host memory that kernels write to
+  // directly, and only when something failed: an operation that went well
+  // moves nothing to report so.
+  int* err = nullptr;
+};
+
+// Workspaces of a context: lent to a SYNC operation for the call, to an event
+// and to a graph until it is gone and the work recorded into it has ended. It
+// grows by blocks as more are out at a time. The last holder (the context, its
+// events, its graphs) frees them, so that events and graphs may be destroyed
+// after their context.
+class WorkspacePool {
+ public:
+  ~WorkspacePool();
+  cudaError_t take(Workspace** out);
+  void give(Workspace* w);
+  std::atomic<bool> closed{false};  // the context is gone
+ private:
+  static constexpr int kBlock = 4096;
+  std::mutex mu_;
+  std::deque<Workspace> all_;       // (a deque: their addresses stay)
+  std::vector<Workspace*> free_;
+  std::vector<int*> blocks_;        // error words, kBlock each
+};
 }  // namespace tp
 
 struct tp_ctx {
@@ -61,17 +91,9 @@ struct tp_ctx {
   // stream adds to the entry's count
   std::unordered_map<tp::HoldKey, int64_t, tp::HoldKeyHash> busy;
   tp_graph* capturing = nullptr;    // graph being captured, if any
+  std::shared_ptr<tp::WorkspacePool> pool;
+  tp::Workspace* own = nullptr;     // of launches that no operation reports for
   // Device workspace, allocated once at creation.
-  // Error words (tp::DeviceError) in pinned host memory that kernels write to
-  // directly, and only when something failed: an operation that went well
-  // moves nothing to report so. words[0] is the context's (launches that no
-  // operation reports for), the next kSyncWords serve SYNC operations in turn,
-  // the rest are lent to events and graphs.
-  int* words = nullptr;
-  std::atomic<uint32_t> sync_word{0};
-  std::vector<int> free_words;      // indices to lend, under mu
-  static constexpr int kSyncWords = 256;
-  static constexpr int kWords = 4096;
   unsigned* d_queue = nullptr;      // tile-queue counters (kQueueSlots)
   float* d_scratch = nullptr;       // small float scratch (kScratchFloats)
   float* d_partial = nullptr;       // matrix-vector partial sums (kPartialFloats)
@@ -98,25 +120,37 @@ struct tp_partition {
   std::atomic<int> busy{0};  // number of in-flight holds
 };
 
+namespace tp {
+// What a replay needs: kept by the graph and by the events that its replays in
+// flight were recorded into.
+struct GraphRun {
+  explicit GraphRun(std::shared_ptr<WorkspacePool> p) : pool(std::move(p)) {}
+  ~GraphRun();
+  std::shared_ptr<WorkspacePool> pool;
+  Workspace* ws = nullptr;           // of the recorded operations
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  bool check_err = false;
+};
+}  // namespace tp
+
 struct tp_event {
   tp_ctx* ctx = nullptr;
+  std::shared_ptr<tp::WorkspacePool> pool;
   cudaEvent_t ev = nullptr;
   bool recorded = false;
   bool check_err = false;
   cudaStream_t stream = nullptr;  // stream of the last record
-  int* err = nullptr;             // error word of the operations recorded into it
-  std::vector<int*> graph_errs;   // error words of the graphs replayed into it
+  tp::Workspace* ws = nullptr;    // of the operations recorded into it
+  std::vector<std::shared_ptr<tp::GraphRun>> replays;  // graphs replayed into it
   std::vector<tp::Hold> held;   // holds released when the event completes (appended per op)
 };
 
 struct tp_graph {
   tp_ctx* ctx = nullptr;
+  std::shared_ptr<tp::GraphRun> run;
   cudaStream_t stream = nullptr;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
   bool ended = false;
-  bool check_err = false;
-  int* err = nullptr;                // error word of the recorded operations
   std::vector<tp_partition*> parts;  // partitions written by recorded nodes
 };
 
@@ -157,6 +191,11 @@ struct DeviceGuard {
 struct Op {
   Op() = default;
   explicit Op(const char* op_name) : name(op_name) {}
+  Op(const Op&) = delete;
+  Op& operator=(const Op&) = delete;
+  ~Op() {
+    if (lent) ctx->pool->give(lent);
+  }
   const char* name = "op";   // entry point, for the TP_LOG trace
   tp_ctx* ctx = nullptr;
   const tp_exec* ex = nullptr;
@@ -164,6 +203,7 @@ struct Op {
   std::vector<tp_partition*> outs;
   bool check_err = false;   // kernel may write the error word
   int* err = nullptr;       // error word for this operation's kernels (set by begin)
+  Workspace* lent = nullptr;  // SYNC: the operation's own workspace
   bool marked = false;
   bool allow_checked = false;  // the op implements TP_EXEC_CHECKED (set before begin)
   bool allow_inject = false;   // the op implements TP_EXEC_INJECT_TIMEOUT (set before begin)
@@ -186,9 +226,6 @@ struct Op {
 // Status of the error in `word` (or, when it holds none, in the context's
 // word), read after the work that may write it has completed; clears it.
 tp_status take_error(tp_ctx* ctx, int* word);
-// An error word to lend (ctx->mu held); the context's own when none is left.
-int* lend_word_locked(tp_ctx* ctx);
-void return_word_locked(tp_ctx* ctx, int* word);
 // Dynamic shared memory a CTA may opt in to (sm_103).
 constexpr int kSmemOptin = 232448;
 // Lets launches of kernel K ask for up to `bytes` of dynamic shared memory.

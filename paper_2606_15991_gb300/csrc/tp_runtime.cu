@@ -141,7 +141,7 @@ static int take_word(int* word) { return __atomic_exchange_n(word, 0, __ATOMIC_A
 
 tp_status take_error(tp_ctx* ctx, int* word) {
   int h = take_word(word);
-  if (h == kDevOk && word != ctx->words) h = take_word(ctx->words);
+  if (h == kDevOk && word != ctx->own->err) h = take_word(ctx->own->err);
   if (h == kDevOk) return TP_OK;
   // a checked launch that gave up part-way may have left claim state
   // behind; the next launch must start from zero
@@ -152,16 +152,42 @@ tp_status take_error(tp_ctx* ctx, int* word) {
   return error_status(h);
 }
 
-int* lend_word_locked(tp_ctx* ctx) {
-  if (ctx->free_words.empty()) return ctx->words;
-  int* w = ctx->words + ctx->free_words.back();
-  ctx->free_words.pop_back();
-  *w = kDevOk;
-  return w;
+WorkspacePool::~WorkspacePool() {
+  for (int* b : blocks_) cudaFreeHost(b);
 }
 
-void return_word_locked(tp_ctx* ctx, int* word) {
-  if (word != ctx->words) ctx->free_words.push_back((int)(word - ctx->words));
+cudaError_t WorkspacePool::take(Workspace** out) {
+  std::lock_guard<std::mutex> lk(mu_);
+  if (free_.empty()) {
+    // allowed while this thread captures, as nothing of it is recorded
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    int* words = nullptr;
+    const cudaError_t e = cudaMallocHost(&words, sizeof(int) * kBlock);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
+    blocks_.push_back(words);
+    for (int i = 0; i < kBlock; ++i) {
+      all_.push_back({words + i});
+      free_.push_back(&all_.back());
+    }
+  }
+  *out = free_.back();
+  free_.pop_back();
+  *(*out)->err = kDevOk;
+  return cudaSuccess;
+}
+
+void WorkspacePool::give(Workspace* w) {
+  if (!w) return;
+  std::lock_guard<std::mutex> lk(mu_);
+  free_.push_back(w);
+}
+
+GraphRun::~GraphRun() {
+  if (exec) cudaGraphExecDestroy(exec);
+  if (graph) cudaGraphDestroy(graph);
+  pool->give(ws);
 }
 
 tp_status claims_for(tp_ctx* ctx, int64_t bits, uint32_t** claims, unsigned** done) {
@@ -287,10 +313,11 @@ tp_status Op::begin_impl(tp_ctx* c, const tp_exec* e, const std::vector<tp_parti
         return fail(TP_ERR_BUSY, "an input reads bytes of a partition with work in flight on another stream");
   }
   if (ex->mode == TP_SYNC) {
-    err = ctx->words + 1 + ctx->sync_word.fetch_add(1) % tp_ctx::kSyncWords;
-    *err = kDevOk;
+    cudaError_t we = ctx->pool->take(&lent);
+    if (we != cudaSuccess) return cuda_fail(we, "allocating operation workspaces");
+    err = lent->err;
   } else {
-    err = ex->mode == TP_ASYNC ? ex->event->err : ctx->capturing->err;
+    err = ex->mode == TP_ASYNC ? ex->event->ws->err : ctx->capturing->run->ws->err;
   }
   if (ex->mode == TP_CAPTURE) {
     for (auto* p : outs) {
@@ -318,11 +345,13 @@ tp_status Op::end(cudaError_t launch_err) {
 
 tp_status Op::end_impl(cudaError_t launch_err) {
   if (launch_err != cudaSuccess) {
+    // kernels launched before the one that failed may still report
+    if (ex->mode != TP_CAPTURE) cudaStreamSynchronize(stream);
     if (marked) release(ctx, outs, stream);
     return cuda_fail(launch_err, "kernel launch");
   }
   if (ex->mode == TP_CAPTURE) {
-    if (check_err) ctx->capturing->check_err = true;
+    if (check_err) ctx->capturing->run->check_err = true;
     return TP_OK;
   }
   if (ex->mode == TP_SYNC) {
@@ -399,7 +428,8 @@ tp_status tp_ctx_create(int32_t device, tp_ctx** out) {
     delete c;
     return fail(TP_ERR_UNSUPPORTED, "this library is built for sm_103a (Blackwell) only");
   }
-  e = cudaMallocHost(&c->words, sizeof(int) * tp_ctx::kWords);
+  c->pool = std::make_shared<WorkspacePool>();
+  e = c->pool->take(&c->own);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_queue, sizeof(unsigned) * tp_ctx::kQueueSlots);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_scratch, sizeof(float) * tp_ctx::kScratchFloats);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_partial, sizeof(float) * tp_ctx::kPartialFloats);
@@ -414,12 +444,9 @@ tp_status tp_ctx_create(int32_t device, tp_ctx** out) {
     cudaFree(c->d_partial);
     cudaFree(c->d_claims);
     cudaFree(c->d_claim_done);
-    cudaFreeHost(c->words);
     delete c;
     return cuda_fail(e, "allocating context workspace");
   }
-  std::fill(c->words, c->words + tp_ctx::kWords, (int)kDevOk);
-  for (int i = tp_ctx::kWords - 1; i > tp_ctx::kSyncWords; --i) c->free_words.push_back(i);
   *out = c;
   return TP_OK;
 }
@@ -431,6 +458,7 @@ tp_status tp_ctx_destroy(tp_ctx* ctx) {
     if (!ctx->busy.empty()) return fail(TP_ERR_BUSY, "context still has work in flight");
     if (ctx->capturing) return fail(TP_ERR_BUSY, "context is capturing a graph");
   }
+  ctx->pool->closed = true;
   // the frees wait for the device, so no kernel is left that could still write
   // an error word
   cudaFree(ctx->d_queue);
@@ -438,7 +466,6 @@ tp_status tp_ctx_destroy(tp_ctx* ctx) {
   cudaFree(ctx->d_partial);
   cudaFree(ctx->d_claims);
   cudaFree(ctx->d_claim_done);
-  cudaFreeHost(ctx->words);
   delete ctx;
   return TP_OK;
 }
@@ -572,29 +599,41 @@ tp_status tp_event_create(tp_ctx* ctx, tp_event** out) {
     delete ev;
     return cuda_fail(e, "cudaEventCreate");
   }
-  std::lock_guard<std::mutex> lk(ctx->mu);
-  ev->err = lend_word_locked(ctx);
+  ev->pool = ctx->pool;
+  e = ev->pool->take(&ev->ws);
+  if (e != cudaSuccess) {
+    cudaEventDestroy(ev->ev);
+    delete ev;
+    return cuda_fail(e, "allocating event workspaces");
+  }
   *out = ev;
   return TP_OK;
 }
 
 static tp_status event_complete(tp_event* ev) {
+  const bool open = !ev->pool->closed;  // (a context that is gone holds nothing)
   std::vector<Hold> held;
-  std::vector<int*> errs;
+  std::vector<std::shared_ptr<GraphRun>> replays;
   bool chk;
   {
-    std::lock_guard<std::mutex> lk(ev->ctx->mu);
+    std::unique_lock<std::mutex> lk;
+    if (open) lk = std::unique_lock<std::mutex>(ev->ctx->mu);
     held.swap(ev->held);
-    errs.swap(ev->graph_errs);
+    replays.swap(ev->replays);
     chk = ev->check_err;
     ev->check_err = false;
     ev->recorded = false;
     for (auto& h : held) release_locked(ev->ctx, h.p, h.stream, h.count);
   }
   if (!chk) return TP_OK;
-  tp_status s = take_error(ev->ctx, ev->err);
-  for (int* w : errs) {
-    const tp_status gs = take_error(ev->ctx, w);
+  auto take = [&](int* word) {
+    if (open) return take_error(ev->ctx, word);
+    const int h = take_word(word);
+    return h == kDevOk ? TP_OK : error_status(h);
+  };
+  tp_status s = take(ev->ws->err);
+  for (auto& r : replays) {
+    const tp_status gs = r->check_err ? take(r->ws->err) : TP_OK;
     if (s == TP_OK) s = gs;
   }
   return s;
@@ -645,12 +684,12 @@ tp_status tp_event_destroy(tp_event* ev) {
     if (cudaEventQuery(ev->ev) == cudaErrorNotReady)
       return fail(TP_ERR_BUSY, "event still holds partitions of unfinished work");
     event_complete(ev);
+  } else if (ev->recorded && (ev->check_err || !ev->replays.empty())) {
+    // work that holds no partition, but may still report to the workspace
+    cudaEventSynchronize(ev->ev);
   }
   cudaEventDestroy(ev->ev);
-  {
-    std::lock_guard<std::mutex> lk(ev->ctx->mu);
-    return_word_locked(ev->ctx, ev->err);
-  }
+  ev->pool->give(ev->ws);
   delete ev;
   return TP_OK;
 }
@@ -664,12 +703,17 @@ tp_status tp_graph_begin(tp_ctx* ctx, void* stream, tp_graph** out) {
   auto* g = new tp_graph();
   g->ctx = ctx;
   g->stream = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal);
+  g->run = std::make_shared<GraphRun>(ctx->pool);
+  cudaError_t e = ctx->pool->take(&g->run->ws);
+  if (e != cudaSuccess) {
+    delete g;
+    return cuda_fail(e, "allocating graph workspaces");
+  }
+  e = cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) {
     delete g;
     return cuda_fail(e, "cudaStreamBeginCapture");
   }
-  g->err = lend_word_locked(ctx);
   ctx->capturing = g;
   *out = g;
   return TP_OK;
@@ -683,16 +727,16 @@ tp_status tp_graph_end(tp_graph* g) {
     g->ctx->capturing = nullptr;
   }
   g->ended = true;
-  cudaError_t e = cudaStreamEndCapture(g->stream, &g->graph);
+  cudaError_t e = cudaStreamEndCapture(g->stream, &g->run->graph);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-  e = cudaGraphInstantiate(&g->exec, g->graph, 0);
+  e = cudaGraphInstantiate(&g->run->exec, g->run->graph, 0);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
   return TP_OK;
 }
 
 tp_status tp_graph_replay(tp_graph* g, const tp_exec* ex) {
   if (!g || !ex) return fail(TP_ERR_INVALID, "null argument");
-  if (!g->ended || !g->exec) return fail(TP_ERR_INVALID, "graph not ended/instantiated");
+  if (!g->ended || !g->run->exec) return fail(TP_ERR_INVALID, "graph not ended/instantiated");
   if (ex->mode == TP_CAPTURE) return fail(TP_ERR_CAPTURE, "a replay cannot itself be captured here");
   if (ex->mode == TP_ASYNC && (!ex->event || ex->event->ctx != g->ctx))
     return fail(TP_ERR_INVALID, "TP_ASYNC needs an event of the graph's context");
@@ -716,7 +760,7 @@ tp_status tp_graph_replay(tp_graph* g, const tp_exec* ex) {
       return es;
     }
   }
-  cudaError_t e = cudaGraphLaunch(g->exec, stream);
+  cudaError_t e = cudaGraphLaunch(g->run->exec, stream);
   if (e != cudaSuccess) {
     release(ctx, g->parts, stream);
     return cuda_fail(e, "cudaGraphLaunch");
@@ -725,7 +769,7 @@ tp_status tp_graph_replay(tp_graph* g, const tp_exec* ex) {
     e = cudaStreamSynchronize(stream);
     release(ctx, g->parts, stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    return g->check_err ? take_error(ctx, g->err) : TP_OK;
+    return g->run->check_err ? take_error(ctx, g->run->ws->err) : TP_OK;
   }
   e = cudaEventRecord(ex->event->ev, stream);
   if (e != cudaSuccess) {
@@ -735,21 +779,21 @@ tp_status tp_graph_replay(tp_graph* g, const tp_exec* ex) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   ex->event->recorded = true;
   ex->event->stream = stream;
-  ex->event->check_err |= g->check_err;
-  auto& errs = ex->event->graph_errs;
-  if (g->check_err && std::find(errs.begin(), errs.end(), g->err) == errs.end()) errs.push_back(g->err);
+  ex->event->check_err |= g->run->check_err;
+  auto& replays = ex->event->replays;
+  if (std::find(replays.begin(), replays.end(), g->run) == replays.end()) replays.push_back(g->run);
   for (auto* p : g->parts) ex->event->held.push_back({p, stream, 1});
   return TP_OK;
 }
 
 tp_status tp_graph_kernel_count(tp_graph* g, int64_t* count) {
   if (!g || !count) return fail(TP_ERR_INVALID, "null argument");
-  if (!g->ended || !g->graph) return fail(TP_ERR_INVALID, "graph not ended");
+  if (!g->ended || !g->run->graph) return fail(TP_ERR_INVALID, "graph not ended");
   size_t n = 0;
-  cudaError_t e = cudaGraphGetNodes(g->graph, nullptr, &n);
+  cudaError_t e = cudaGraphGetNodes(g->run->graph, nullptr, &n);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGraphGetNodes");
   std::vector<cudaGraphNode_t> nodes(n);
-  if (n > 0) e = cudaGraphGetNodes(g->graph, nodes.data(), &n);
+  if (n > 0) e = cudaGraphGetNodes(g->run->graph, nodes.data(), &n);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGraphGetNodes");
   int64_t k = 0;
   for (size_t i = 0; i < n; ++i) {
@@ -764,16 +808,13 @@ tp_status tp_graph_kernel_count(tp_graph* g, int64_t* count) {
 
 tp_status tp_graph_destroy(tp_graph* g) {
   if (!g) return fail(TP_ERR_INVALID, "null graph");
-  {
+  if (!g->run->pool->closed) {
     std::lock_guard<std::mutex> lk(g->ctx->mu);
     for (auto* p : g->parts)
       if (p->busy.load()) return fail(TP_ERR_BUSY, "graph replay still in flight");
     if (g->ctx->capturing == g) return fail(TP_ERR_BUSY, "graph still capturing; call tp_graph_end");
-    return_word_locked(g->ctx, g->err);
   }
-  if (g->exec) cudaGraphExecDestroy(g->exec);
-  if (g->graph) cudaGraphDestroy(g->graph);
-  delete g;
+  delete g;  // (replays in flight that hold no partition keep what they use)
   return TP_OK;
 }
 
@@ -919,7 +960,7 @@ tp_status tp_gemm_unchecked(tp_ctx* ctx, void* c, const tp_tensor* a, const tp_t
   tp_exec ex{};
   ex.mode = TP_SYNC;
   ex.stream = stream;
-  return launch_gemm_tc(ctx, &p, a, b, cfg, &ex, static_cast<cudaStream_t>(stream), ctx->words);
+  return launch_gemm_tc(ctx, &p, a, b, cfg, &ex, static_cast<cudaStream_t>(stream), ctx->own->err);
 }
 
 }  // extern "C"

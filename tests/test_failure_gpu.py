@@ -142,3 +142,28 @@ def test_each_operation_reports_its_own_failure(ctx):
         tp.tp_event_destroy(ev)
     for g in graphs:
         tp.tp_graph_destroy(g)
+
+
+def test_destroyed_in_flight_reports_to_nobody_else(ctx):
+    """An event, and a graph, destroyed while work without an output partition
+    runs that will report a timeout: what is created next does not see it, and
+    the replay's event does."""
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    gone, replay = tp.tp_event_create(ctx), tp.tp_event_create(ctx)
+    tp.tp_diag_bounded_wait(ctx, 200_000_000, False, tp.make_exec(tp.ASYNC, s1, gone))
+    tp.tp_event_destroy(gone)
+    g = tp.tp_graph_begin(ctx, s1)
+    tp.tp_diag_bounded_wait(ctx, 200_000_000, False, tp.make_exec(tp.CAPTURE, s1))
+    tp.tp_graph_end(g)
+    tp.tp_graph_replay(g, tp.make_exec(tp.ASYNC, s1, replay))
+    tp.tp_graph_destroy(g)
+    fresh = [tp.tp_event_create(ctx) for _ in range(2)]
+    for ev, s in zip(fresh, (s1, s2)):
+        tp.tp_diag_bounded_wait(ctx, 1_000_000, True, tp.make_exec(tp.ASYNC, s, ev))
+    for ev in fresh:
+        tp.tp_event_wait(ev)
+    with pytest.raises(tp.TPError) as e:
+        tp.tp_event_wait(replay)
+    assert e.value.status == tp._lib.ERR_TIMEOUT
+    for ev in fresh + [replay]:
+        tp.tp_event_destroy(ev)

@@ -4,6 +4,7 @@ import ctypes
 import glob
 import os
 import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -71,3 +72,88 @@ def test_shared_memory_limits_are_never_lowered(host):
             tp.tp_partition_destroy(p)
     tp.tp_ctx_destroy(ctx)
     assert host.fake_lowered() == 0
+
+
+def _wait_op(ctx, ok, ex):
+    """An operation without an output partition whose kernel gives up (or not)."""
+    tp.tp_diag_bounded_wait(ctx, 1_000_000, ok, ex)
+
+
+def _times_out(event):
+    with pytest.raises(tp.TPError) as e:
+        tp.tp_event_wait(event)
+    return e.value.status == _lib.ERR_TIMEOUT
+
+
+def test_event_destroyed_in_flight_keeps_its_word(host):
+    ctx = tp.tp_ctx_create(0)
+    ev = tp.tp_event_create(ctx)
+    _wait_op(ctx, False, _exec(tp.ASYNC, S1, ev))
+    tp.tp_event_destroy(ev)
+    fresh = tp.tp_event_create(ctx)
+    _wait_op(ctx, True, _exec(tp.ASYNC, S2, fresh))
+    host.fake_finish()
+    tp.tp_event_wait(fresh)      # not the first event's late timeout
+    tp.tp_event_destroy(fresh)
+    tp.tp_ctx_destroy(ctx)
+
+
+def test_graph_destroyed_in_flight_keeps_its_word(host):
+    ctx = tp.tp_ctx_create(0)
+    replay, fresh = tp.tp_event_create(ctx), None
+    g = tp.tp_graph_begin(ctx, S1)
+    _wait_op(ctx, False, _exec(tp.CAPTURE, S1))
+    tp.tp_graph_end(g)
+    tp.tp_graph_replay(g, _exec(tp.ASYNC, S1, replay))
+    tp.tp_graph_destroy(g)
+    fresh = tp.tp_event_create(ctx)
+    _wait_op(ctx, True, _exec(tp.ASYNC, S2, fresh))
+    host.fake_finish()
+    tp.tp_event_wait(fresh)
+    assert _times_out(replay)
+    for ev in (replay, fresh):
+        tp.tp_event_destroy(ev)
+    tp.tp_ctx_destroy(ctx)
+
+
+def test_any_number_of_events_report_their_own_errors(host):
+    ctx = tp.tp_ctx_create(0)
+    events = [tp.tp_event_create(ctx) for _ in range(5000)]
+    for i, ev in enumerate(events):
+        _wait_op(ctx, i % 2 == 0, _exec(tp.ASYNC, S1, ev))
+    host.fake_finish()
+    for i, ev in enumerate(events):
+        assert i % 2 == 0 or _times_out(ev)
+        tp.tp_event_wait(ev)
+    _wait_op(ctx, True, _exec())
+    for ev in events:
+        tp.tp_event_destroy(ev)
+    tp.tp_ctx_destroy(ctx)
+    assert host.fake_hosts() == 0
+
+
+def test_events_and_graphs_outlive_their_context(host_path):
+    """In a process whose allocator overwrites what is freed."""
+    child = f"""
+import ctypes
+L = ctypes.CDLL({host_path!r})
+V = ctypes.c_void_p
+ctx, ev, used, g = V(), V(), V(), V()
+class Exec(ctypes.Structure):
+    _fields_ = [("mode", ctypes.c_int32), ("flags", ctypes.c_int32)] + [(n, V) for n in "seco"]
+def ok(st): assert st == 0, st
+ok(L.tp_ctx_create(0, ctypes.byref(ctx)))
+ok(L.tp_event_create(ctx, ctypes.byref(ev)))
+ok(L.tp_event_create(ctx, ctypes.byref(used)))
+ok(L.tp_graph_begin(ctx, V(0x100), ctypes.byref(g)))
+ok(L.tp_graph_end(g))
+ok(L.tp_diag_bounded_wait(ctx, ctypes.c_int64(1000000), 0, ctypes.byref(Exec(1, 0, 0x100, used.value))))
+ok(L.tp_ctx_destroy(ctx))
+ok(L.tp_event_destroy(ev))
+ok(L.tp_graph_destroy(g))
+assert L.tp_event_wait(used) == {_lib.ERR_TIMEOUT}
+ok(L.tp_event_destroy(used))
+assert L.fake_hosts() == 0
+"""
+    subprocess.run([sys.executable, "-c", child], check=True, timeout=120,
+                   env={**os.environ, "MALLOC_PERTURB_": "165"})
