@@ -1230,8 +1230,14 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
   int64_t slice_cols = slices == 1 ? ni : ((ni + slices - 1) / slices + kSCols - 1) / kSCols * kSCols;
   if (slices > 1) slices = (int32_t)((ni + slice_cols - 1) / slice_cols);
   // (x slices arrive by bulk copies, whose sizes are multiples of 16 bytes)
-  const bool streamed = stream_ok(a_in) && (slices == 1 || ni % 4 == 0) && d * slices <= tp_ctx::kPartialFloats;
+  const bool streamed = stream_ok(a_in) && (slices == 1 || ni % 4 == 0) && d * slices <= WorkspacePool::kPartialFloats;
+  float* partial = nullptr;
   if (d > 0 && ni > 0 && streamed) {
+    s = slices > 1 ? o.partial(&partial) : TP_OK;
+    if (s != TP_OK) {
+      o.abort();
+      return s;
+    }
     o.check_err = true;  // the streaming kernel's waits are bounded
     // 32-row units; with slices, a finish kernel adds the partial sums to h
     // in slice order
@@ -1248,7 +1254,7 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
     sa.rgroups = 8;
     sa.y0 = a.y;
     sa.y1 = a.y;
-    sa.partial = ctx->d_partial;
+    sa.partial = partial;
     sa.x = a.x;
     sa.early_weights = (ex->flags & TP_EXEC_STATIC_WEIGHTS) ? 1 : 0;
     sa.counts = sa.slices > 1 ? nullptr : a.counts;
@@ -1268,33 +1274,38 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
       attr[0].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      e = a.counts ? cudaLaunchKernelEx(&cfg, residual_finish_kernel<true>, a.y, (const float*)ctx->d_partial, d,
+      e = a.counts ? cudaLaunchKernelEx(&cfg, residual_finish_kernel<true>, a.y, (const float*)partial, d,
                                         (int)sa.slices, a.counts, a.owner)
-                   : cudaLaunchKernelEx(&cfg, residual_finish_kernel<false>, a.y, (const float*)ctx->d_partial, d,
+                   : cudaLaunchKernelEx(&cfg, residual_finish_kernel<false>, a.y, (const float*)partial, d,
                                         (int)sa.slices, (uint32_t*)nullptr, (int32_t*)nullptr);
       if (e == cudaSuccess) e = cudaGetLastError();
     }
     return o.end(e);
   }
   // few long rows: split K into 8 slices, one slice per CTA (so 4 CTAs fit
-  // per SM); partial sums go to context scratch allocated once, and a
+  // per SM); partial sums go to the operation's workspace, and a
   // finish kernel adds them to h in slice order
   const int parts = 8;
   if (d > 0 && ni > 0) {
-    if (d * parts > tp_ctx::kPartialFloats || ni < 8 * parts) e = launch_gemv<kResidual, 4, 4>(a, gemv_grid(ctx, ni), o.stream);
+    if (d * parts > WorkspacePool::kPartialFloats || ni < 8 * parts) e = launch_gemv<kResidual, 4, 4>(a, gemv_grid(ctx, ni), o.stream);
     else {
       const int64_t slice = ((ni / 8 + parts - 1) / parts) * 8 + 8;
       const size_t smem = (size_t)((slice + 3) & ~int64_t(3)) * sizeof(float);
       constexpr auto k = gemv_partial_kernel<8>;
+      s = o.partial(&partial);
+      if (s != TP_OK) {
+        o.abort();
+        return s;
+      }
       e = smem > (size_t)kSmemOptin ? cudaErrorInvalidValue : allow_smem<k>(kSmemOptin);
       if (e == cudaSuccess) {
         const int grid = ctx->sm_count * 4;  // a multiple of `parts` on every GB300 SM count used (152)
-        k<<<(grid / parts) * parts, kThreads, smem, o.stream>>>(a, parts, ctx->d_partial);
+        k<<<(grid / parts) * parts, kThreads, smem, o.stream>>>(a, parts, partial);
         const unsigned fg = (unsigned)((d + kThreads - 1) / kThreads);
         if (a.counts)
-          residual_finish_kernel<true><<<fg, kThreads, 0, o.stream>>>(a.y, ctx->d_partial, d, parts, a.counts, a.owner);
+          residual_finish_kernel<true><<<fg, kThreads, 0, o.stream>>>(a.y, partial, d, parts, a.counts, a.owner);
         else
-          residual_finish_kernel<false><<<fg, kThreads, 0, o.stream>>>(a.y, ctx->d_partial, d, parts, nullptr, nullptr);
+          residual_finish_kernel<false><<<fg, kThreads, 0, o.stream>>>(a.y, partial, d, parts, nullptr, nullptr);
         e = cudaGetLastError();
       }
     }

@@ -60,24 +60,33 @@ struct Workspace {
   // moves nothing to report so.
   int* err = nullptr;
 };
+// A device buffer of kPartialFloats for matrix-vector partial sums, kept by
+// what may still use it: the operation being launched, the event that it is
+// recorded into, its graph.
+using Partial = std::shared_ptr<float>;
 
 // Workspaces of a context: lent to a SYNC operation for the call, to an event
 // and to a graph until it is gone and the work recorded into it has ended. It
 // grows by blocks as more are out at a time. The last holder (the context, its
-// events, its graphs) frees them, so that events and graphs may be destroyed
-// after their context.
-class WorkspacePool {
+// events, its graphs) frees the words, so that events and graphs may be
+// destroyed after their context; buffers on the device go with the context.
+class WorkspacePool : public std::enable_shared_from_this<WorkspacePool> {
  public:
   ~WorkspacePool();
   cudaError_t take(Workspace** out);
   void give(Workspace* w);
-  std::atomic<bool> closed{false};  // the context is gone
+  cudaError_t partial(Partial* out);
+  void close();                     // the context goes, with no work in flight
+  std::atomic<bool> closed{false};
+  static constexpr int64_t kPartialFloats = int64_t(1) << 20;
  private:
   static constexpr int kBlock = 4096;
   std::mutex mu_;
   std::deque<Workspace> all_;       // (a deque: their addresses stay)
   std::vector<Workspace*> free_;
   std::vector<int*> blocks_;        // error words, kBlock each
+  std::vector<float*> partials_;    // every buffer of partial sums, and the idle ones
+  std::vector<float*> free_partials_;
 };
 }  // namespace tp
 
@@ -96,13 +105,11 @@ struct tp_ctx {
   // Device workspace, allocated once at creation.
   unsigned* d_queue = nullptr;      // tile-queue counters (kQueueSlots)
   float* d_scratch = nullptr;       // small float scratch (kScratchFloats)
-  float* d_partial = nullptr;       // matrix-vector partial sums (kPartialFloats)
   uint32_t* d_claims = nullptr;     // tile-claim bitmap of checked launches (kClaimBits), all clear
   unsigned* d_claim_done = nullptr; // CTAs of the running checked launch that finished
   std::atomic<uint32_t> queue_slot{0};
   static constexpr int kQueueSlots = 256;
   static constexpr int kScratchFloats = 4096;
-  static constexpr int64_t kPartialFloats = int64_t(1) << 20;
   static constexpr int64_t kClaimBits = int64_t(1) << 26;   // 8 MiB
 };
 
@@ -131,6 +138,7 @@ struct GraphRun {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool check_err = false;
+  Partial partial;                   // of its operations, which run one after another
 };
 }  // namespace tp
 
@@ -142,6 +150,7 @@ struct tp_event {
   bool check_err = false;
   cudaStream_t stream = nullptr;  // stream of the last record
   tp::Workspace* ws = nullptr;    // of the operations recorded into it
+  std::vector<tp::Partial> partials;  // that their work in flight uses
   std::vector<std::shared_ptr<tp::GraphRun>> replays;  // graphs replayed into it
   std::vector<tp::Hold> held;   // holds released when the event completes (appended per op)
 };
@@ -151,6 +160,7 @@ struct tp_graph {
   std::shared_ptr<tp::GraphRun> run;
   cudaStream_t stream = nullptr;
   bool ended = false;
+  bool uses_partial = false;         // a recorded operation does
   std::vector<tp_partition*> parts;  // partitions written by recorded nodes
 };
 
@@ -204,6 +214,7 @@ struct Op {
   bool check_err = false;   // kernel may write the error word
   int* err = nullptr;       // error word for this operation's kernels (set by begin)
   Workspace* lent = nullptr;  // SYNC: the operation's own workspace
+  Partial sums;             // its partial sums (partial())
   bool marked = false;
   bool allow_checked = false;  // the op implements TP_EXEC_CHECKED (set before begin)
   bool allow_inject = false;   // the op implements TP_EXEC_INJECT_TIMEOUT (set before begin)
@@ -220,6 +231,9 @@ struct Op {
   tp_status end_impl(cudaError_t launch_err);
   // Undo begin() after a failure that launched nothing (keeps the detail).
   void abort();
+  // A buffer of WorkspacePool::kPartialFloats that no work uses which may run
+  // beside this operation's.
+  tp_status partial(float** out);
   bool capturing() const { return ex->mode == TP_CAPTURE; }
 };
 

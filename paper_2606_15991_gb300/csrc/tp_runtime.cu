@@ -156,15 +156,20 @@ WorkspacePool::~WorkspacePool() {
   for (int* b : blocks_) cudaFreeHost(b);
 }
 
+// Allocations while this thread captures a stream (for work that is not
+// recorded) are allowed.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 cudaError_t WorkspacePool::take(Workspace** out) {
   std::lock_guard<std::mutex> lk(mu_);
   if (free_.empty()) {
-    // allowed while this thread captures, as nothing of it is recorded
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
+    RelaxedCapture relaxed;
     int* words = nullptr;
     const cudaError_t e = cudaMallocHost(&words, sizeof(int) * kBlock);
-    cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) return e;
     blocks_.push_back(words);
     for (int i = 0; i < kBlock; ++i) {
@@ -182,6 +187,32 @@ void WorkspacePool::give(Workspace* w) {
   if (!w) return;
   std::lock_guard<std::mutex> lk(mu_);
   free_.push_back(w);
+}
+
+cudaError_t WorkspacePool::partial(Partial* out) {
+  std::lock_guard<std::mutex> lk(mu_);
+  if (free_partials_.empty()) {
+    RelaxedCapture relaxed;
+    float* p = nullptr;
+    const cudaError_t e = cudaMalloc(&p, sizeof(float) * kPartialFloats);
+    if (e != cudaSuccess) return e;
+    partials_.push_back(p);
+    free_partials_.push_back(p);
+  }
+  *out = Partial(free_partials_.back(), [pool = shared_from_this()](float* p) {
+    std::lock_guard<std::mutex> lk(pool->mu_);
+    if (!pool->closed) pool->free_partials_.push_back(p);
+  });
+  free_partials_.pop_back();
+  return cudaSuccess;
+}
+
+void WorkspacePool::close() {
+  std::lock_guard<std::mutex> lk(mu_);
+  closed = true;
+  for (float* p : partials_) cudaFree(p);
+  partials_.clear();
+  free_partials_.clear();
 }
 
 GraphRun::~GraphRun() {
@@ -331,6 +362,26 @@ tp_status Op::begin_impl(tp_ctx* c, const tp_exec* e, const std::vector<tp_parti
   return TP_OK;
 }
 
+tp_status Op::partial(float** out) {
+  if (ex->mode == TP_CAPTURE) {
+    ctx->capturing->uses_partial = true;  // (tp_graph_begin took it)
+    sums = ctx->capturing->run->partial;
+  } else if (ex->mode == TP_ASYNC) {
+    // one of the event's, whose work runs before this on the same stream,
+    // unless a launch of another thread is about to use it
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    for (auto& p : ex->event->partials)
+      if (p.use_count() == 1) {
+        sums = p;
+        break;
+      }
+  }
+  cudaError_t e = sums ? cudaSuccess : ctx->pool->partial(&sums);
+  if (e != cudaSuccess) return cuda_fail(e, "allocating partial sums");
+  *out = sums.get();
+  return TP_OK;
+}
+
 void Op::abort() {
   if (marked) release(ctx, outs, stream);
   marked = false;
@@ -370,6 +421,9 @@ tp_status Op::end_impl(cudaError_t launch_err) {
   ev->recorded = true;
   ev->stream = stream;
   ev->check_err |= check_err;
+  if (sums && std::find(ev->partials.begin(), ev->partials.end(), sums) == ev->partials.end())
+    ev->partials.push_back(std::move(sums));
+  sums.reset();
   for (auto* p : outs) ev->held.push_back({p, stream, 1});
   return TP_OK;
 }
@@ -430,9 +484,11 @@ tp_status tp_ctx_create(int32_t device, tp_ctx** out) {
   }
   c->pool = std::make_shared<WorkspacePool>();
   e = c->pool->take(&c->own);
+  Partial first;  // (allocated here, ahead of its use)
+  if (e == cudaSuccess) e = c->pool->partial(&first);
+  first.reset();
   if (e == cudaSuccess) e = cudaMalloc(&c->d_queue, sizeof(unsigned) * tp_ctx::kQueueSlots);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_scratch, sizeof(float) * tp_ctx::kScratchFloats);
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_partial, sizeof(float) * tp_ctx::kPartialFloats);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_claims, (size_t)tp_ctx::kClaimBits / 8);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_claim_done, 256);
   if (e == cudaSuccess) e = cudaMemset(c->d_claims, 0, (size_t)tp_ctx::kClaimBits / 8);
@@ -441,9 +497,9 @@ tp_status tp_ctx_create(int32_t device, tp_ctx** out) {
   if (e != cudaSuccess) {
     cudaFree(c->d_queue);
     cudaFree(c->d_scratch);
-    cudaFree(c->d_partial);
     cudaFree(c->d_claims);
     cudaFree(c->d_claim_done);
+    c->pool->close();
     delete c;
     return cuda_fail(e, "allocating context workspace");
   }
@@ -458,14 +514,13 @@ tp_status tp_ctx_destroy(tp_ctx* ctx) {
     if (!ctx->busy.empty()) return fail(TP_ERR_BUSY, "context still has work in flight");
     if (ctx->capturing) return fail(TP_ERR_BUSY, "context is capturing a graph");
   }
-  ctx->pool->closed = true;
   // the frees wait for the device, so no kernel is left that could still write
   // an error word
   cudaFree(ctx->d_queue);
   cudaFree(ctx->d_scratch);
-  cudaFree(ctx->d_partial);
   cudaFree(ctx->d_claims);
   cudaFree(ctx->d_claim_done);
+  ctx->pool->close();
   delete ctx;
   return TP_OK;
 }
@@ -614,12 +669,14 @@ static tp_status event_complete(tp_event* ev) {
   const bool open = !ev->pool->closed;  // (a context that is gone holds nothing)
   std::vector<Hold> held;
   std::vector<std::shared_ptr<GraphRun>> replays;
+  std::vector<Partial> partials;
   bool chk;
   {
     std::unique_lock<std::mutex> lk;
     if (open) lk = std::unique_lock<std::mutex>(ev->ctx->mu);
     held.swap(ev->held);
     replays.swap(ev->replays);
+    partials.swap(ev->partials);
     chk = ev->check_err;
     ev->check_err = false;
     ev->recorded = false;
@@ -704,7 +761,9 @@ tp_status tp_graph_begin(tp_ctx* ctx, void* stream, tp_graph** out) {
   g->ctx = ctx;
   g->stream = static_cast<cudaStream_t>(stream);
   g->run = std::make_shared<GraphRun>(ctx->pool);
+  // nothing may be allocated while operations are recorded
   cudaError_t e = ctx->pool->take(&g->run->ws);
+  if (e == cudaSuccess) e = ctx->pool->partial(&g->run->partial);
   if (e != cudaSuccess) {
     delete g;
     return cuda_fail(e, "allocating graph workspaces");
@@ -727,6 +786,7 @@ tp_status tp_graph_end(tp_graph* g) {
     g->ctx->capturing = nullptr;
   }
   g->ended = true;
+  if (!g->uses_partial) g->run->partial.reset();
   cudaError_t e = cudaStreamEndCapture(g->stream, &g->run->graph);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
   e = cudaGraphInstantiate(&g->run->exec, g->run->graph, 0);

@@ -350,3 +350,41 @@ def test_gemv_unit_shapes_within_summation_bound(ctx, rows, k, pitch):
     tp.tp_decode_down_residual(ctx, p, w, x)
     assert np.all(np.abs(_f(h) - (h0 + ref)) <= bound + 2 * U32 * (np.abs(h0) + np.abs(ref) + bound))
     tp.tp_partition_destroy(p)
+
+
+def test_down_projections_in_flight_together(ctx):
+    """Down projections over K slices (two kernels and a buffer of partial sums
+    between them) on two streams, and a graph of one on a third, each on its own
+    h: every result is the one that the product gives alone."""
+    d, ni, rounds = 512, 16384, 20
+    ws = [_w(d, ni, 60 + i) for i in range(3)]
+    xs = [_vec(ni, 70 + i) for i in range(3)]
+    hs = [torch.zeros(d, device="cuda") for _ in range(3)]
+    ps = [tp.tp_partition_create(ctx, h, (d,)) for h in hs]
+    want = []
+    for w, x, h, p in zip(ws, xs, hs, ps):
+        for _ in range(rounds):
+            tp.tp_decode_down_residual(ctx, p, w, x)
+        want.append(h.clone())
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    g = tp.tp_graph_begin(ctx, streams[2])
+    tp.tp_decode_down_residual(ctx, ps[2], ws[2], xs[2], tp.make_exec(tp.CAPTURE, streams[2]))
+    tp.tp_graph_end(g)
+    evs = [tp.tp_event_create(ctx) for _ in range(3)]
+    for _ in range(3):
+        for h in hs:
+            h.zero_()
+        torch.cuda.synchronize()
+        for _ in range(rounds):
+            for i in range(2):
+                tp.tp_decode_down_residual(ctx, ps[i], ws[i], xs[i], tp.make_exec(tp.ASYNC, streams[i], evs[i]))
+            tp.tp_graph_replay(g, tp.make_exec(tp.ASYNC, streams[2], evs[2]))
+        for ev in evs:
+            tp.tp_event_wait(ev)
+        for h, r in zip(hs, want):
+            assert torch.equal(h, r)
+    for ev in evs:
+        tp.tp_event_destroy(ev)
+    tp.tp_graph_destroy(g)
+    for p in ps:
+        tp.tp_partition_destroy(p)

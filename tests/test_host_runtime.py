@@ -36,6 +36,8 @@ def host(host_path, monkeypatch):
         f = getattr(L, name)
         f.argtypes, f.restype = args, _lib._RESTYPES.get(name, ctypes.c_int32)
     monkeypatch.setattr(_lib, "_lib", L)
+    for which in (0, 1):
+        L.fake_workspaces(which, None, ctypes.c_int64(0))
     yield L
     L.fake_finish()
 
@@ -157,3 +159,45 @@ assert L.fake_hosts() == 0
 """
     subprocess.run([sys.executable, "-c", child], check=True, timeout=120,
                    env={**os.environ, "MALLOC_PERTURB_": "165"})
+
+
+def _down(ctx, h, p, ex, ni=16384):
+    """A down projection over K slices: partial sums, and a finish kernel."""
+    tp.tp_decode_down_residual(ctx, p, torch.zeros(h.numel(), ni, dtype=torch.bfloat16), torch.zeros(ni), ex)
+
+
+def _addresses(host, which):
+    out = (ctypes.c_uint64 * 4096)()
+    n = host.fake_workspaces(which, out, ctypes.c_int64(4096))
+    return list(out[:n])
+
+
+def test_partial_sums_of_work_in_flight_do_not_share_a_buffer(host):
+    ctx = tp.tp_ctx_create(0)
+    hs = [torch.zeros(64) for _ in range(4)]
+    ps = [tp.tp_partition_create(ctx, h, (64,)) for h in hs]
+    g = tp.tp_graph_begin(ctx, S1)
+    for _ in range(2):
+        _down(ctx, hs[0], ps[0], _exec(tp.CAPTURE, S1))
+    tp.tp_graph_end(g)
+    graph = set(_addresses(host, 0))
+    assert len(graph) == 1
+    evs = [tp.tp_event_create(ctx) for _ in range(3)]
+    seen = set()
+    for _ in range(50):
+        tp.tp_graph_replay(g, _exec(tp.ASYNC, S1, evs[0]))
+        for i in (1, 2):
+            _down(ctx, hs[i], ps[i], _exec(tp.ASYNC, S2 + i, evs[i]))
+        _down(ctx, hs[3], ps[3], _exec(tp.SYNC, S2))
+        now = _addresses(host, 0)
+        assert len(set(now)) == 3 and not graph & set(now)
+        seen |= set(now)
+        for ev in evs:
+            tp.tp_event_wait(ev)
+    assert len(seen) == 3   # reused, not one for each operation
+    for ev in evs:
+        tp.tp_event_destroy(ev)
+    tp.tp_graph_destroy(g)
+    for p in ps:
+        tp.tp_partition_destroy(p)
+    tp.tp_ctx_destroy(ctx)
