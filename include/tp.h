@@ -234,7 +234,8 @@ tp_status tp_version(int32_t* major, int32_t* minor);
 /* --------------------------------------------------------------- context */
 /* Creates a context on CUDA device `device` (§3.2 ExecutionContext: device,
  * stream and memory pool). Allocates the context's device workspace (error
- * word, queue counters, scale scratch) once, so later calls can be captured.
+ * words, queue counters, partial sums, scale scratch), so later calls can be
+ * captured; more of them only as more work is in flight at a time.
  * Errors: TP_ERR_INVALID (null out), TP_ERR_CUDA (no such device / no sm_103). */
 tp_status tp_ctx_create(int32_t device, tp_ctx** out);
 /* Frees the context and its workspace. TP_ERR_BUSY if work is still in flight.

@@ -824,7 +824,7 @@ tp_status tp_grouped_gemm(tp_ctx* ctx, tp_grouped_plan* plan, int32_t num_progra
   if (s != TP_OK) return s;
   o.check_err = true;
   unsigned* q = nullptr;
-  s = queue_counter(ctx, o.stream, &q);
+  s = o.queue(&q);
   if (s != TP_OK) {
     o.abort();
     return s;

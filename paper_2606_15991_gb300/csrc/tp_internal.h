@@ -60,10 +60,14 @@ struct Workspace {
   // moves nothing to report so.
   int* err = nullptr;
 };
-// A device buffer of kPartialFloats for matrix-vector partial sums, kept by
-// what may still use it: the operation being launched, the event that it is
-// recorded into, its graph.
-using Partial = std::shared_ptr<float>;
+// Device memory, kept by what may still use it: the operation being launched,
+// the event that it is recorded into, its graph.
+using Partial = std::shared_ptr<float>;      // matrix-vector partial sums (kPartialFloats)
+using Counter = std::shared_ptr<unsigned>;   // of a tile queue
+struct Scratch {
+  std::vector<Partial> partials;
+  std::vector<Counter> counters;
+};
 
 // Workspaces of a context: lent to a SYNC operation for the call, to an event
 // and to a graph until it is gone and the work recorded into it has ended. It
@@ -75,7 +79,8 @@ class WorkspacePool : public std::enable_shared_from_this<WorkspacePool> {
   ~WorkspacePool();
   cudaError_t take(Workspace** out);
   void give(Workspace* w);
-  cudaError_t partial(Partial* out);
+  cudaError_t get(Partial* out);
+  cudaError_t get(Counter* out);
   void close();                     // the context goes, with no work in flight
   std::atomic<bool> closed{false};
   static constexpr int64_t kPartialFloats = int64_t(1) << 20;
@@ -87,6 +92,8 @@ class WorkspacePool : public std::enable_shared_from_this<WorkspacePool> {
   std::vector<int*> blocks_;        // error words, kBlock each
   std::vector<float*> partials_;    // every buffer of partial sums, and the idle ones
   std::vector<float*> free_partials_;
+  std::vector<unsigned*> counter_blocks_;  // kBlock each
+  std::vector<unsigned*> free_counters_;
 };
 }  // namespace tp
 
@@ -103,12 +110,9 @@ struct tp_ctx {
   std::shared_ptr<tp::WorkspacePool> pool;
   tp::Workspace* own = nullptr;     // of launches that no operation reports for
   // Device workspace, allocated once at creation.
-  unsigned* d_queue = nullptr;      // tile-queue counters (kQueueSlots)
   float* d_scratch = nullptr;       // small float scratch (kScratchFloats)
   uint32_t* d_claims = nullptr;     // tile-claim bitmap of checked launches (kClaimBits), all clear
   unsigned* d_claim_done = nullptr; // CTAs of the running checked launch that finished
-  std::atomic<uint32_t> queue_slot{0};
-  static constexpr int kQueueSlots = 256;
   static constexpr int kScratchFloats = 4096;
   static constexpr int64_t kClaimBits = int64_t(1) << 26;   // 8 MiB
 };
@@ -138,7 +142,7 @@ struct GraphRun {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool check_err = false;
-  Partial partial;                   // of its operations, which run one after another
+  Scratch scratch;
 };
 }  // namespace tp
 
@@ -150,7 +154,7 @@ struct tp_event {
   bool check_err = false;
   cudaStream_t stream = nullptr;  // stream of the last record
   tp::Workspace* ws = nullptr;    // of the operations recorded into it
-  std::vector<tp::Partial> partials;  // that their work in flight uses
+  tp::Scratch scratch;            // that their work in flight uses
   std::vector<std::shared_ptr<tp::GraphRun>> replays;  // graphs replayed into it
   std::vector<tp::Hold> held;   // holds released when the event completes (appended per op)
 };
@@ -214,7 +218,8 @@ struct Op {
   bool check_err = false;   // kernel may write the error word
   int* err = nullptr;       // error word for this operation's kernels (set by begin)
   Workspace* lent = nullptr;  // SYNC: the operation's own workspace
-  Partial sums;             // its partial sums (partial())
+  Partial sums;             // device memory of its own (partial(), queue())
+  Counter counter;
   bool marked = false;
   bool allow_checked = false;  // the op implements TP_EXEC_CHECKED (set before begin)
   bool allow_inject = false;   // the op implements TP_EXEC_INJECT_TIMEOUT (set before begin)
@@ -234,6 +239,9 @@ struct Op {
   // A buffer of WorkspacePool::kPartialFloats that no work uses which may run
   // beside this operation's.
   tp_status partial(float** out);
+  // Likewise a tile-queue counter, zeroed on the operation's stream.
+  tp_status queue(unsigned** out);
+  void keep_scratch();  // hands both to the event or graph (ctx->mu held)
   bool capturing() const { return ex->mode == TP_CAPTURE; }
 };
 
@@ -265,8 +273,6 @@ tp_status event_claim(tp_event* ev, cudaStream_t stream);
 // The context's tile-claim bitmap for one checked launch (TP_EXEC_CHECKED)
 // that may set up to `bits` bits; the launch's last CTA clears them again.
 tp_status claims_for(tp_ctx* ctx, int64_t bits, uint32_t** claims, unsigned** done);
-// Reserve a tile-queue counter for one launch and zero it on `stream`.
-tp_status queue_counter(tp_ctx* ctx, cudaStream_t stream, unsigned** out);
 
 // Kernel launchers (defined in the kernel translation units).
 enum MapOp : int { kMapAxpy = 0, kMapGeluMul = 1, kMapScale = 2, kMapAddAccum = 3 };

@@ -189,7 +189,7 @@ void WorkspacePool::give(Workspace* w) {
   free_.push_back(w);
 }
 
-cudaError_t WorkspacePool::partial(Partial* out) {
+cudaError_t WorkspacePool::get(Partial* out) {
   std::lock_guard<std::mutex> lk(mu_);
   if (free_partials_.empty()) {
     RelaxedCapture relaxed;
@@ -207,12 +207,33 @@ cudaError_t WorkspacePool::partial(Partial* out) {
   return cudaSuccess;
 }
 
+cudaError_t WorkspacePool::get(Counter* out) {
+  std::lock_guard<std::mutex> lk(mu_);
+  if (free_counters_.empty()) {
+    RelaxedCapture relaxed;
+    unsigned* p = nullptr;
+    const cudaError_t e = cudaMalloc(&p, sizeof(unsigned) * kBlock);
+    if (e != cudaSuccess) return e;
+    counter_blocks_.push_back(p);
+    for (int i = 0; i < kBlock; ++i) free_counters_.push_back(p + i);
+  }
+  *out = Counter(free_counters_.back(), [pool = shared_from_this()](unsigned* p) {
+    std::lock_guard<std::mutex> lk(pool->mu_);
+    if (!pool->closed) pool->free_counters_.push_back(p);
+  });
+  free_counters_.pop_back();
+  return cudaSuccess;
+}
+
 void WorkspacePool::close() {
   std::lock_guard<std::mutex> lk(mu_);
   closed = true;
   for (float* p : partials_) cudaFree(p);
+  for (unsigned* p : counter_blocks_) cudaFree(p);
   partials_.clear();
   free_partials_.clear();
+  counter_blocks_.clear();
+  free_counters_.clear();
 }
 
 GraphRun::~GraphRun() {
@@ -225,15 +246,6 @@ tp_status claims_for(tp_ctx* ctx, int64_t bits, uint32_t** claims, unsigned** do
   if (bits > tp_ctx::kClaimBits) return fail(TP_ERR_UNSUPPORTED, "too many tiles for a checked launch");
   *claims = ctx->d_claims;
   *done = ctx->d_claim_done;
-  return TP_OK;
-}
-
-tp_status queue_counter(tp_ctx* ctx, cudaStream_t stream, unsigned** out) {
-  uint32_t slot = ctx->queue_slot.fetch_add(1) % tp_ctx::kQueueSlots;
-  unsigned* q = ctx->d_queue + slot;
-  cudaError_t e = cudaMemsetAsync(q, 0, sizeof(unsigned), stream);
-  if (e != cudaSuccess) return cuda_fail(e, "resetting tile-queue counter");
-  *out = q;
   return TP_OK;
 }
 
@@ -362,27 +374,63 @@ tp_status Op::begin_impl(tp_ctx* c, const tp_exec* e, const std::vector<tp_parti
   return TP_OK;
 }
 
+// One of the event's or graph's, whose work runs before this operation's on the
+// same stream, unless a launch of another thread is about to use it.
+template <typename P>
+static P idle(const std::vector<P>& v) {
+  for (const P& p : v)
+    if (p.use_count() == 1) return p;
+  return nullptr;
+}
+
+template <typename P>
+static void keep(std::vector<P>* v, const P& p) {
+  if (p && std::find(v->begin(), v->end(), p) == v->end()) v->push_back(p);
+}
+
 tp_status Op::partial(float** out) {
-  if (ex->mode == TP_CAPTURE) {
-    ctx->capturing->uses_partial = true;  // (tp_graph_begin took it)
-    sums = ctx->capturing->run->partial;
-  } else if (ex->mode == TP_ASYNC) {
-    // one of the event's, whose work runs before this on the same stream,
-    // unless a launch of another thread is about to use it
+  if (!lent) {
     std::lock_guard<std::mutex> lk(ctx->mu);
-    for (auto& p : ex->event->partials)
-      if (p.use_count() == 1) {
-        sums = p;
-        break;
-      }
+    if (capturing()) ctx->capturing->uses_partial = true;
+    sums = idle(capturing() ? ctx->capturing->run->scratch.partials : ex->event->scratch.partials);
   }
-  cudaError_t e = sums ? cudaSuccess : ctx->pool->partial(&sums);
+  const cudaError_t e = sums ? cudaSuccess : ctx->pool->get(&sums);
   if (e != cudaSuccess) return cuda_fail(e, "allocating partial sums");
   *out = sums.get();
   return TP_OK;
 }
 
+tp_status Op::queue(unsigned** out) {
+  if (!lent) {
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    counter = idle(capturing() ? ctx->capturing->run->scratch.counters : ex->event->scratch.counters);
+  }
+  cudaError_t e = counter ? cudaSuccess : ctx->pool->get(&counter);
+  if (e != cudaSuccess) return cuda_fail(e, "allocating tile-queue counters");
+  e = cudaMemsetAsync(counter.get(), 0, sizeof(unsigned), stream);
+  if (e != cudaSuccess) return cuda_fail(e, "resetting tile-queue counter");
+  *out = counter.get();
+  return TP_OK;
+}
+
+void Op::keep_scratch() {
+  Scratch& to = capturing() ? ctx->capturing->run->scratch : ex->event->scratch;
+  keep(&to.partials, sums);
+  keep(&to.counters, counter);
+  sums.reset();
+  counter.reset();
+}
+
 void Op::abort() {
+  if (counter) {
+    // its reset is enqueued, or recorded
+    if (capturing()) {
+      std::lock_guard<std::mutex> lk(ctx->mu);
+      keep_scratch();
+    } else {
+      cudaStreamSynchronize(stream);
+    }
+  }
   if (marked) release(ctx, outs, stream);
   marked = false;
   trace(*this, "aborted", TP_ERR_INVALID);
@@ -396,13 +444,21 @@ tp_status Op::end(cudaError_t launch_err) {
 
 tp_status Op::end_impl(cudaError_t launch_err) {
   if (launch_err != cudaSuccess) {
-    // kernels launched before the one that failed may still report
-    if (ex->mode != TP_CAPTURE) cudaStreamSynchronize(stream);
+    // what was enqueued, or recorded, before the failure still uses its words
+    // and scratch
+    if (capturing()) {
+      std::lock_guard<std::mutex> lk(ctx->mu);
+      keep_scratch();
+    } else {
+      cudaStreamSynchronize(stream);
+    }
     if (marked) release(ctx, outs, stream);
     return cuda_fail(launch_err, "kernel launch");
   }
   if (ex->mode == TP_CAPTURE) {
     if (check_err) ctx->capturing->run->check_err = true;
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    keep_scratch();
     return TP_OK;
   }
   if (ex->mode == TP_SYNC) {
@@ -414,6 +470,7 @@ tp_status Op::end_impl(cudaError_t launch_err) {
   tp_event* ev = ex->event;
   const cudaError_t e = cudaEventRecord(ev->ev, stream);
   if (e != cudaSuccess) {
+    cudaStreamSynchronize(stream);
     release(ctx, outs, stream);
     return cuda_fail(e, "cudaEventRecord");
   }
@@ -421,9 +478,7 @@ tp_status Op::end_impl(cudaError_t launch_err) {
   ev->recorded = true;
   ev->stream = stream;
   ev->check_err |= check_err;
-  if (sums && std::find(ev->partials.begin(), ev->partials.end(), sums) == ev->partials.end())
-    ev->partials.push_back(std::move(sums));
-  sums.reset();
+  keep_scratch();
   for (auto* p : outs) ev->held.push_back({p, stream, 1});
   return TP_OK;
 }
@@ -484,18 +539,18 @@ tp_status tp_ctx_create(int32_t device, tp_ctx** out) {
   }
   c->pool = std::make_shared<WorkspacePool>();
   e = c->pool->take(&c->own);
-  Partial first;  // (allocated here, ahead of its use)
-  if (e == cudaSuccess) e = c->pool->partial(&first);
-  first.reset();
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_queue, sizeof(unsigned) * tp_ctx::kQueueSlots);
+  {
+    Partial first;  // (allocated here, ahead of their use)
+    Counter counters;
+    if (e == cudaSuccess) e = c->pool->get(&first);
+    if (e == cudaSuccess) e = c->pool->get(&counters);
+  }
   if (e == cudaSuccess) e = cudaMalloc(&c->d_scratch, sizeof(float) * tp_ctx::kScratchFloats);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_claims, (size_t)tp_ctx::kClaimBits / 8);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_claim_done, 256);
   if (e == cudaSuccess) e = cudaMemset(c->d_claims, 0, (size_t)tp_ctx::kClaimBits / 8);
   if (e == cudaSuccess) e = cudaMemset(c->d_claim_done, 0, 256);
-  if (e == cudaSuccess) e = cudaMemset(c->d_queue, 0, sizeof(unsigned) * tp_ctx::kQueueSlots);
   if (e != cudaSuccess) {
-    cudaFree(c->d_queue);
     cudaFree(c->d_scratch);
     cudaFree(c->d_claims);
     cudaFree(c->d_claim_done);
@@ -516,7 +571,6 @@ tp_status tp_ctx_destroy(tp_ctx* ctx) {
   }
   // the frees wait for the device, so no kernel is left that could still write
   // an error word
-  cudaFree(ctx->d_queue);
   cudaFree(ctx->d_scratch);
   cudaFree(ctx->d_claims);
   cudaFree(ctx->d_claim_done);
@@ -669,14 +723,14 @@ static tp_status event_complete(tp_event* ev) {
   const bool open = !ev->pool->closed;  // (a context that is gone holds nothing)
   std::vector<Hold> held;
   std::vector<std::shared_ptr<GraphRun>> replays;
-  std::vector<Partial> partials;
+  Scratch scratch;
   bool chk;
   {
     std::unique_lock<std::mutex> lk;
     if (open) lk = std::unique_lock<std::mutex>(ev->ctx->mu);
     held.swap(ev->held);
     replays.swap(ev->replays);
-    partials.swap(ev->partials);
+    std::swap(scratch, ev->scratch);
     chk = ev->check_err;
     ev->check_err = false;
     ev->recorded = false;
@@ -763,7 +817,11 @@ tp_status tp_graph_begin(tp_ctx* ctx, void* stream, tp_graph** out) {
   g->run = std::make_shared<GraphRun>(ctx->pool);
   // nothing may be allocated while operations are recorded
   cudaError_t e = ctx->pool->take(&g->run->ws);
-  if (e == cudaSuccess) e = ctx->pool->partial(&g->run->partial);
+  Scratch& scratch = g->run->scratch;
+  scratch.partials.resize(1);
+  scratch.counters.resize(1);
+  if (e == cudaSuccess) e = ctx->pool->get(&scratch.partials[0]);
+  if (e == cudaSuccess) e = ctx->pool->get(&scratch.counters[0]);
   if (e != cudaSuccess) {
     delete g;
     return cuda_fail(e, "allocating graph workspaces");
@@ -786,7 +844,7 @@ tp_status tp_graph_end(tp_graph* g) {
     g->ctx->capturing = nullptr;
   }
   g->ended = true;
-  if (!g->uses_partial) g->run->partial.reset();
+  if (!g->uses_partial) g->run->scratch.partials.clear();
   cudaError_t e = cudaStreamEndCapture(g->stream, &g->run->graph);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
   e = cudaGraphInstantiate(&g->run->exec, g->run->graph, 0);
@@ -906,7 +964,7 @@ static tp_status map_op(tp_ctx* ctx, tp_partition* out, int op, float alpha, con
   o.check_err = (ex->flags & TP_EXEC_CHECKED) != 0;
   unsigned* q = nullptr;
   if (out->kind == TP_MAP_QUEUE) {
-    s = queue_counter(ctx, o.stream, &q);
+    s = o.queue(&q);
     if (s != TP_OK) {
       o.abort();
       return s;
@@ -958,7 +1016,7 @@ tp_status tp_gemm(tp_ctx* ctx, tp_partition* c, const tp_tensor* a, const tp_ten
   if (s != TP_OK) return s;
   unsigned* q = nullptr;
   if (c->kind == TP_MAP_QUEUE) {
-    s = queue_counter(ctx, o.stream, &q);
+    s = o.queue(&q);
     if (s != TP_OK) {
       o.abort();
       return s;

@@ -201,3 +201,31 @@ def test_partial_sums_of_work_in_flight_do_not_share_a_buffer(host):
     for p in ps:
         tp.tp_partition_destroy(p)
     tp.tp_ctx_destroy(ctx)
+
+
+def test_tile_queues_of_work_in_flight_do_not_share_a_counter(host):
+    ctx = tp.tp_ctx_create(0)
+    x, z = torch.zeros(4096), [torch.zeros(4096) for _ in range(3)]
+    ps = [tp.tp_partition_create(ctx, t, (512,)) for t in z]
+    for p in ps:
+        tp.tp_partition_map(p, _lib.MAP_QUEUE, 3)
+
+    def run(i, ex):
+        tp.tp_map_scale(ctx, ps[i], x, x, ex)
+
+    g = tp.tp_graph_begin(ctx, S1)
+    run(0, _exec(tp.CAPTURE, S1))
+    tp.tp_graph_end(g)
+    graph = _addresses(host, 1)
+    ev = tp.tp_event_create(ctx)
+    for _ in range(600):
+        run(1, _exec(tp.ASYNC, S2, ev))
+        run(2, _exec(tp.SYNC, S1))
+        now = _addresses(host, 1)
+        assert len(now) == 2 and len(set(now + graph)) == 3
+        tp.tp_event_wait(ev)
+    tp.tp_event_destroy(ev)
+    tp.tp_graph_destroy(g)
+    for p in ps:
+        tp.tp_partition_destroy(p)
+    tp.tp_ctx_destroy(ctx)

@@ -434,3 +434,36 @@ def test_tile_groups_equal_one_tile(ctx, op, dt, kind, P, shape, tile):
         assert own.min() >= 0 and own.max() < P
     else:
         assert np.array_equal(own, opart.owner_map(shape, tile, P or None, kind).reshape(-1))
+
+
+def test_queue_maps_in_flight_together(ctx):
+    """A recorded queue map replayed while more queue maps than there were
+    counters run on another stream: each tile of each is run once (the maps add
+    to what is there)."""
+    n = 1 << 20
+    x, y = (t.reshape(-1) for t in _inputs(n, "f32")[:2])
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    outs = [torch.zeros(n, device="cuda") for _ in range(2)]
+    ps = [tp.tp_partition_create(ctx, o, (256,)) for o in outs]
+    for p in ps:
+        tp.tp_partition_map(p, tp.MAP_QUEUE, 8)
+    want = torch.zeros(n, device="cuda")
+    p = tp.tp_partition_create(ctx, want, (256,))
+    for _ in range(300):
+        tp.tp_map_add_accum(ctx, p, x, y)
+    tp.tp_partition_destroy(p)
+    g = tp.tp_graph_begin(ctx, s1)
+    tp.tp_map_add_accum(ctx, ps[0], x, y, tp.make_exec(tp.CAPTURE, s1))
+    tp.tp_graph_end(g)
+    evs = [tp.tp_event_create(ctx) for _ in range(2)]
+    torch.cuda.synchronize()
+    for _ in range(300):
+        tp.tp_graph_replay(g, tp.make_exec(tp.ASYNC, s1, evs[0]))
+        tp.tp_map_add_accum(ctx, ps[1], x, y, tp.make_exec(tp.ASYNC, s2, evs[1]))
+    for ev in evs:
+        tp.tp_event_wait(ev)
+        tp.tp_event_destroy(ev)
+    assert torch.equal(outs[0], want) and torch.equal(outs[1], want)
+    tp.tp_graph_destroy(g)
+    for p in ps:
+        tp.tp_partition_destroy(p)
