@@ -35,7 +35,8 @@ struct tp_mlp {
   float* v = nullptr;
   float* h1 = nullptr;      // [B, H] activations
   float* h2 = nullptr;
-  float* y = nullptr;       // [B, C] scores (propose)
+  float* y = nullptr;       // [B, C] scores (propose, and outputs that overlap X)
+  float* grads = nullptr;   // gradients whose output overlaps X
   float* dy = nullptr;      // [B, C] unscaled loss gradient
   float* dz1 = nullptr;     // [B, H]
   float* dz2 = nullptr;
@@ -249,10 +250,10 @@ struct GradsArgs {
   const float* part;  // rows_kernel's partial sums
   float* G;           // gradients out, or null
   float* loss;        // or null
-  float* P;           // Adam: parameters and moments
+  float* P;           // Adam: parameters and moments, or null: no step
   float* m;
   float* v;
-  float lr, c1, c2;   // lr = 0: no Adam step
+  float lr, c1, c2;
 };
 
 __device__ __forceinline__ void grad_out(const GradsArgs& a, int64_t i, float g) {
@@ -417,6 +418,13 @@ cudaError_t launch_rows(tp_mlp* n, const float* X, const float* T, const float* 
            : launch_pdl<rows_kernel<false>>(a, row_ctas(B), threads, smem, st);
 }
 
+// An output over the bytes of X: the kernels write outputs while other CTAs
+// read X, so it is written to the network's own buffer and copied out last.
+bool overlap(const float* out, size_t bytes, const float* x, size_t xbytes) {
+  const uintptr_t o = reinterpret_cast<uintptr_t>(out), i = reinterpret_cast<uintptr_t>(x);
+  return o < i + xbytes && i < o + bytes;
+}
+
 tp_status launch_forward(tp_mlp* n, const float* X, int B, float* Y, cudaStream_t st) {
   const cudaError_t e = launch_rows(n, X, nullptr, nullptr, B, Y, st);
   return e == cudaSuccess ? TP_OK : cuda_fail(e, "mlp forward");
@@ -485,7 +493,8 @@ tp_status tp_mlp_create(tp_ctx* ctx, int32_t in, int32_t hidden, int32_t out, in
   const size_t P = n->nparams * sizeof(float), BH = (size_t)max_batch * hidden * sizeof(float),
                BC = (size_t)max_batch * out * sizeof(float);
   cudaError_t e = cudaSuccess;
-  for (auto pr : {std::make_pair(&n->params, P), std::make_pair(&n->m, P), std::make_pair(&n->v, P),
+  for (auto pr : {std::make_pair(&n->params, P), std::make_pair(&n->grads, P), std::make_pair(&n->m, P),
+                  std::make_pair(&n->v, P),
                   std::make_pair(&n->h1, BH), std::make_pair(&n->h2, BH), std::make_pair(&n->y, BC),
                   std::make_pair(&n->dy, BC), std::make_pair(&n->dz1, BH), std::make_pair(&n->dz2, BH),
                   std::make_pair(&n->part, 2 * (size_t)row_ctas(max_batch) * sizeof(float)),
@@ -495,7 +504,7 @@ tp_status tp_mlp_create(tp_ctx* ctx, int32_t in, int32_t hidden, int32_t out, in
   if (e == cudaSuccess) e = cudaMemset(n->m, 0, P);
   if (e == cudaSuccess) e = cudaMemset(n->v, 0, P);
   if (e != cudaSuccess) {
-    for (float* p : {n->params, n->m, n->v, n->h1, n->h2, n->y, n->dy, n->dz1, n->dz2, n->part, n->xbuf}) cudaFree(p);
+    for (float* p : {n->params, n->grads, n->m, n->v, n->h1, n->h2, n->y, n->dy, n->dz1, n->dz2, n->part, n->xbuf}) cudaFree(p);
     delete n;
     return cuda_fail(e, "allocating the MLP");
   }
@@ -505,7 +514,7 @@ tp_status tp_mlp_create(tp_ctx* ctx, int32_t in, int32_t hidden, int32_t out, in
 
 tp_status tp_mlp_destroy(tp_mlp* n) {
   if (!n) return fail(TP_ERR_INVALID, "null mlp");
-  for (float* p : {n->params, n->m, n->v, n->h1, n->h2, n->y, n->dy, n->dz1, n->dz2, n->part, n->xbuf}) cudaFree(p);
+  for (float* p : {n->params, n->grads, n->m, n->v, n->h1, n->h2, n->y, n->dy, n->dz1, n->dz2, n->part, n->xbuf}) cudaFree(p);
   delete n;
   return TP_OK;
 }
@@ -538,10 +547,12 @@ tp_status tp_mlp_forward(tp_mlp* n, const float* X, int32_t batch, float* Y, con
   DeviceGuard guard(n->ctx);
   if (batch < 1 || batch > n->max_batch) return fail(TP_ERR_SHAPE, "batch must be 1..max_batch");
   cudaStream_t st = static_cast<cudaStream_t>(ex->stream);
-  tp_status s = launch_forward(n, X, batch, Y, st);
+  const size_t bytes = (size_t)batch * n->out * sizeof(float);
+  const bool over = overlap(Y, bytes, X, (size_t)batch * n->in * sizeof(float));
+  tp_status s = launch_forward(n, X, batch, over ? n->y : Y, st);
   if (s != TP_OK) return s;
-  cudaError_t e = cudaSuccess;
-  if (ex->mode == TP_SYNC) e = cudaStreamSynchronize(st);
+  cudaError_t e = over ? cudaMemcpyAsync(Y, n->y, bytes, cudaMemcpyDeviceToDevice, st) : cudaSuccess;
+  if (e == cudaSuccess && ex->mode == TP_SYNC) e = cudaStreamSynchronize(st);
   return e == cudaSuccess ? TP_OK : cuda_fail(e, "mlp forward output");
 }
 
@@ -551,10 +562,12 @@ tp_status tp_mlp_loss_grad(tp_mlp* n, const float* X, const float* T, const floa
   DeviceGuard guard(n->ctx);
   if (batch < 1 || batch > n->max_batch) return fail(TP_ERR_SHAPE, "batch must be 1..max_batch");
   cudaStream_t st = static_cast<cudaStream_t>(ex->stream);
-  tp_status s = launch_loss_grad(n, X, T, V, batch, loss, grads, 0, 0.f, st);
+  const size_t bytes = n->nparams * sizeof(float);
+  const bool over = grads && overlap(grads, bytes, X, (size_t)batch * n->in * sizeof(float));
+  tp_status s = launch_loss_grad(n, X, T, V, batch, loss, over ? n->grads : grads, 0, 0.f, st);
   if (s != TP_OK) return s;
-  cudaError_t e = cudaSuccess;
-  if (ex->mode == TP_SYNC) e = cudaStreamSynchronize(st);
+  cudaError_t e = over ? cudaMemcpyAsync(grads, n->grads, bytes, cudaMemcpyDeviceToDevice, st) : cudaSuccess;
+  if (e == cudaSuccess && ex->mode == TP_SYNC) e = cudaStreamSynchronize(st);
   return e == cudaSuccess ? TP_OK : cuda_fail(e, "mlp gradients");
 }
 

@@ -32,7 +32,7 @@ uint64_t issued = 0, finished = 0;
 cudaStream_t capturing = nullptr;
 Graph* recording = nullptr;
 int lowered = 0;
-std::vector<uint64_t> partials, queues;   // workspace addresses given to kernels, in launch order
+std::vector<uint64_t> seen[3];             // in order: partial sums given to kernels, counters reset, copies' targets
 int hosts = 0;                            // pinned allocations alive
 
 // (built on first use: kernels are registered by other files' initialisers)
@@ -58,7 +58,7 @@ cudaError_t launch(const void* f, void** args, size_t smem, cudaStream_t st) {
     w.word = *static_cast<int**>(args[0]);
     w.value = *static_cast<bool*>(args[2]) ? 0 : 1;
   }
-  if (n.find("residual_finish_kernel") != std::string::npos) partials.push_back(*static_cast<uint64_t*>(args[1]));
+  if (n.find("residual_finish_kernel") != std::string::npos) seen[0].push_back(*static_cast<uint64_t*>(args[1]));
   if (recording && st == capturing) recording->work.push_back(w);
   else {
     flying.push_back(w);
@@ -77,9 +77,9 @@ extern "C" {
 void fake_finish() { finish(); }
 int fake_lowered() { return lowered; }
 int fake_hosts() { return hosts; }
-int64_t fake_workspaces(int which, uint64_t* out, int64_t room) {
+int64_t fake_seen(int which, uint64_t* out, int64_t room) {
   std::lock_guard<std::recursive_mutex> lk(mu);
-  auto& v = which ? queues : partials;
+  auto& v = seen[which];
   const int64_t n = (int64_t)v.size();
   for (int64_t i = 0; i < n && i < room; ++i) out[i] = v[i];
   v.clear();
@@ -159,11 +159,15 @@ cudaError_t cudaFreeHost(void* p) {
   return cudaSuccess;
 }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { finish(); std::memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void* d, const void*, size_t, cudaMemcpyKind, cudaStream_t) {
+  std::lock_guard<std::recursive_mutex> lk(mu);
+  seen[2].push_back(reinterpret_cast<uint64_t>(d));
+  return cudaSuccess;
+}
 cudaError_t cudaMemset(void* d, int v, size_t n) { std::memset(d, v, n); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void* d, int, size_t n, cudaStream_t) {
   std::lock_guard<std::recursive_mutex> lk(mu);
-  if (n == sizeof(unsigned)) queues.push_back(reinterpret_cast<uint64_t>(d));
+  if (n == sizeof(unsigned)) seen[1].push_back(reinterpret_cast<uint64_t>(d));
   return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) { *p = nullptr; return cudaErrorInvalidSymbol; }

@@ -36,8 +36,8 @@ def host(host_path, monkeypatch):
         f = getattr(L, name)
         f.argtypes, f.restype = args, _lib._RESTYPES.get(name, ctypes.c_int32)
     monkeypatch.setattr(_lib, "_lib", L)
-    for which in (0, 1):
-        L.fake_workspaces(which, None, ctypes.c_int64(0))
+    for which in range(3):
+        L.fake_seen(which, None, ctypes.c_int64(0))
     yield L
     L.fake_finish()
 
@@ -168,7 +168,7 @@ def _down(ctx, h, p, ex, ni=16384):
 
 def _addresses(host, which):
     out = (ctypes.c_uint64 * 4096)()
-    n = host.fake_workspaces(which, out, ctypes.c_int64(4096))
+    n = host.fake_seen(which, out, ctypes.c_int64(4096))
     return list(out[:n])
 
 
@@ -228,4 +228,22 @@ def test_tile_queues_of_work_in_flight_do_not_share_a_counter(host):
     tp.tp_graph_destroy(g)
     for p in ps:
         tp.tp_partition_destroy(p)
+    tp.tp_ctx_destroy(ctx)
+
+
+def test_mlp_outputs_over_their_input_are_copied_out_last(host):
+    """An output that overlaps X is written when nothing reads X any more."""
+    f, h, c, b = 9, 8, 4, 6
+    ctx = tp.tp_ctx_create(0)
+    m = tp.tp_mlp_create(ctx, f, h, c, b, np.zeros(f * h + h * h + h * c + 2 * h + c, np.float32))
+    buf, t, loss = torch.zeros(400), torch.zeros(b, c), torch.zeros(1)
+    x = buf[:b * f].view(b, f)
+    for at in (0, 10, b * f - 1, b * f):
+        y = buf[at:]
+        want = [y.data_ptr()] if at < b * f else []
+        tp.tp_mlp_forward(m, x, y, _exec())
+        assert _addresses(host, 2) == want
+        tp.tp_mlp_loss_grad(m, x, t, t, loss, y, _exec())
+        assert _addresses(host, 2) == want
+    tp.tp_mlp_destroy(m)
     tp.tp_ctx_destroy(ctx)

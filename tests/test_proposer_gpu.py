@@ -383,3 +383,24 @@ def test_mlp_sizes_match_oracle(ctx, f, h, c, b):
     assert np.max(np.abs(got - want)[sure], initial=0.0) <= 2e-5
     assert np.max(np.abs(got - p0)) <= 1.01e-3
     tp.tp_mlp_destroy(m)
+
+
+def test_mlp_outputs_may_lie_over_their_input(ctx):
+    """Y and the gradients written over X are what they are elsewhere."""
+    f, h, c, b = 9, 40, 33, 300
+    m = tp.tp_mlp_create(ctx, f, h, c, b, proposer.init_params(f, h, c, seed=4))
+    n = tp.tp_mlp_num_params(m)
+    x0 = torch.from_numpy(synth.uniform(b * f, 5, 0, 4, dtype=np.float64).astype(np.float32)).cuda()
+    T = torch.rand(b, c, device="cuda")
+    V = torch.ones(b, c, device="cuda")
+    Y, G = torch.empty(b, c, device="cuda"), torch.empty(n, device="cuda")
+    tp.tp_mlp_forward(m, x0.view(b, f), Y)
+    tp.tp_mlp_loss_grad(m, x0.view(b, f), T, V, None, G)
+    for at in (0, 7, b * f - 1):
+        for call, want in ((lambda x, y: tp.tp_mlp_forward(m, x, y), Y.view(-1)),
+                           (lambda x, y: tp.tp_mlp_loss_grad(m, x, T, V, None, y), G)):
+            buf = torch.zeros(b * f + max(b * c, n), device="cuda")
+            buf[:b * f] = x0
+            call(buf[:b * f].view(b, f), buf[at:])
+            assert torch.equal(buf[at:at + want.numel()], want)
+    tp.tp_mlp_destroy(m)
