@@ -35,7 +35,8 @@ def nvcc() -> str:
 
 def _headers_digest() -> str:
     h = hashlib.sha256()
-    for p in sorted(glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))):
+    for p in sorted(glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) +
+                    glob.glob(os.path.join(INCLUDE, "*.h"))):
         h.update(open(p, "rb").read())
     h.update(" ".join(CFLAGS).encode())
     return h.hexdigest()[:16]

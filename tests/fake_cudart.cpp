@@ -33,6 +33,7 @@ cudaStream_t capturing = nullptr;
 Graph* recording = nullptr;
 int lowered = 0;
 std::vector<uint64_t> seen[3];             // in order: partial sums given to kernels, counters reset, copies' targets
+std::string last;                         // kernel launched last
 int hosts = 0;                            // pinned allocations alive
 
 // (built on first use: kernels are registered by other files' initialisers)
@@ -52,6 +53,7 @@ void finish() {
 cudaError_t launch(const void* f, void** args, size_t smem, cudaStream_t st) {
   std::lock_guard<std::recursive_mutex> lk(mu);
   const std::string& n = names()[f];
+  last = n;
   if (smem > 48 * 1024 && (!limits.count(f) || smem > (size_t)limits[f])) return cudaErrorInvalidValue;
   Work w;
   if (n.find("bounded_wait_kernel") != std::string::npos) {
@@ -77,6 +79,7 @@ extern "C" {
 void fake_finish() { finish(); }
 int fake_lowered() { return lowered; }
 int fake_hosts() { return hosts; }
+const char* fake_last_kernel() { return last.c_str(); }
 int64_t fake_seen(int which, uint64_t* out, int64_t room) {
   std::lock_guard<std::recursive_mutex> lk(mu);
   auto& v = seen[which];

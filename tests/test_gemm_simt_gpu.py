@@ -261,3 +261,27 @@ def test_split_products_of_two_sizes_from_two_threads(ctx):
     assert errors == []
     for m in ops:
         assert torch.equal(ops[m][2], want[m])
+
+
+@pytest.mark.parametrize("split", [1, 2, 4])
+def test_write_counts_of_every_operand_layout(ctx, split):
+    """Rows on 16-byte boundaries, off them, and transposed operands: each
+    element is written once, by its tile's program, and the counted launch
+    gives the uncounted one's bits."""
+    m, n, k = 130, 100, 72
+    a = torch.from_numpy(synth.uniform(m * k, seed=31)).reshape(m, k).cuda()
+    b = torch.from_numpy(synth.uniform(k * n, seed=32)).reshape(k, n).cuda()
+
+    def layouts(t):
+        yield t
+        off = torch.empty(t.numel() + 1, device="cuda")[1:].view(t.shape)
+        off.copy_(t)
+        yield off
+        yield t.t().contiguous().t()
+
+    for la in layouts(a):
+        for lb in layouts(b):
+            c, counts, owner = _gemm(ctx, la, lb, bk=32, split_k=split, count=True)
+            assert opart.check_counts(counts.cpu().numpy())["ok"]
+            assert np.array_equal(owner.cpu().numpy(), opart.gemm_owner_map(m, n, 64, 64))
+            assert torch.equal(c, _gemm(ctx, la, lb, bk=32, split_k=split)[0])

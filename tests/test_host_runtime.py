@@ -3,6 +3,7 @@
 import ctypes
 import glob
 import os
+import re
 import subprocess
 import sys
 
@@ -246,4 +247,39 @@ def test_mlp_outputs_over_their_input_are_copied_out_last(host):
         tp.tp_mlp_loss_grad(m, x, t, t, loss, y, _exec())
         assert _addresses(host, 2) == want
     tp.tp_mlp_destroy(m)
+    tp.tp_ctx_destroy(ctx)
+
+
+def test_counted_fp32_products_run_the_kernel_of_the_uncounted(host):
+    """Write counts are evidence for the kernel that the operands' layout picks."""
+    host.fake_last_kernel.restype = ctypes.c_char_p
+
+    def form():      # fetch of A, fetch of B, split
+        return re.search(rb"gemm_f32_kernelILi(\d)ELi(\d)ELb(\d)E", host.fake_last_kernel()).groups()
+
+    ctx = tp.tp_ctx_create(0)
+    m, n, k = 70, 66, 40
+    c = torch.zeros(m, n)
+    p = tp.tp_partition_create(ctx, c, (64, 64))
+    counts = torch.zeros(m * n, dtype=torch.int32)
+
+    def layouts(r, cols):
+        buf = torch.zeros(r * 80 + 8)
+        at = -buf.data_ptr() // 4 % 4
+        yield buf[at:].as_strided((r, cols), (80, 1))
+        yield buf[at + 1:].as_strided((r, cols), (80, 1))
+        yield torch.zeros(cols, r).t()
+
+    seen = set()
+    for split in (1, 2):
+        for a in layouts(m, k):
+            for b in layouts(k, n):
+                tp.tp_gemm(ctx, p, a, b, tp.gemm_config(split_k=split), _exec())
+                plain = form()
+                tp.tp_gemm(ctx, p, a, b, tp.gemm_config(split_k=split),
+                           tp.make_exec(stream=S1, write_counts=counts, write_owner=counts))
+                assert form() == plain
+                seen.add(plain)
+    assert len(seen) == 18
+    tp.tp_partition_destroy(p)
     tp.tp_ctx_destroy(ctx)
