@@ -1064,11 +1064,12 @@ tp_status tp_gemv(tp_ctx* ctx, tp_partition* y, const tp_tensor* w, const tp_ten
     // Streamed, but for matrices of a few boxes, where the stream's set-up
     // shows (32 x 64: 2.8 us streamed, 2.0 per lane; 1000 x 1000: 3.2 and
     // 3.6), for few rows that are not whole column blocks, whose units can't
-    // be cut below 16 rows (300 x 4104: 5.5 and 4.8), and for x that the bulk
-    // copies or shared memory cannot take.
+    // be cut below 16 rows (300 x 4104: 5.5 and 4.8), for x that the bulk
+    // copies or shared memory cannot take, and for rows that overlap (a view
+    // with a row stride below k), which a tensor map does not describe.
     StreamArgs sa = whole_x_args(ctx, a, kPlain);
     const bool few = k % kSCols != 0 && sa.units < ctx->sm_count / 4;
-    if (stream_ok(x) && whole_x_stages(k) > 0 && rows * k >= (int64_t(1) << 16) && !few) {
+    if (stream_ok(x) && whole_x_stages(k) > 0 && a.ld >= k && rows * k >= (int64_t(1) << 16) && !few) {
       o.check_err = true;  // its waits are bounded
       tp_status ls = launch_stream(ctx, sa, w, false, w, false, o.stream, o.err);
       if (ls != TP_OK) {

@@ -388,3 +388,26 @@ def test_down_projections_in_flight_together(ctx):
     tp.tp_graph_destroy(g)
     for p in ps:
         tp.tp_partition_destroy(p)
+
+
+@pytest.mark.parametrize("stride", [0, 8, 1016])
+def test_gemv_of_overlapping_rows(ctx, stride):
+    """A weight view whose rows overlap: the bits of its contiguous copy, read
+    by the same kernel (65000 elements, too few to be streamed)."""
+    rows, k = 63, 1024
+    w = _w(1, rows * k, 9).view(-1).as_strided((rows, k), (stride, 1))
+    x = _vec(k, 10)
+    out = []
+    for m in (w, w.contiguous()):
+        y = torch.full((rows,), float("nan"), device="cuda")
+        p = tp.tp_partition_create(ctx, y, (rows,))
+        tp.tp_gemv(ctx, p, m, x)
+        tp.tp_partition_destroy(p)
+        out.append(y)
+    assert torch.equal(*out)
+    big = _w(1, 90 * 1024, 9).view(-1).as_strided((90, k), (stride, 1))   # streamed when contiguous
+    y = torch.full((90,), float("nan"), device="cuda")
+    p = tp.tp_partition_create(ctx, y, (90,))
+    tp.tp_gemv(ctx, p, big, x)
+    tp.tp_partition_destroy(p)
+    assert np.all(np.abs(_f(y) - _f(big) @ _f(x)) <= _gemv_bound(big, x))

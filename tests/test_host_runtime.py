@@ -283,3 +283,19 @@ def test_counted_fp32_products_run_the_kernel_of_the_uncounted(host):
     assert len(seen) == 18
     tp.tp_partition_destroy(p)
     tp.tp_ctx_destroy(ctx)
+
+
+def test_gemv_of_overlapping_rows_takes_no_tensor_map(host):
+    host.fake_last_kernel.restype = ctypes.c_char_p
+    ctx = tp.tp_ctx_create(0)
+    rows, k = 256, 1024
+    buf = torch.zeros(rows * k + 8, dtype=torch.bfloat16)
+    buf = buf[-(buf.data_ptr() // 2) % 8:]
+    xb = torch.zeros(k + 4)
+    x, y = xb[-(xb.data_ptr() // 4) % 4:][:k], torch.zeros(rows)
+    p = tp.tp_partition_create(ctx, y, (rows,))
+    for stride, kernel in ((k, b"gemv_stream_kernel"), (8, b"gemv_kernel"), (0, b"gemv_kernel")):
+        tp.tp_gemv(ctx, p, buf.as_strided((rows, k), (stride, 1)), x, _exec())
+        assert kernel in host.fake_last_kernel()
+    tp.tp_partition_destroy(p)
+    tp.tp_ctx_destroy(ctx)
