@@ -16,16 +16,16 @@
 // in the epilogue, and down projection + residual add. Unfused kernels (one
 // per step, the plain per-call path): rmsnorm, gemv, silu_mul, residual_add.
 //
-// The fused path streams the weights through TMA (gemv_stream_kernel): a
-// producer thread copies blocks of 32 rows x 256 columns (16 KB per box; a
-// 3-D box brings 16 gate rows with their 16 up partners) into a ring of
-// shared-memory stages, and eight consumer warps take four rows each; every
-// lane multiplies 8 consecutive weights of a row by the matching 8 entries of
-// x, which sits in shared memory (whole, or one K slice at a time brought by
-// bulk copies), into four fixed-order accumulators. A TMA copy into one SM
-// costs about the same time whatever its size, so a few large copies keep a
-// stream going at the DRAM read rate, above what per-lane 16-byte loads reach
-// here.
+// The fused path and gemv stream the weights through TMA (gemv_stream_kernel):
+// a producer warp, one elected lane of it, copies blocks of 32 rows x 256
+// columns (16 KB per box; a 3-D box brings 16 gate rows with their 16 up
+// partners) into a ring of shared-memory stages, and eight consumer warps take
+// four rows each; every lane multiplies 8 consecutive weights of a row by the
+// matching 8 entries of x, which sits in shared memory (whole, or one K slice
+// at a time brought by bulk copies), into four fixed-order accumulators.
+// Issuing a copy and handing its stage over cost the roles the same time
+// whatever the copy's size, so a few large copies keep a stream going at the
+// DRAM read rate, above what per-lane 16-byte loads reach here.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -445,90 +445,88 @@ __global__ void __launch_bounds__(kSThreads, 1)
     // what a copy cost to issue bounded the stream: 5120 x 25600 41.9 us, 20896
     // x 2848 23.1, 10240 x 5120 19.2, a fused layer of d = 5120 133.1; so 38.3
     // (6.85 TB/s), 19.7, 17.5 and 128.1 us (6.96 TB/s).
-    {
-      uint32_t filled = 0, xfilled = 0;  // ring stages and x buffers filled so far
-      int stage = 0;
-      uint32_t phase = 0;
-      int64_t t = 0;  // units taken by this CTA
-      bool ok = true;
-      const uint64_t pol = policy_evict_first();  // weights are read once
-      if (!p.early_weights) grid_dependency_wait();
-      for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x, ++t) {
-        bool second;
-        int64_t rb;
-        int32_t slice;
-        decode_unit(u, &second, &rb, &slice);
-        const bool pair = (second ? p.epi1 : p.epi0) == kSiluPair;
-        const CUtensorMap* m = second ? &map1 : &map0;
-        const int32_t r0 = (int32_t)(rb * (pair ? kSPairRows : urows));
-        auto issue = [&](int64_t st) {
-          if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.err, p.wait_ns)) return false;
-          const int32_t c0 = (int32_t)(slice * p.slice_cols + st * stage_cols);  // 512-byte aligned
-          const uint32_t dst = base + (uint32_t)kSStage * stage;
-          if (elect_one()) {
-            mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kSStage);
-            if (pair) tma_load_3d(dst, m, c0, r0, 0, full_bar(stage), pol);  // g rows, then their u rows
-            else if (rgroups < 8 && p.box3) tma_load_3d(dst, m, 0, r0, c0 / kSCols, full_bar(stage), pol);
-            else
-              for (int cb = 0; cb < cblocks; ++cb)  // a block past the last column arrives as zeros
-                tma_load_2d(dst + (uint32_t)(cb * urows * kSCols * 2), m, c0 + cb * kSCols, r0, full_bar(stage), pol);
-          }
-          __syncwarp();
-          ++filled;
-          if (++stage == nst) { stage = 0; phase ^= 1u; }
-          return true;
-        };
-        int64_t st = 0;
-        if (kBulkX && t == 0) {
-          // weights first when they may go early, then the whole of x
-          if (p.early_weights) {
-            for (; st < stages_per_unit && st < nst && ok; ++st) ok = issue(st);
-            if (!ok) break;
-            grid_dependency_wait();  // x is the previous kernels' output
-          }
-          const uint32_t bytes = (uint32_t)(p.k / 4) * 16u;
-          if (bytes) {
-            if (elect_one()) {
-              mbar_arrive_expect_tx(xfull_bar(0), bytes);
-              bulk_copy_g2s(xs0, p.x, bytes, xfull_bar(0));
-            }
-            __syncwarp();
-            ++xfilled;
-          }
+    uint32_t filled = 0, xfilled = 0;  // ring stages and x buffers filled so far
+    int stage = 0;
+    uint32_t phase = 0;
+    int64_t t = 0;  // units taken by this CTA
+    bool ok = true;
+    const uint64_t pol = policy_evict_first();  // weights are read once
+    if (!p.early_weights) grid_dependency_wait();
+    for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x, ++t) {
+      bool second;
+      int64_t rb;
+      int32_t slice;
+      decode_unit(u, &second, &rb, &slice);
+      const bool pair = (second ? p.epi1 : p.epi0) == kSiluPair;
+      const CUtensorMap* m = second ? &map1 : &map0;
+      const int32_t r0 = (int32_t)(rb * (pair ? kSPairRows : urows));
+      auto issue = [&](int64_t st) {
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.err, p.wait_ns)) return false;
+        const int32_t c0 = (int32_t)(slice * p.slice_cols + st * stage_cols);  // 512-byte aligned
+        const uint32_t dst = base + (uint32_t)kSStage * stage;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kSStage);
+          if (pair) tma_load_3d(dst, m, c0, r0, 0, full_bar(stage), pol);  // g rows, then their u rows
+          else if (rgroups < 8 && p.box3) tma_load_3d(dst, m, 0, r0, c0 / kSCols, full_bar(stage), pol);
+          else
+            for (int cb = 0; cb < cblocks; ++cb)  // a block past the last column arrives as zeros
+              tma_load_2d(dst + (uint32_t)(cb * urows * kSCols * 2), m, c0 + cb * kSCols, r0, full_bar(stage), pol);
         }
-        if (p.slices > 1) {
-          if (t == 0) {
-            // consumers start on x only after this copy, so at most a ring's
-            // worth of stages goes first
-            if (p.early_weights)
-              for (; st < stages_per_unit && st < nst && ok; ++st) ok = issue(st);
-            if (!ok) break;
-            grid_dependency_wait();  // x is the previous kernels' output
-          }
-          // this unit's slice of x (whole 8-float pieces: k is a multiple of 8)
-          const int xb = (int)(t % xbufs);
-          if (!mbar_wait_warp(xempty_bar(xb), (uint32_t)(((t / xbufs) & 1) ^ 1), abort_flag, p.err, p.wait_ns)) {
-            ok = false;
-            break;
-          }
-          const int64_t c0 = (int64_t)slice * p.slice_cols;
-          const uint32_t bytes = (uint32_t)(min(p.slice_cols, p.k - c0) * 4);
+        __syncwarp();
+        ++filled;
+        if (++stage == nst) { stage = 0; phase ^= 1u; }
+        return true;
+      };
+      int64_t st = 0;
+      if (kBulkX && t == 0) {
+        // weights first when they may go early, then the whole of x
+        if (p.early_weights) {
+          for (; st < stages_per_unit && st < nst && ok; ++st) ok = issue(st);
+          if (!ok) break;
+          grid_dependency_wait();  // x is the previous kernels' output
+        }
+        const uint32_t bytes = (uint32_t)(p.k / 4) * 16u;
+        if (bytes) {
           if (elect_one()) {
-            mbar_arrive_expect_tx(xfull_bar(xb), bytes);
-            bulk_copy_g2s(xs0 + 4u * xstride * (uint32_t)xb, p.x + c0, bytes, xfull_bar(xb));
+            mbar_arrive_expect_tx(xfull_bar(0), bytes);
+            bulk_copy_g2s(xs0, p.x, bytes, xfull_bar(0));
           }
           __syncwarp();
           ++xfilled;
         }
-        for (; st < stages_per_unit && ok; ++st) ok = issue(st);
       }
-      if (!ok) {
-        // every copy this warp issued lands before the CTA retires
-        for (uint32_t s2 = 0; s2 < (uint32_t)nst && s2 < filled; ++s2)
-          mbar_wait(full_bar((int)s2), ((filled - s2 - 1u) / (uint32_t)nst) & 1u, nullptr, nullptr, 200000000ull);
-        for (uint32_t b = 0; b < (uint32_t)xbufs && b < xfilled; ++b)
-          mbar_wait(xfull_bar((int)b), ((xfilled - b - 1u) / (uint32_t)xbufs) & 1u, nullptr, nullptr, 200000000ull);
+      if (p.slices > 1) {
+        if (t == 0) {
+          // consumers start on x only after this copy, so at most a ring's
+          // worth of stages goes first
+          if (p.early_weights)
+            for (; st < stages_per_unit && st < nst && ok; ++st) ok = issue(st);
+          if (!ok) break;
+          grid_dependency_wait();  // x is the previous kernels' output
+        }
+        // this unit's slice of x (whole 16-byte pieces: k is a multiple of 4)
+        const int xb = (int)(t % xbufs);
+        if (!mbar_wait_warp(xempty_bar(xb), (uint32_t)(((t / xbufs) & 1) ^ 1), abort_flag, p.err, p.wait_ns)) {
+          ok = false;
+          break;
+        }
+        const int64_t c0 = (int64_t)slice * p.slice_cols;
+        const uint32_t bytes = (uint32_t)(min(p.slice_cols, p.k - c0) * 4);
+        if (elect_one()) {
+          mbar_arrive_expect_tx(xfull_bar(xb), bytes);
+          bulk_copy_g2s(xs0 + 4u * xstride * (uint32_t)xb, p.x + c0, bytes, xfull_bar(xb));
+        }
+        __syncwarp();
+        ++xfilled;
       }
+      for (; st < stages_per_unit && ok; ++st) ok = issue(st);
+    }
+    if (!ok) {
+      // every copy this warp issued lands before the CTA retires
+      for (uint32_t s2 = 0; s2 < (uint32_t)nst && s2 < filled; ++s2)
+        mbar_wait(full_bar((int)s2), ((filled - s2 - 1u) / (uint32_t)nst) & 1u, nullptr, nullptr, 200000000ull);
+      for (uint32_t b = 0; b < (uint32_t)xbufs && b < xfilled; ++b)
+        mbar_wait(xfull_bar((int)b), ((xfilled - b - 1u) / (uint32_t)xbufs) & 1u, nullptr, nullptr, 200000000ull);
     }
     __syncwarp();
   } else {
@@ -1203,7 +1201,8 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
   a.counts = ex->write_counts;
   a.owner = ex->write_owner;
   cudaError_t e = cudaSuccess;
-  if (d > 0 && ni > 0 && stream_ok(a_in) && ni <= kSMaxXCols) {
+  if (d == 0 || ni == 0) return o.end(e);
+  if (stream_ok(a_in) && ni <= kSMaxXCols) {
     // x whole in shared memory and units shaped to the matrix: one launch,
     // each row summed in one place (4096 x 4096: 11.1 us in two K slices and
     // a finish kernel, 8.4 so; 5120 x 5120: 15.6 and 11.3)
@@ -1227,21 +1226,20 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
   const int64_t max_cols = stream_max_slice_cols();
   int64_t slices64 = (ni + max_cols - 1) / max_cols;
   while (row_blocks * slices64 < 4 * (int64_t)ctx->sm_count && ni / (slices64 + 1) >= 2048) ++slices64;
-  int32_t slices = (int32_t)slices64;
-  int64_t slice_cols = slices == 1 ? ni : ((ni + slices - 1) / slices + kSCols - 1) / kSCols * kSCols;
-  if (slices > 1) slices = (int32_t)((ni + slice_cols - 1) / slice_cols);
-  // (x slices arrive by bulk copies, whose sizes are multiples of 16 bytes)
-  const bool streamed = stream_ok(a_in) && (slices == 1 || ni % 4 == 0) && d * slices <= WorkspacePool::kPartialFloats;
+  const int64_t slice_cols = ((ni + slices64 - 1) / slices64 + kSCols - 1) / kSCols * kSCols;
+  const int32_t slices = (int32_t)((ni + slice_cols - 1) / slice_cols);
+  // (x slices arrive by bulk copies, whose sizes are multiples of 16 bytes;
+  // one that fits whole was streamed above)
+  const bool streamed = stream_ok(a_in) && ni > kSMaxXCols && ni % 4 == 0 && d * slices <= WorkspacePool::kPartialFloats;
   float* partial = nullptr;
-  if (d > 0 && ni > 0 && streamed) {
-    s = slices > 1 ? o.partial(&partial) : TP_OK;
+  if (streamed) {
+    s = o.partial(&partial);
     if (s != TP_OK) {
       o.abort();
       return s;
     }
     o.check_err = true;  // the streaming kernel's waits are bounded
-    // 32-row units; with slices, a finish kernel adds the partial sums to h
-    // in slice order
+    // 32-row units; a finish kernel adds the partial sums to h in slice order
     StreamArgs sa{};
     sa.k = ni;
     sa.slices = slices;
@@ -1258,57 +1256,51 @@ tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor*
     sa.partial = partial;
     sa.x = a.x;
     sa.early_weights = (ex->flags & TP_EXEC_STATIC_WEIGHTS) ? 1 : 0;
-    sa.counts = sa.slices > 1 ? nullptr : a.counts;
-    sa.owner = sa.slices > 1 ? nullptr : a.owner;
     tp_status ls = launch_stream(ctx, sa, w_down, false, w_down, false, o.stream, o.err);
     if (ls != TP_OK) {
       o.abort();
       return ls;
     }
-    if (sa.slices > 1) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)((d + kThreads - 1) / kThreads));
-      cfg.blockDim = dim3(kThreads);
-      cfg.stream = o.stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      e = a.counts ? cudaLaunchKernelEx(&cfg, residual_finish_kernel<true>, a.y, (const float*)partial, d,
-                                        (int)sa.slices, a.counts, a.owner)
-                   : cudaLaunchKernelEx(&cfg, residual_finish_kernel<false>, a.y, (const float*)partial, d,
-                                        (int)sa.slices, (uint32_t*)nullptr, (int32_t*)nullptr);
-      if (e == cudaSuccess) e = cudaGetLastError();
-    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((d + kThreads - 1) / kThreads));
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = o.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = a.counts ? cudaLaunchKernelEx(&cfg, residual_finish_kernel<true>, a.y, (const float*)partial, d,
+                                      (int)sa.slices, a.counts, a.owner)
+                 : cudaLaunchKernelEx(&cfg, residual_finish_kernel<false>, a.y, (const float*)partial, d,
+                                      (int)sa.slices, (uint32_t*)nullptr, (int32_t*)nullptr);
+    if (e == cudaSuccess) e = cudaGetLastError();
     return o.end(e);
   }
   // few long rows: split K into 8 slices, one slice per CTA (so 4 CTAs fit
   // per SM); partial sums go to the operation's workspace, and a
   // finish kernel adds them to h in slice order
   const int parts = 8;
-  if (d > 0 && ni > 0) {
-    if (d * parts > WorkspacePool::kPartialFloats || ni < 8 * parts) e = launch_gemv<kResidual, 4, 4>(a, gemv_grid(ctx, ni), o.stream);
-    else {
-      const int64_t slice = ((ni / 8 + parts - 1) / parts) * 8 + 8;
-      const size_t smem = (size_t)((slice + 3) & ~int64_t(3)) * sizeof(float);
-      constexpr auto k = gemv_partial_kernel<8>;
-      s = o.partial(&partial);
-      if (s != TP_OK) {
-        o.abort();
-        return s;
-      }
-      e = smem > (size_t)kSmemOptin ? cudaErrorInvalidValue : allow_smem<k>(kSmemOptin);
-      if (e == cudaSuccess) {
-        const int grid = ctx->sm_count * 4;  // a multiple of `parts` on every GB300 SM count used (152)
-        k<<<(grid / parts) * parts, kThreads, smem, o.stream>>>(a, parts, partial);
-        const unsigned fg = (unsigned)((d + kThreads - 1) / kThreads);
-        if (a.counts)
-          residual_finish_kernel<true><<<fg, kThreads, 0, o.stream>>>(a.y, partial, d, parts, a.counts, a.owner);
-        else
-          residual_finish_kernel<false><<<fg, kThreads, 0, o.stream>>>(a.y, partial, d, parts, nullptr, nullptr);
-        e = cudaGetLastError();
-      }
+  if (d * parts > WorkspacePool::kPartialFloats || ni < 8 * parts) e = launch_gemv<kResidual, 4, 4>(a, gemv_grid(ctx, ni), o.stream);
+  else {
+    const int64_t slice = ((ni / 8 + parts - 1) / parts) * 8 + 8;
+    const size_t smem = (size_t)((slice + 3) & ~int64_t(3)) * sizeof(float);
+    constexpr auto k = gemv_partial_kernel<8>;
+    s = o.partial(&partial);
+    if (s != TP_OK) {
+      o.abort();
+      return s;
+    }
+    e = smem > (size_t)kSmemOptin ? cudaErrorInvalidValue : allow_smem<k>(kSmemOptin);
+    if (e == cudaSuccess) {
+      const int grid = ctx->sm_count * 4;  // a multiple of `parts` on every GB300 SM count used (152)
+      k<<<(grid / parts) * parts, kThreads, smem, o.stream>>>(a, parts, partial);
+      const unsigned fg = (unsigned)((d + kThreads - 1) / kThreads);
+      if (a.counts)
+        residual_finish_kernel<true><<<fg, kThreads, 0, o.stream>>>(a.y, partial, d, parts, a.counts, a.owner);
+      else
+        residual_finish_kernel<false><<<fg, kThreads, 0, o.stream>>>(a.y, partial, d, parts, nullptr, nullptr);
+      e = cudaGetLastError();
     }
   }
   return o.end(e);

@@ -14,7 +14,7 @@
 // A persistent CTA (or CTA pair) runs one program:
 //   warp 0   TMA producer: streams (A, B) K-slices into a ring of shared-
 //            memory stages (128-byte swizzle), guarded by full/empty mbarriers;
-//   warp 1   MMA issuer: one thread issues tcgen05.mma into one of two TMEM
+//   warp 1   MMA issuer: an elected lane issues tcgen05.mma into one of two TMEM
 //            accumulators and commits each consumed stage back to the producer;
 //   warps 2-5 epilogue: tcgen05.ld the finished accumulator (each warp owns the
 //            32 TMEM lanes its warp index selects: tile rows 32q..32q+31 of a
