@@ -494,7 +494,8 @@ tp_status tp_residual_add(tp_ctx* ctx, tp_partition* h, const tp_tensor* d, cons
 tp_status tp_decode_norm_qkv_gu(tp_ctx* ctx, tp_partition* qkv, tp_partition* a_out, const tp_tensor* h,
                                 const tp_tensor* gamma, const tp_tensor* w_qkv, const tp_tensor* w_gu, float eps,
                                 const tp_exec* ex);
-/* Fused: h <- h + W_down a, in one launch. */
+/* Fused: h <- h + W_down a, in one launch; in two (K slices, then their sums
+ * added to h) when a has more than 8192 entries or is not 16-byte aligned. */
 tp_status tp_decode_down_residual(tp_ctx* ctx, tp_partition* h, const tp_tensor* w_down, const tp_tensor* a_in,
                                   const tp_exec* ex);
 

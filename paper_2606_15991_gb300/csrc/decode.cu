@@ -895,7 +895,14 @@ int whole_x_stages(int64_t k) {
 //    8 rows 20.3 / 12.5 / 42.0 / 83.5    4 rows 26.8 / 15.3 / 41.9 / 124
 //   per-lane gemv_kernel 21.3 / 14.0 / 62.5 / 78.3
 // and, since the producer's warp runs converged, 17.5 / 11.1 / 38.3 / 73.8 with
-// the shapes that the rule takes.
+// the shapes that the rule takes. Those replay one matrix, of which L2 keeps a
+// part; over 400 MB of matrices in turn, with the rule's shape and the best of
+// the four: 19.0 / 18.9, 11.5 / 11.3, 41.9 / 41.5, 78.5 / 78.5, and at sizes
+// that it was not fitted to
+//   7168 x 2048 7.7 / 7.7    4096 x 14336 20.8 / 20.4  28672 x 4096 39.0 / 38.4
+//   1536 x 6144 5.9 / 5.8    2048 x 7168 7.2 / 7.2     24576 x 1536 15.0 / 15.0
+//   8192 x 8192 23.5 / 23.5  640 x 12800 5.7 / 5.7     300 x 20480 5.2 / 5.2
+// (the last 18.4 in units of 32 rows).
 void unit_rows(StreamArgs* a, int64_t rows, int64_t k, int sms) {
   a->rgroups = 8;
   a->box3 = 0;

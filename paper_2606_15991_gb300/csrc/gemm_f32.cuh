@@ -153,8 +153,9 @@ __device__ __forceinline__ void fetch_block(uint32_t dst, const float* src, int6
 // CTAs share an SM, so their barriers and tails overlap. A's rows stay as
 // stored (padded to 36 floats: the four rows a warp reads at once lie in
 // different banks).
-// Bound by the FMA pipe (over 70 % busy at 2048^3, ncu) and the issue of what
-// feeds it. Against the kernels this replaces (register-staged, 256 threads of
+// Bound by the FMA pipe (busy 69 % of the cycles at 2048^3, ncu) and the issue
+// of what feeds it. One product over and over in a replayed graph, its operands
+// in L2, against the kernels this replaces (register-staged, 256 threads of
 // 4 x 4 at one CTA per SM; TMA-fed with a producer warp for aligned operands):
 //   2048^3 aligned 419 -> 343 us, unaligned 628 -> 352
 //   1000 x 3001 x 777, nothing aligned, 184 -> 109 us

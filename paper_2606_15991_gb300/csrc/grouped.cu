@@ -81,9 +81,10 @@ constexpr uint32_t kStageX = 128 * 128;   // 128 rows x 128 bytes per CTA
 // B-operand rows per CTA, K blocks per stage and stage count: one CTA holds
 // up to 256 rows, one K block per stage (4 stages of 48 KB); a CTA of a pair
 // holds up to 128 rows, two K blocks per stage (3 stages of 64 KB), so each
-// operand arrives as one 3-D TMA box of two K blocks. A TMA copy costs about
-// the same time whatever its size, so a swap tile streams its B slab in
-// 32 KB copies at twice the rate of 16 KB ones.
+// operand arrives as one 3-D TMA box of two K blocks: fewer copies and stages
+// to hand over for the bytes. The 34 problems of M <= 64 of the 64-problem group
+// take 734 us so, 760 us with one block per stage; the whole group 4.08 ms
+// either way (launches back to back).
 #ifndef TP_GROUPED_PAIR_KC
 #define TP_GROUPED_PAIR_KC 2
 #endif
@@ -98,7 +99,9 @@ template <bool kPair> struct Ring {
 //   3 K blocks per stage | MMA columns << 32   4 B-operand rows per CTA | stream_x << 32
 constexpr int kEntry = 5;  // 64-bit words
 constexpr size_t kWordsBytes = 8 + 8 * kEntry * kRing;
-constexpr int kWideKc = 3;  // K blocks per stage of a swap problem with few B rows (pairs)
+// K blocks per stage of a swap problem with few B rows (pairs): the problems
+// above 734 us, 759 us with two.
+constexpr int kWideKc = 3;
 constexpr uint32_t kStageC = 4u * 2u * 4096u;  // epilogue staging: 4 warps x 2 buffers x (32 rows x 128 B)
 // Longest partial last 256-row band of a normal problem that CTA pairs run
 // as a swap-AB tail (0 = never)
@@ -216,11 +219,13 @@ __global__ void __launch_bounds__(kThreads, 1) grouped_kernel(const __grid_const
     // issued. (A slot's tiles are column-major over the problem's tile grid,
     // so consecutive ones share a B slab while the problem's A stays in L2.)
     // Dequeuing and decoding at the start of each tile instead left a bubble
-    // of about 1.5 us there, longer than the ring covers: 64 problems 3999 us,
-    // 3917 us dequeued ahead; 200 problems of 512^3 104 and 94 us. (Since then
-    // warp_index, which keeps both issuing roles in uniform registers: 64
-    // problems 3917 and 3784 us, the 14 with M <= 256 399 and 385 us, all of
-    // M <= 256 at 6.69 TB/s of operands.)
+    // of about 1.5 us there, longer than the ring covers: 200 problems of 512^3
+    // 104 us, 94 us dequeued ahead; the 64-problem group, one launch after a
+    // pause, 3999 and 3917 us. (Since then warp_index, which keeps both issuing
+    // roles in uniform registers: that launch 3784-3843 us over runs, 14
+    // problems of M <= 256 399 and 385 us.) Launches back to back, where the
+    // power cap sets the clock, take 4.08 ms, and neither step moved them by
+    // more than runs differ.
     int64_t nxt_slot = 0, nxt_entry = 0;
     int32_t nxt_tiles_r = 1, nxt_nk = 0, nxt_kc = 1, nxt_bn = 0, nxt_box = 0, nxt_stream = 0;
     auto dequeue = [&](int step, int64_t j) -> bool {

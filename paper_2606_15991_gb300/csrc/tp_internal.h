@@ -68,8 +68,14 @@ struct Scratch {
   std::vector<Partial> partials;
   std::vector<Counter> counters;
 };
+// What one SYNC operation at a time has of these.
+struct Lent {
+  Workspace* ws = nullptr;
+  Partial sums;
+  Counter counter;
+};
 
-// Workspaces of a context: lent to a SYNC operation for the call, to an event
+// Workspaces of a context: lent to SYNC operations, each for its call, to an event
 // and to a graph until it is gone and the work recorded into it has ended. It
 // grows by blocks as more are out at a time. The last holder (the context, its
 // events, its graphs) frees the words, so that events and graphs may be
@@ -109,6 +115,7 @@ struct tp_ctx {
   tp_graph* capturing = nullptr;    // graph being captured, if any
   std::shared_ptr<tp::WorkspacePool> pool;
   tp::Workspace* own = nullptr;     // of launches that no operation reports for
+  std::vector<tp::Lent> idle;       // of SYNC operations that have ended (under mu)
   // Device workspace, allocated once at creation.
   float* d_scratch = nullptr;       // small float scratch (kScratchFloats)
   uint32_t* d_claims = nullptr;     // tile-claim bitmap of checked launches (kClaimBits), all clear
@@ -205,11 +212,6 @@ struct DeviceGuard {
 struct Op {
   Op() = default;
   explicit Op(const char* op_name) : name(op_name) {}
-  Op(const Op&) = delete;
-  Op& operator=(const Op&) = delete;
-  ~Op() {
-    if (lent) ctx->pool->give(lent);
-  }
   const char* name = "op";   // entry point, for the TP_LOG trace
   tp_ctx* ctx = nullptr;
   const tp_exec* ex = nullptr;
@@ -217,9 +219,8 @@ struct Op {
   std::vector<tp_partition*> outs;
   bool check_err = false;   // kernel may write the error word
   int* err = nullptr;       // error word for this operation's kernels (set by begin)
-  Workspace* lent = nullptr;  // SYNC: the operation's own workspace
-  Partial sums;             // device memory of its own (partial(), queue())
-  Counter counter;
+  Lent lent;                // SYNC: the operation's workspace; and its device memory (partial(), queue())
+  bool queued = false;      // the counter's reset is enqueued or recorded
   bool marked = false;
   bool allow_checked = false;  // the op implements TP_EXEC_CHECKED (set before begin)
   bool allow_inject = false;   // the op implements TP_EXEC_INJECT_TIMEOUT (set before begin)
@@ -242,6 +243,7 @@ struct Op {
   // Likewise a tile-queue counter, zeroed on the operation's stream.
   tp_status queue(unsigned** out);
   void keep_scratch();  // hands both to the event or graph (ctx->mu held)
+  void release();       // ends the outputs' holds, returns a SYNC operation's workspace
   bool capturing() const { return ex->mode == TP_CAPTURE; }
 };
 

@@ -356,9 +356,15 @@ tp_status Op::begin_impl(tp_ctx* c, const tp_exec* e, const std::vector<tp_parti
         return fail(TP_ERR_BUSY, "an input reads bytes of a partition with work in flight on another stream");
   }
   if (ex->mode == TP_SYNC) {
-    cudaError_t we = ctx->pool->take(&lent);
-    if (we != cudaSuccess) return cuda_fail(we, "allocating operation workspaces");
-    err = lent->err;
+    if (ctx->idle.empty()) {
+      cudaError_t we = ctx->pool->take(&lent.ws);
+      if (we != cudaSuccess) return cuda_fail(we, "allocating operation workspaces");
+    } else {
+      lent = std::move(ctx->idle.back());
+      ctx->idle.pop_back();
+      *lent.ws->err = kDevOk;
+    }
+    err = lent.ws->err;
   } else {
     err = ex->mode == TP_ASYNC ? ex->event->ws->err : ctx->capturing->run->ws->err;
   }
@@ -377,7 +383,7 @@ tp_status Op::begin_impl(tp_ctx* c, const tp_exec* e, const std::vector<tp_parti
 // One of the event's or graph's, whose work runs before this operation's on the
 // same stream, unless a launch of another thread is about to use it.
 template <typename P>
-static P idle(const std::vector<P>& v) {
+static P unused(const std::vector<P>& v) {
   for (const P& p : v)
     if (p.use_count() == 1) return p;
   return nullptr;
@@ -389,41 +395,46 @@ static void keep(std::vector<P>* v, const P& p) {
 }
 
 tp_status Op::partial(float** out) {
-  if (!lent) {
+  if (ex->mode != TP_SYNC) {
     std::lock_guard<std::mutex> lk(ctx->mu);
     if (capturing()) ctx->capturing->uses_partial = true;
-    sums = idle(capturing() ? ctx->capturing->run->scratch.partials : ex->event->scratch.partials);
+    lent.sums = unused(capturing() ? ctx->capturing->run->scratch.partials : ex->event->scratch.partials);
   }
-  const cudaError_t e = sums ? cudaSuccess : ctx->pool->get(&sums);
+  const cudaError_t e = lent.sums ? cudaSuccess : ctx->pool->get(&lent.sums);
   if (e != cudaSuccess) return cuda_fail(e, "allocating partial sums");
-  *out = sums.get();
+  *out = lent.sums.get();
   return TP_OK;
 }
 
 tp_status Op::queue(unsigned** out) {
-  if (!lent) {
+  if (ex->mode != TP_SYNC) {
     std::lock_guard<std::mutex> lk(ctx->mu);
-    counter = idle(capturing() ? ctx->capturing->run->scratch.counters : ex->event->scratch.counters);
+    lent.counter = unused(capturing() ? ctx->capturing->run->scratch.counters : ex->event->scratch.counters);
   }
-  cudaError_t e = counter ? cudaSuccess : ctx->pool->get(&counter);
+  cudaError_t e = lent.counter ? cudaSuccess : ctx->pool->get(&lent.counter);
   if (e != cudaSuccess) return cuda_fail(e, "allocating tile-queue counters");
-  e = cudaMemsetAsync(counter.get(), 0, sizeof(unsigned), stream);
+  e = cudaMemsetAsync(lent.counter.get(), 0, sizeof(unsigned), stream);
   if (e != cudaSuccess) return cuda_fail(e, "resetting tile-queue counter");
-  *out = counter.get();
+  queued = true;
+  *out = lent.counter.get();
   return TP_OK;
 }
 
 void Op::keep_scratch() {
   Scratch& to = capturing() ? ctx->capturing->run->scratch : ex->event->scratch;
-  keep(&to.partials, sums);
-  keep(&to.counters, counter);
-  sums.reset();
-  counter.reset();
+  keep(&to.partials, lent.sums);
+  keep(&to.counters, lent.counter);
+  lent = {};
+}
+
+void Op::release() {
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  for (auto* p : outs) release_locked(ctx, p, stream);
+  if (lent.ws) ctx->idle.push_back(std::move(lent));
 }
 
 void Op::abort() {
-  if (counter) {
-    // its reset is enqueued, or recorded
+  if (queued) {
     if (capturing()) {
       std::lock_guard<std::mutex> lk(ctx->mu);
       keep_scratch();
@@ -431,7 +442,7 @@ void Op::abort() {
       cudaStreamSynchronize(stream);
     }
   }
-  if (marked) release(ctx, outs, stream);
+  if (marked) release();
   marked = false;
   trace(*this, "aborted", TP_ERR_INVALID);
 }
@@ -452,7 +463,7 @@ tp_status Op::end_impl(cudaError_t launch_err) {
     } else {
       cudaStreamSynchronize(stream);
     }
-    if (marked) release(ctx, outs, stream);
+    if (marked) release();
     return cuda_fail(launch_err, "kernel launch");
   }
   if (ex->mode == TP_CAPTURE) {
@@ -463,15 +474,15 @@ tp_status Op::end_impl(cudaError_t launch_err) {
   }
   if (ex->mode == TP_SYNC) {
     const cudaError_t e = cudaStreamSynchronize(stream);
-    release(ctx, outs, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    return check_err ? take_error(ctx, err) : TP_OK;
+    const tp_status s = e != cudaSuccess ? cuda_fail(e, "cudaStreamSynchronize") : check_err ? take_error(ctx, err) : TP_OK;
+    release();
+    return s;
   }
   tp_event* ev = ex->event;
   const cudaError_t e = cudaEventRecord(ev->ev, stream);
   if (e != cudaSuccess) {
     cudaStreamSynchronize(stream);
-    release(ctx, outs, stream);
+    release();
     return cuda_fail(e, "cudaEventRecord");
   }
   std::lock_guard<std::mutex> lk(ctx->mu);
