@@ -804,8 +804,8 @@ def decode_row(tp, ctx, dev, stream, peaks):
             "weight_gbs_graph": wbytes / (ms_graph * 1e-3) / 1e9, "roofline_ms": roof,
             "frac_of_roofline": roof / ms_graph, "launches_graph": launches_graph, "launches_plain": 6 * L,
             "note": "plain = 6 kernels per layer, each launched and synchronised on its own (per-call sync); "
-                    "speedup_bound_vs_plain = plain time / HBM roofline time, the largest speed-up any "
-                    "implementation streaming the weights once could reach against it"}
+                    "speedup_bound_vs_plain = plain time / HBM roofline time (the weights once at the "
+                    "measured copy rate, which a stream that mostly reads can pass)"}
 
 
 def grouped_rooflines_ms(shapes, peaks) -> tuple:
